@@ -43,7 +43,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <type_traits>
 #include <vector>
 
 #include "apply.cuh"
@@ -512,13 +511,14 @@ __global__ void ir_rhs_kernel(int64_t N, int64_t NS, double wrow, int nrhs, int6
   }
 }
 
-// x += s_c d: the FP32 correction of an inner solve into the FP64 solution
+// x += s_c d: the correction of an inner solve or a pass into the FP64 solution
 // (s = nullptr: every column with s_c = 1; s_c = -1 takes a correction back)
-__global__ void ir_add_kernel(int64_t N, int nrhs, int64_t ld, const double *s, const float *d32, double *x) {
+template <typename T>
+__global__ void add_kernel(int64_t N, int nrhs, int64_t ld, const double *s, const T *d, double *x) {
   CPM_ROWS_COLS_LOOP(N, nrhs, i, c) {
     int64_t o = i * ld + c;
     const double sc = s ? s[c] : 1.0;
-    if (sc != 0.0) x[o] += sc * (double)d32[o];
+    if (sc != 0.0) x[o] += sc * (double)d[o];
   }
 }
 
@@ -544,7 +544,7 @@ struct SolveWork {
   float *v32[6] = {};        // FP32 Krylov vectors (FP32_IR inner solves)
   float *d32 = nullptr;      // FP32_IR correction of one inner solve
   double *r64 = nullptr;     // FP64 residual
-  double *xc = nullptr;      // FP64 scratch of the rounding-floor estimate
+  double *xc = nullptr;      // FP64 scratch: correction of an FP64 pass, rounding-floor estimate of FP32_IR
   double *part = nullptr, *sc = nullptr, *out = nullptr, *cols = nullptr;
   unsigned *ticket = nullptr;
   double *h_pin = nullptr;   // host mirror: [NSC * ld] scalars, then [NQMAX * ld] dots
@@ -591,10 +591,10 @@ cpm_status cpm_reserve_solve(cpm_ctx *c, int64_t ld, bool fp32) {
   };
   for (auto &p : w->v64) al((void **)&p, n * sizeof(double));
   al((void **)&w->r64, n * sizeof(double));
+  al((void **)&w->xc, n * sizeof(double));
   if (fp32) {
     for (auto &p : w->v32) al((void **)&p, n * sizeof(float));
     al((void **)&w->d32, n * sizeof(float));
-    al((void **)&w->xc, n * sizeof(double));
   }
   w->G = 2 * c->nsm;
   // partials for up to 4 blocks per SM (the autotuner's widest choice)
@@ -746,27 +746,22 @@ cpm_status krylov_run(cpm_ctx *c, const Op<T> &op, TX *x, const Vecs<T> &V, Solv
   return CPM_OK;
 }
 
-// BiCGSTAB on the iterated system (op) with right-hand side f; x holds the
-// initial guess (x_zero: x = 0, which a wider accumulator TX requires)
-template <typename T, typename TX>
-cpm_status bicgstab(cpm_ctx *c, const Op<T> &op, const T *f, TX *x, bool x_zero, const Vecs<T> &V, SolveWork *w,
-                    int nrhs, int64_t ld, const Conv &cv, int maxit, int check_every, int *iters, int *restarts,
-                    bool *broke, cudaStream_t st) {
+// BiCGSTAB on the iterated system (op) with right-hand side f from x (in the
+// original variables); the correction accumulates in d (zero on entry).  Adding
+// a few hundred steps up apart from x and joining the two once keeps the true
+// residual near its rounding floor where the iteration's steps are large, and
+// leaves the captured iterations independent of the caller's x.
+cpm_status bicgstab(cpm_ctx *c, const Op<double> &op, const double *f, const double *x, double *d,
+                    const Vecs<double> &V, SolveWork *w, int nrhs, int64_t ld, const Conv &cv, int maxit,
+                    int check_every, int *iters, int *restarts, bool *broke, cudaStream_t st) {
   const int64_t N = c->NS + c->NC;
   const Red R = red_of(w, nrhs);
-  cpm_status rc = CPM_OK;
-  if (!x_zero) {
-    if constexpr (std::is_same<T, TX>::value) {
-      rc = op(c, x, V.r, nrhs, ld, st, true);  // r = R A x (x in the original variables)
-      if (rc) return rc;
-    } else {
-      return CPM_ERR_ARG;
-    }
-  }
-  init_kernel<T><<<(unsigned)w->G, KT, 0, st>>>(R, cv, N, ld, x_zero, f, V.r, V.rh, V.p, V.v);
+  cpm_status rc = op(c, x, V.r, nrhs, ld, st, true);  // r = R A x
+  if (rc) return rc;
+  init_kernel<double><<<(unsigned)w->G, KT, 0, st>>>(R, cv, N, ld, false, f, V.r, V.rh, V.p, V.v);
   cpm_count_launches(c, 1);
   *broke = false;
-  return krylov_run<T, TX>(c, op, x, V, w, nrhs, ld, cv, maxit, check_every, iters, restarts, broke, st);
+  return krylov_run<double, double>(c, op, d, V, w, nrhs, ld, cv, maxit, check_every, iters, restarts, broke, st);
 }
 
 // FP64 residual r64 = f - A x and its squared weighted norms per column:
@@ -909,7 +904,7 @@ cpm_status ir_refine(cpm_ctx *c, ApplyFn<double> ap64, const Op<float> &op32, do
     rc = krylov_run<float, float>(c, op32, w->d32, V, w, nrhs, ld, cv, maxit - it_total, check_every, &it, &rs,
                                   &broke, st);
     if (rc) return rc;
-    ir_add_kernel<<<g, 256, 0, st>>>(N, nrhs, ld, nullptr, w->d32, x);
+    add_kernel<float><<<g, 256, 0, st>>>(N, nrhs, ld, nullptr, w->d32, x);
     cpm_count_launches(c, 1);
     it_total += it;
     nrs += rs;
@@ -931,7 +926,7 @@ cpm_status ir_refine(cpm_ctx *c, ApplyFn<double> ap64, const Op<float> &op32, do
     if (back) {
       if (trace) std::fprintf(stderr, "[cpm ir] steps taken back after refinement %d\n", nrep);
       CPM_CUDA_TRY(cudaMemcpyAsync(w->cols, flag.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, st));
-      ir_add_kernel<<<g, 256, 0, st>>>(N, nrhs, ld, w->cols, w->d32, x);
+      add_kernel<float><<<g, 256, 0, st>>>(N, nrhs, ld, w->cols, w->d32, x);
       cpm_count_launches(c, 1);
       rc = residual64(c, ap64, m, n, f, x, w, nrhs, ld, wrow, rn2, fn2, st, rhs_w, &rv2);
       if (rc) return rc;
@@ -965,9 +960,12 @@ cpm_status fp64_passes(cpm_ctx *c, ApplyFn<double> ap64, bool left, double dS, d
       rhs = V.t;
     }
     int it = 0, rs = 0;
-    cpm_status rc = bicgstab<double, double>(c, op, rhs, x, false, V, w, nrhs, ld, cv, maxit - *iters, check_every,
-                                             &it, &rs, broke, st);
+    CPM_CUDA_TRY(cudaMemsetAsync(w->xc, 0, sizeof(double) * (size_t)N * (size_t)ld, st));
+    cpm_status rc = bicgstab(c, op, rhs, x, w->xc, V, w, nrhs, ld, cv, maxit - *iters, check_every, &it, &rs, broke,
+                             st);
     if (rc) return rc;
+    add_kernel<double><<<cpm_grid(N * nrhs, 256), 256, 0, st>>>(N, nrhs, ld, nullptr, w->xc, x);
+    cpm_count_launches(c, 1);
     *iters += it;
     *restarts += rs;
     rc = residual64(c, ap64, m, n, f, x, w, nrhs, ld, wrow, rn2, fn2, st);
