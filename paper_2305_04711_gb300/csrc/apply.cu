@@ -455,6 +455,39 @@ template void cpm_launch_combine<double>(const ApplyArgs<double> &, double, doub
 template void cpm_launch_combine<float>(const ApplyArgs<float> &, float, float, float, float, const float *,
                                         const float *, float *, int, int64_t, cudaStream_t, bool);
 
+// the kernels of one product v = R A C u with the intermediate a ([N_S][ld]);
+// returns the number of launches
+template <typename T>
+static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T *a, T *v, int nrhs, int64_t ld,
+                          cudaStream_t st) {
+  ApplyArgs<T> A = cpm_apply_args<T>(c);
+  const bool diff = true;
+  // batched layouts whose columns fill whole warps use the warp-per-row kernels;
+  // two adjacent columns per lane need an even column count and 2-element alignment
+  const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
+                                           reinterpret_cast<uintptr_t>(a)) % (2 * sizeof(T)) == 0);
+  if (nrhs > 32 && nrhs <= 64 && nrhs % 2 == 0 && aligned2)
+    return launch_batched<T, 2>(c, A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
+  if (nrhs >= 16 && nrhs <= 32)
+    return launch_batched<T, 1>(c, A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
+  int launched = 0;
+  if (nrhs == 1 && c->ncells > 0 && c->tune.single_mode == 2) {
+    launched = cpm_launch_fused1<T>(c, A, m, n, rowscale, cs, u, a, v, st);
+    if (launched) return launched;
+  }
+  if (nrhs == 1 && c->ncells > 0 && c->tune.single_mode == 1) {
+    cpm_launch_gather1<T>(c, A, cs, u, a, st);
+    launched = 1 + cpm_launch_correct_few<T>(c, cs, u, a, 1, ld, st);
+  } else if (nrhs < 16) {
+    launched = cpm_launch_gather_tile<T>(c, cs, u, a, nrhs, ld, st, diff);
+  } else {
+    cpm_launch_gather<T>(A, cs, u, a, nrhs, ld, st, diff);
+    launched = 1;
+  }
+  cpm_launch_combine<T>(A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
+  return launched + 1;
+}
+
 // v = R A C u using the context's reserved scratch for a (no allocation): R
 // scales the PDE rows of the result by `rowscale` and C the PDE entries of the
 // input by `colscale` (1 and 1 for the plain product); BC rows and BC entries
@@ -464,34 +497,9 @@ template <typename T>
 cpm_status cpm_apply_rc_T(cpm_ctx *c, double m, double n, double rowscale, double colscale, const T *u, T *v,
                           int nrhs, int64_t ld, cudaStream_t st) {
   if (sizeof(T) * (size_t)c->NS * (size_t)ld > c->a_scratch.bytes) return CPM_ERR_CAPACITY;
-  ApplyArgs<T> A = cpm_apply_args<T>(c);
   T *a = reinterpret_cast<T *>(c->a_scratch.p);
-  const bool diff = true;
-  const T cs = T(colscale);
   cpm_prof_begin(c, st);
-  // batched layouts whose columns fill whole warps use the warp-per-row kernels
-  const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
-                                           reinterpret_cast<uintptr_t>(a)) % (2 * sizeof(T)) == 0);
-  int launched = 2;
-  // two adjacent columns per lane need an even column count and 2-element alignment
-  if (nrhs > 32 && nrhs <= 64 && nrhs % 2 == 0 && aligned2)
-    launched = launch_batched<T, 2>(c, A, (T)m, (T)n, (T)rowscale, cs, u, a, v, nrhs, ld, st, diff);
-  else if (nrhs >= 16 && nrhs <= 32)
-    launched = launch_batched<T, 1>(c, A, (T)m, (T)n, (T)rowscale, cs, u, a, v, nrhs, ld, st, diff);
-  else if (nrhs == 1 && c->ncells > 0) {
-    // default: the per-cell gather, then the combine; 1: per-row gather; 2: the
-    // fused persistent product (fused1.cu)
-    launched = (c->tune.single_mode == 2)
-                   ? cpm_launch_fused1<T>(c, A, (T)m, (T)n, (T)rowscale, cs, u, a, v, st)
-                   : 0;
-    if (launched == 0) {
-      launched = 1 + cpm_launch_gather1<T>(c, A, cs, u, a, st, diff);
-      cpm_launch_combine<T>(A, (T)m, (T)n, (T)rowscale, cs, u, a, v, nrhs, ld, st, diff);
-    }
-  } else {
-    cpm_launch_gather<T>(A, cs, u, a, nrhs, ld, st, diff);
-    cpm_launch_combine<T>(A, (T)m, (T)n, (T)rowscale, cs, u, a, v, nrhs, ld, st, diff);
-  }
+  const int launched = launch_product<T>(c, (T)m, (T)n, (T)rowscale, (T)colscale, u, a, v, nrhs, ld, st);
   cpm_prof_end(c, st, c->NS * (int64_t)nrhs);
   cpm_count_launches(c, launched);
   CPM_CUDA_TRY(cudaGetLastError());
@@ -534,8 +542,8 @@ void cpm_prof_end(cpm_ctx *c, cudaStream_t st, int64_t row_rhs) {
 }
 
 cpm_status cpm_internal_extend(cpm_ctx *c, const double *u, double *a, int nrhs, int64_t ld, cudaStream_t st) {
-  ApplyArgs<double> A = cpm_apply_args<double>(c);
-  cpm_launch_gather<double>(A, 1.0, u, a, nrhs, ld, st, false);
+  if (nrhs < 16) cpm_launch_gather_tile<double>(c, 1.0, u, a, nrhs, ld, st, false);
+  else cpm_launch_gather<double>(cpm_apply_args<double>(c), 1.0, u, a, nrhs, ld, st, false);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }
@@ -603,20 +611,8 @@ cpm_status cpm_apply_noalloc_T(cpm_ctx *c, double m, double n, const T *u, T *v,
   void *p = nullptr;
   cpm_status rc = noalloc_scratch(&p);
   if (rc) return rc;
-  T *a = reinterpret_cast<T *>(p);
-  ApplyArgs<T> A = cpm_apply_args<T>(c);
-  const bool diff = true;  // the same arithmetic as cpm_apply
-  const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
-                                           reinterpret_cast<uintptr_t>(a)) % (2 * sizeof(T)) == 0);
-  int launched = 2;
-  if (nrhs > 32 && nrhs <= 64 && nrhs % 2 == 0 && aligned2)
-    launched = launch_batched<T, 2>(c, A, (T)m, (T)n, T(1), T(1), u, a, v, nrhs, ld, st, diff);
-  else if (nrhs >= 16 && nrhs <= 32)
-    launched = launch_batched<T, 1>(c, A, (T)m, (T)n, T(1), T(1), u, a, v, nrhs, ld, st, diff);
-  else {
-    cpm_launch_gather<T>(A, T(1), u, a, nrhs, ld, st, diff);
-    cpm_launch_combine<T>(A, (T)m, (T)n, T(1), T(1), u, a, v, nrhs, ld, st, diff);
-  }
+  // the same kernels as cpm_apply
+  const int launched = launch_product<T>(c, (T)m, (T)n, T(1), T(1), u, reinterpret_cast<T *>(p), v, nrhs, ld, st);
   cpm_count_launches(c, launched);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;

@@ -57,10 +57,16 @@ int cpm_launch_gather_cells(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const
 
 cpm_status cpm_internal_surface_gradient(cpm_ctx *c, const double *u, double *X, int normalize, cudaStream_t st);
 cpm_status cpm_internal_surface_divergence(cpm_ctx *c, const double *X, double *b, cudaStream_t st);
-// single right-hand side: E u for all PDE rows in cell order plus the
-// flipped-entry correction; returns the number of kernels launched
+// one or a few right-hand sides (tile.cu): cs (E u - u) (diff) or cs E u on all
+// PDE rows plus the flipped-entry correction; returns the number of kernels launched
 template <typename T>
-int cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st, bool diff);
+int cpm_launch_gather_tile(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st, bool diff);
+// the flipped-entry correction alone (0 or 1 launches)
+template <typename T>
+int cpm_launch_correct_few(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st);
+// single right-hand side: one thread per row in cell order, without the correction
+template <typename T>
+void cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st);
 
 // the cell gather's default x passes for a stencil of np1 nodes per axis, the
 // precision and the columns per lane (1 or 2); the autotuner starts from it

@@ -380,6 +380,19 @@ __global__ void cell_lines_kernel(BandView v, const uint32_t *cell_key, int64_t 
   }
 }
 
+// the rows' fractional stencil positions in cell order, so that a warp's rows
+// read them as one contiguous run
+__global__ void cell_frac_kernel(const int32_t *rows, int64_t NS, const double *t64, double *tc64, float *tc32) {
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < NS; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = rows[q];
+    for (int e = 0; e < 3; ++e) {
+      const double t = t64[3 * i + e];
+      tc64[3 * q + e] = t;
+      tc32[3 * q + e] = (float)t;
+    }
+  }
+}
+
 __global__ void row_cell_kernel(const int32_t *cell_start, int64_t ncells, int32_t *row_cell) {
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncells; c += (int64_t)gridDim.x * blockDim.x)
     for (int32_t q = cell_start[c]; q < cell_start[c + 1]; ++q) row_cell[q] = (int32_t)c;
@@ -429,93 +442,6 @@ __global__ void __launch_bounds__(256) gather1_kernel(ApplyArgs<T> A, const int3
   }
 }
 
-// single right-hand side, one thread per cell: the thread loads the cell's
-// NP^dim node values once (as differences to the base node's value) and applies
-// the separable weights of each of the cell's rows to them, so the node loads
-// and index arithmetic are shared by the ~5 rows of a cell instead of repeated
-// per row.  FP32 x pairs go through packed FMAs.
-template <typename T, int DIM, int NP>
-__global__ void __launch_bounds__(128) gather1c_kernel(ApplyArgs<T> A, const int32_t *__restrict__ cstart,
-                                                       const uint32_t *__restrict__ ckey,
-                                                       const int32_t *__restrict__ crows,
-                                                       const int2 *__restrict__ lines, int64_t ncells, T cs,
-                                                       const T *__restrict__ u, T *__restrict__ a) {
-  constexpr int NZ = (DIM == 3) ? NP : 1;
-  constexpr bool PAIR = (sizeof(T) == 4);
-  for (int64_t cid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; cid < ncells;
-       cid += (int64_t)gridDim.x * blockDim.x) {
-    const int lx = (int)(__ldg(ckey + cid) & 7u);
-    const int split = (lx + NP - 1 < 8) ? NP : 8 - lx;
-    const int2 *ln = lines + cid * 16;
-    const T uc = __ldg(u + __ldg(&ln[0].x));
-    T d[NZ][NP][NP];  // [cz][cy][cx]
-#pragma unroll
-    for (int cz = 0; cz < NZ; ++cz)
-#pragma unroll
-      for (int cy = 0; cy < NP; ++cy) {
-        const int2 se = __ldg(ln + cz * 4 + cy);
-#pragma unroll
-        for (int cx = 0; cx < NP; ++cx) {
-          const int32_t idx = (cx < split) ? (se.x + cx) : (se.y + (cx - split));
-          d[cz][cy][cx] = __ldg(u + idx) - uc;
-        }
-      }
-    const int32_t q1 = __ldg(cstart + cid + 1);
-    for (int32_t q = __ldg(cstart + cid); q < q1; ++q) {
-      const int64_t row = __ldg(crows + q);
-      T wx[4], wy[4], wz[4];
-      cpm_lagrange<NP, T>(__ldg(A.t + 3 * row), wx);
-      cpm_lagrange<NP, T>(__ldg(A.t + 3 * row + 1), wy);
-      if (DIM == 3) cpm_lagrange<NP, T>(__ldg(A.t + 3 * row + 2), wz);
-      else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
-      T P[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-      for (int cz = 0; cz < NZ; ++cz)
-#pragma unroll
-        for (int cy = 0; cy < NP; ++cy) {
-          const T w = wy[cy] * wz[cz];
-          if constexpr (PAIR) {
-            const float2 p01 = __ffma2_rn(make_float2(w, w), make_float2(d[cz][cy][0], d[cz][cy][1]),
-                                          make_float2(P[0], P[1]));
-            P[0] = p01.x; P[1] = p01.y;
-            if constexpr (NP == 4) {
-              const float2 p23 = __ffma2_rn(make_float2(w, w), make_float2(d[cz][cy][2], d[cz][cy][3]),
-                                            make_float2(P[2], P[3]));
-              P[2] = p23.x; P[3] = p23.y;
-            } else {
-              P[2] += w * d[cz][cy][2];
-            }
-          } else {
-#pragma unroll
-            for (int cx = 0; cx < NP; ++cx) P[cx] += w * d[cz][cy][cx];
-          }
-        }
-      T acc = T(0);
-#pragma unroll
-      for (int cx = 0; cx < NP; ++cx) acc += wx[cx] * P[cx];
-      acc += uc - __ldg(u + row);
-      a[row] = cs * acc;
-    }
-  }
-}
-
-// single right-hand side correction: one thread per row with flipped entries
-template <typename T>
-__global__ void __launch_bounds__(256) correct1_kernel(const int32_t *__restrict__ crow,
-                                                       const int32_t *__restrict__ cstart,
-                                                       const int32_t *__restrict__ cnode,
-                                                       const int32_t *__restrict__ ccol, const T *__restrict__ cw,
-                                                       int64_t ncorr, T cs, const T *__restrict__ u,
-                                                       T *__restrict__ a) {
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ncorr; q += (int64_t)gridDim.x * blockDim.x) {
-    T acc = T(0);
-    const int32_t e1 = __ldg(cstart + q + 1);
-    for (int32_t e = __ldg(cstart + q); e < e1; ++e)
-      acc += __ldg(cw + e) * (__ldg(u + __ldg(ccol + e)) - cs * __ldg(u + __ldg(cnode + e)));
-    a[__ldg(crow + q)] += acc;
-  }
-}
-
 }  // namespace
 
 void cpm_free_cells(cpm_ctx *c) {
@@ -523,6 +449,8 @@ void cpm_free_cells(cpm_ctx *c) {
   cudaFree(c->d_cell_start); cudaFree(c->d_cell_rows); cudaFree(c->d_cell_key); cudaFree(c->d_nbr8);
   cudaFree(c->d_corr_row); cudaFree(c->d_corr_start); cudaFree(c->d_corr_node); cudaFree(c->d_corr_col);
   cudaFree(c->d_corr_w64); cudaFree(c->d_corr_w32); cudaFree(c->d_cell_lines); cudaFree(c->d_row_cell);
+  cudaFree(c->d_tc64); cudaFree(c->d_tc32);
+  c->d_tc64 = nullptr; c->d_tc32 = nullptr;
   c->d_cell_lines = nullptr; c->d_row_cell = nullptr;
   c->d_cell_start = nullptr; c->d_cell_rows = nullptr; c->d_cell_key = nullptr; c->d_nbr8 = nullptr;
   c->d_corr_row = nullptr; c->d_corr_start = nullptr; c->d_corr_node = nullptr; c->d_corr_col = nullptr;
@@ -570,6 +498,9 @@ cpm_status cpm_build_cells(cpm_ctx *c) {
   set_i32_kernel<<<1, 1, 0, st>>>(c->d_cell_start + c->ncells, h_tot);
   TRY(cudaMalloc(&c->d_cell_lines, sizeof(int2) * 16 * std::max<int64_t>(c->ncells, 1)));
   TRY(cudaMalloc(&c->d_row_cell, sizeof(int32_t) * std::max<int64_t>(c->NS, 1)));
+  TRY(cudaMalloc(&c->d_tc64, sizeof(double) * 3 * std::max<int64_t>(c->NS, 1)));
+  TRY(cudaMalloc(&c->d_tc32, sizeof(float) * 3 * std::max<int64_t>(c->NS, 1)));
+  cell_frac_kernel<<<cpm_grid(c->NS, 256), 256, 0, st>>>(c->d_cell_rows, c->NS, c->d_t64, c->d_tc64, c->d_tc32);
   if (c->ncells > 0) {
     cell_lines_kernel<<<cpm_grid(c->ncells * 16, 256), 256, 0, st>>>(c->view(), c->d_cell_key, c->ncells,
                                                                     reinterpret_cast<int2 *>(c->d_cell_lines));
@@ -701,50 +632,20 @@ template int cpm_launch_gather_cells<double>(const cpm_ctx *, const ApplyArgs<do
                                              double *, int, int64_t, cudaStream_t, bool, int);
 
 template <typename T>
-int cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st, bool diff) {
-  if (c->ncells == 0) return 0;
+void cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st) {
   const unsigned g = cpm_grid(c->NS, 256);
   const int2 *lines = reinterpret_cast<const int2 *>(c->d_cell_lines);
-  if (diff && c->tune.single_mode != 1) {
-    // one thread per cell (the difference form only)
-    const unsigned gc = cpm_grid(c->ncells, 128);
-#define CPM_G1C(D, NP)                                                                                           \
-  gather1c_kernel<T, D, NP><<<gc, 128, 0, st>>>(A, c->d_cell_start, c->d_cell_key, c->d_cell_rows, lines, c->ncells, \
-                                                cs, u, a)
-    if (c->dim == 3) {
-      if (c->p == 2) CPM_G1C(3, 3); else CPM_G1C(3, 4);
-    } else {
-      if (c->p == 2) CPM_G1C(2, 3); else CPM_G1C(2, 4);
-    }
-#undef CPM_G1C
-  } else {
-#define CPM_G1(D, NP)                                                                                       \
-  do {                                                                                                      \
-    if (diff)                                                                                               \
-      gather1_kernel<T, true, D, NP><<<g, 256, 0, st>>>(A, c->d_cell_rows, c->d_row_cell, c->d_cell_key, lines, \
-                                                        c->NS, cs, u, a);                                   \
-    else                                                                                                    \
-      gather1_kernel<T, false, D, NP><<<g, 256, 0, st>>>(A, c->d_cell_rows, c->d_row_cell, c->d_cell_key,     \
-                                                         lines, c->NS, cs, u, a);                           \
-  } while (0)
+#define CPM_G1(D, NP)                                                                                         \
+  gather1_kernel<T, true, D, NP><<<g, 256, 0, st>>>(A, c->d_cell_rows, c->d_row_cell, c->d_cell_key, lines, \
+                                                    c->NS, cs, u, a)
   if (c->dim == 3) {
     if (c->p == 2) CPM_G1(3, 3); else CPM_G1(3, 4);
   } else {
     if (c->p == 2) CPM_G1(2, 3); else CPM_G1(2, 4);
   }
 #undef CPM_G1
-  }
-  if (c->ncorr > 0) {
-    const T *cw;
-    if constexpr (sizeof(T) == 8) cw = reinterpret_cast<const T *>(c->d_corr_w64);
-    else cw = reinterpret_cast<const T *>(c->d_corr_w32);
-    correct1_kernel<T><<<cpm_grid(c->ncorr, 256), 256, 0, st>>>(c->d_corr_row, c->d_corr_start, c->d_corr_node,
-                                                                c->d_corr_col, cw, c->ncorr, cs, u, a);
-    return 2;
-  }
-  return 1;
 }
-template int cpm_launch_gather1<float>(const cpm_ctx *, const ApplyArgs<float> &, float, const float *, float *,
-                                       cudaStream_t, bool);
-template int cpm_launch_gather1<double>(const cpm_ctx *, const ApplyArgs<double> &, double, const double *, double *,
-                                        cudaStream_t, bool);
+template void cpm_launch_gather1<float>(const cpm_ctx *, const ApplyArgs<float> &, float, const float *, float *,
+                                        cudaStream_t);
+template void cpm_launch_gather1<double>(const cpm_ctx *, const ApplyArgs<double> &, double, const double *, double *,
+                                         cudaStream_t);

@@ -1,0 +1,402 @@
+// tile.cu -- E u for one or a few right-hand sides: warp tiles of stencil cells.
+//
+// A warp takes CT consecutive cells (cells.cu) and stages the differences of
+// their node values to each cell's base-node value in shared memory, then its
+// lanes take the tile's rows (~5 per cell, in cell order), one row each: the
+// weights of the row, the separable sum over the cell's nodes from shared
+// memory, and a_i = sum_j w_j (u_j - u_c) + (u_c - u_i).  Rows, not cells, are
+// spread over the lanes because cells hold between 1 and a dozen rows: one
+// thread per cell left a warp waiting for its fullest cell, and 64 FP64 node
+// values per thread left 2 blocks of 128 threads per SM.  The staging loads
+// take 8 stencil lines of 4 consecutive DOFs per instruction.
+//
+// FP64 without the FP64 pipe.  This chip runs 2 FP64 lanes per clock and SM
+// (1/64 of FP32; 1.25 TFLOP/s measured), but 32 lanes of 32 x 32 + 64 bit
+// integer multiply-adds.  The weighted sum therefore runs in integers that are
+// wider than a double's 53 bits:
+//  * the differences of a cell, exact or rounded once as doubles, become
+//    integers X of 61 bits relative to the largest of the cell;
+//  * the Lagrange weights are formed as integers W = 6 w 2^60 (times 6, so that
+//    no division rounds) from the fractional position t, of which every bit is
+//    kept;
+//  * operands split at bit 32 into signed halves, X = Xh 2^32 + Xl, and a sum of
+//    products is sum Wh Xh + (sum Wh Xl + Wl Xh) / 2^32 in units of 2^64: three
+//    multiply-adds a term into two 64-bit sums that cannot overflow (|Xh| <= 2^29
+//    and |Wh| < 2^31, four terms with sum |w| <= 1.25).  Wl Xl, at most a quarter
+//    of a unit, is left out.  Split at the word size, the halves and the result
+//    are registers, not shifts;
+//  * the sum is the next axis's operand as it stands: an axis scales by
+//    6 2^60 / 2^64 and its sum of |weights|, so operands shrink from 2^61 to
+//    2^57.7 and the last unit stays below 2^-56 of the largest difference.
+// The sum is converted back once, exactly scaled, with one FP64 rounding: its
+// error is a few 2^-56 of the largest difference in the cell, where 84 rounded
+// FP64 operations leave a few 2^-53 of the partial sums.  A cell whose
+// differences are not finite or whose largest one is below 2^-940 goes through
+// plain FP64.
+#include <algorithm>
+
+#include "apply.cuh"
+#include "cpm_internal.cuh"
+
+namespace {
+
+constexpr int TW = 4;  // warps per block; warps are independent
+
+// ---- fixed-point pieces ------------------------------------------------------
+
+// signed halves of x = xh 2^32 + xl
+__device__ __forceinline__ void halves(long long x, int32_t &xh, int32_t &xl) {
+  xl = (int32_t)x;
+  xh = (int32_t)((unsigned long long)x >> 32) + (int32_t)((uint32_t)xl >> 31);
+}
+
+__device__ __forceinline__ long long high_word(long long cr) { return (long long)(int32_t)(cr >> 32); }
+
+// a b + c, one instruction
+__device__ __forceinline__ long long mad_wide(int32_t a, int32_t b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+
+__device__ __forceinline__ void mac(long long &hh, long long &cr, int32_t wh, int32_t wl, int32_t xh, int32_t xl) {
+  hh = mad_wide(wh, xh, hh);
+  cr = mad_wide(wh, xl, cr);
+  cr = mad_wide(wl, xh, cr);
+}
+
+// a b / 2^64 to within 1.25 units
+__device__ __forceinline__ long long mul_high(long long a, long long b) {
+  int32_t ah, al, bh, bl;
+  halves(a, ah, al);
+  halves(b, bh, bl);
+  return mad_wide(ah, bh, high_word(mad_wide(al, bh, mad_wide(ah, bl, 0))));
+}
+
+// 6 2^60 times the Lagrange weights of one axis, in halves.  With tau = t - 1 (exact):
+//   cubic      q = tau (tau - 1), P = q tau:
+//              6 w = { 2q - P, 3 (P - q - 2 tau + 2), 3 (2 tau - P), P + q }
+//   quadratic  6 w = { 3 (tau^2 - tau), 6 (1 - tau^2), 3 (tau^2 + tau) }
+template <int NP>
+__device__ __forceinline__ void fixed_weights(double t, int32_t (&wh)[4], int32_t (&wl)[4]) {
+  const long long b = __double_as_longlong(t);
+  const int sh = (int)(b >> 52) - 1023;  // t is in [1/2, 2] up to rounding: sh in -2 .. 1
+  long long t60 = (long long)(((b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll) << 8);
+  t60 = (sh >= 0) ? (t60 << sh) : (t60 >> min(-sh, 62));
+  const long long one = 1ll << 60, tau = t60 - one;
+  long long w[4];
+  if constexpr (NP == 4) {
+    const long long q = mul_high(tau << 2, (tau - one) << 2);  // 2^62 x 2^62 -> 2^60
+    const long long P = mul_high(q << 2, tau << 2);
+    const long long c = P - 2 * tau;
+    w[0] = 2 * q - P;
+    w[1] = 3 * (c - q + 2 * one);
+    w[2] = -3 * c;
+    w[3] = P + q;
+  } else {
+    const long long s = mul_high(tau << 2, tau << 2);
+    w[0] = 3 * (s - tau);
+    w[1] = 6 * (one - s);
+    w[2] = 3 * (s + tau);
+    w[3] = 0;
+  }
+#pragma unroll
+  for (int k = 0; k < NP; ++k) halves(w[k], wh[k], wl[k]);
+}
+
+// E u - u_c of one row in plain FP64 (the rare cells outside the integer range)
+template <int DIM, int NP>
+__device__ __noinline__ double slow_row(const double *t, const int2 *ln, int split, const double *u, int64_t ld,
+                                        double uc) {
+  double wx[4], wy[4], wz[4];
+  cpm_lagrange<NP, double>(t[0], wx);
+  cpm_lagrange<NP, double>(t[1], wy);
+  if (DIM == 3) cpm_lagrange<NP, double>(t[2], wz);
+  else { wz[0] = 1.0; wz[1] = wz[2] = wz[3] = 0.0; }
+  double acc = 0.0;
+  for (int cz = 0; cz < ((DIM == 3) ? NP : 1); ++cz)
+    for (int cy = 0; cy < NP; ++cy) {
+      const int2 se = ln[cz * 4 + cy];
+      for (int cx = 0; cx < NP; ++cx) {
+        const int32_t idx = (cx < split) ? (se.x + cx) : (se.y + (cx - split));
+        acc += (wx[cx] * (wy[cy] * wz[cz])) * (u[(int64_t)idx * ld] - uc);
+      }
+    }
+  return acc;
+}
+
+template <typename T> struct Node;
+template <> struct Node<float> { typedef float t; };
+template <> struct Node<double> { typedef int2 t; };
+
+struct TileArgs {
+  const int32_t *cstart, *crows, *row_cell;
+  const uint32_t *ckey;
+  const int2 *lines;
+  int64_t ncells;
+};
+
+// DIFF: a_i = cs (E u - u)_i; otherwise a_i = cs (E u)_i.
+//
+// FP64, sphere h = 1/128 (1.70M rows, 309k cells): 140 us (one thread per cell in
+// FP64 arithmetic: 820 us), with the multiply-add pipe busy 55 % and the integer
+// pipe 46 %; what is left is the latency of the staging loads at 24 warps per SM,
+// which is why they are unrolled over 8 cells.  FP32, bumpy sphere h = 1/320
+// (10.7M rows): 250 us (272 us), held by L1 wavefronts (74 %).
+template <typename T, bool DIFF, int DIM, int NP, int CT>
+__global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
+    gather_tile_kernel(TileArgs A, const T *__restrict__ tc, T cs, const T *__restrict__ u, T *__restrict__ a,
+                       int nrhs, int64_t ld) {
+  constexpr int NZ = (DIM == 3) ? NP : 1;
+  constexpr int SLOTS = 16 * NZ;                           // 4 x 4 x NZ, x fastest
+  constexpr bool FX = (sizeof(T) == 8);
+  typedef typename Node<T>::t V;
+  constexpr int STR = SLOTS + 16 / (int)sizeof(V);         // one 16-byte pad: cells start 4 banks apart
+  constexpr int PER = (SLOTS + 31) / 32;                   // node slots of a lane per cell (3D)
+  constexpr int CPI = (SLOTS < 32) ? 32 / SLOTS : 1;       // cells per staging step (2D: two)
+  __shared__ __align__(16) V s_d[TW][CT][STR];
+  __shared__ T s_uc[TW][CT];
+  __shared__ T s_sc[FX ? TW : 1][FX ? CT : 1];             // FP64: scale of a cell's integers; < 0: plain FP64
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t c0 = ((int64_t)blockIdx.x * TW + w) * CT;
+  if (c0 >= A.ncells) return;
+  const int nc = (int)min((int64_t)CT, A.ncells - c0);
+  const int32_t q0 = __ldg(A.cstart + c0), q1 = __ldg(A.cstart + c0 + nc);
+  for (int r = 0; r < nrhs; ++r) {
+    const T *ur = u + r;
+    // ---- stage the tile's node values as differences to each cell's base node
+#pragma unroll(FX ? 8 : 4)
+    for (int cb = 0; cb < nc; cb += CPI) {
+      const int sub = (CPI > 1) ? lane / SLOTS : 0;
+      const int c = cb + sub;
+      const bool live = c < nc;
+      const int64_t cid = c0 + (live ? c : 0);
+      const int lx = (int)(__ldg(A.ckey + cid) & 7u);
+      const int split = (lx + NP - 1 < 8) ? NP : 8 - lx;
+      T v[PER];
+      bool on[PER];
+#pragma unroll
+      for (int k = 0; k < PER; ++k) {
+        const int slot = (CPI > 1) ? (lane & (SLOTS - 1)) : lane + 32 * k;
+        const int x = slot & 3, ln = slot >> 2;
+        on[k] = live && slot < SLOTS && x < NP && (ln & 3) < NP;
+        v[k] = T(0);
+        if (on[k]) {
+          const int2 se = __ldg(A.lines + cid * 16 + ln);
+          const int32_t idx = (x < split) ? (se.x + x) : (se.y + (x - split));
+          v[k] = __ldg(ur + (int64_t)idx * ld);
+        }
+      }
+      const T uc = __shfl_sync(0xffffffffu, v[0], (CPI > 1) ? sub * SLOTS : 0);
+      T d[PER];
+#pragma unroll
+      for (int k = 0; k < PER; ++k) d[k] = on[k] ? v[k] - uc : T(0);
+      if constexpr (FX) {
+        // exponent of the cell's largest difference
+        unsigned top = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k)  // (a denormal may have all its bits in the low word)
+          top = max(top, ((unsigned)__double2hiint(d[k]) & 0x7FFFFFFFu) | (unsigned)(__double2loint(d[k]) != 0));
+        if (CPI > 1) {
+#pragma unroll
+          for (int o = SLOTS / 2; o; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        } else {
+          top = __reduce_max_sync(0xffffffffu, top);
+        }
+        const int em = (int)(top >> 20);
+        // |d| < 2^(em - 1022); X = d 2^(1083 - em), |X| < 2^61
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+          const int slot = (CPI > 1) ? (lane & (SLOTS - 1)) : lane + 32 * k;
+          const int hi = __double2hiint(d[k]);
+          const int e = (hi >> 20) & 0x7FF;
+          unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xFFFFFu) | 0x100000u) << 32) |
+                                 (unsigned)__double2loint(d[k]);
+          m = (e == 0) ? 0ull : ((m << 8) >> min(em - e, 63));
+          const long long X = (hi < 0) ? -(long long)m : (long long)m;
+          if (SLOTS % 32 == 0 || slot < SLOTS) {
+            int2 o;
+            halves(X, o.x, o.y);
+            if (live) s_d[w][c][slot] = o;
+          }
+        }
+        if (live && (lane & (SLOTS - 1 < 31 ? SLOTS - 1 : 31)) == 0) {
+          // every axis multiplied by 6 / 16
+          constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;
+          const bool plain = em >= 2040 || (em < 83 && top != 0u);
+          // back * 2^(em - 1083): the exponent field moved
+          const double sc = __hiloint2double(__double2hiint(back) + ((em - 1083) * (1 << 20)), __double2loint(back));
+          s_sc[w][c] = plain ? -1.0 : (top == 0u ? 1.0 : sc);
+          s_uc[w][c] = uc;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+          const int slot = (CPI > 1) ? (lane & (SLOTS - 1)) : lane + 32 * k;
+          if (live && slot < SLOTS) s_d[w][c][slot] = d[k];
+        }
+        if (live && (lane & (SLOTS - 1 < 31 ? SLOTS - 1 : 31)) == 0) s_uc[w][c] = uc;
+      }
+    }
+    __syncwarp();
+    // ---- the tile's rows, one per lane
+    for (int32_t q = q0 + lane; q < q1; q += 32) {
+      const int64_t row = __ldg(A.crows + q);
+      const int c = (int)(__ldg(A.row_cell + q) - c0);
+      const T *tq = tc + 3 * (int64_t)q;
+      const T uc = s_uc[w][c];
+      const T ui = DIFF ? __ldg(ur + row * ld) : T(0);
+      T acc;
+      if constexpr (FX) {
+        int32_t wxh[4], wxl[4], wyh[4], wyl[4], wzh[4], wzl[4];
+        fixed_weights<NP>(__ldg(tq), wxh, wxl);
+        fixed_weights<NP>(__ldg(tq + 1), wyh, wyl);
+        if (DIM == 3) fixed_weights<NP>(__ldg(tq + 2), wzh, wzl);
+        const int4 *dn = reinterpret_cast<const int4 *>(&s_d[w][c][0]);
+        long long zh = 0, zr = 0;
+#pragma unroll
+        for (int cz = 0; cz < NZ; ++cz) {
+          long long yh = 0, yr = 0;
+#pragma unroll
+          for (int cy = 0; cy < NP; ++cy) {
+            const int4 p = dn[(cz * 4 + cy) * 2], s = dn[(cz * 4 + cy) * 2 + 1];
+            long long xh = 0, xr = 0;
+            mac(xh, xr, wxh[0], wxl[0], p.x, p.y);
+            mac(xh, xr, wxh[1], wxl[1], p.z, p.w);
+            mac(xh, xr, wxh[2], wxl[2], s.x, s.y);
+            if (NP == 4) mac(xh, xr, wxh[3], wxl[3], s.z, s.w);
+            int32_t lh, ll;
+            halves(xh + high_word(xr), lh, ll);
+            mac(yh, yr, wyh[cy], wyl[cy], lh, ll);
+          }
+          if constexpr (DIM == 3) {
+            int32_t mh, ml;
+            halves(yh + high_word(yr), mh, ml);
+            mac(zh, zr, wzh[cz], wzl[cz], mh, ml);
+          } else {
+            zh = yh;
+            zr = yr;
+          }
+        }
+        const double sc = s_sc[w][c];
+        const double base = DIFF ? uc - ui : uc;
+        if (sc > 0.0) {
+          acc = fma(sc, (double)(zh + high_word(zr)), base);
+        } else {
+          const int64_t cid = c0 + c;
+          const int lx = (int)(__ldg(A.ckey + cid) & 7u);
+          acc = slow_row<DIM, NP>(tq, A.lines + cid * 16, (lx + NP - 1 < 8) ? NP : 8 - lx, ur, ld, uc) + base;
+        }
+      } else {
+        T wx[4], wy[4], wz[4];
+        cpm_lagrange<NP, T>(__ldg(tq), wx);
+        cpm_lagrange<NP, T>(__ldg(tq + 1), wy);
+        if (DIM == 3) cpm_lagrange<NP, T>(__ldg(tq + 2), wz);
+        else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
+        const float4 *dn = reinterpret_cast<const float4 *>(&s_d[w][c][0]);
+        float2 p01 = make_float2(0.0f, 0.0f), p23 = p01;
+#pragma unroll
+        for (int cz = 0; cz < NZ; ++cz)
+#pragma unroll
+          for (int cy = 0; cy < NP; ++cy) {
+            const float g = wy[cy] * wz[cz];
+            const float4 p = dn[cz * 4 + cy];
+            p01 = __ffma2_rn(make_float2(g, g), make_float2(p.x, p.y), p01);
+            p23 = __ffma2_rn(make_float2(g, g), make_float2(p.z, p.w), p23);
+          }
+        acc = wx[0] * p01.x;
+        acc += wx[1] * p01.y;
+        acc += wx[2] * p23.x;
+        if (NP == 4) acc += wx[3] * p23.y;
+        acc += DIFF ? uc - ui : uc;
+      }
+      if (cs != T(1)) acc *= cs;
+      a[row * ld + r] = acc;
+    }
+    __syncwarp();
+  }
+}
+
+// a_i += sum over the row's flipped entries of w (u_twin - cs u_node): four lanes
+// per row and column.  A row has up to 32 flipped entries; one thread walking
+// them was a chain of that many dependent loads (20 us on the sphere at h = 1/128).
+template <typename T>
+__global__ void __launch_bounds__(256) correct_few_kernel(const int32_t *__restrict__ crow,
+                                                          const int32_t *__restrict__ cstart,
+                                                          const int32_t *__restrict__ cnode,
+                                                          const int32_t *__restrict__ ccol, const T *__restrict__ cw,
+                                                          int64_t ncorr, T cs, const T *__restrict__ u,
+                                                          T *__restrict__ a, int nrhs, int64_t ld) {
+  const int sub = threadIdx.x & 3;
+  const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 2;
+  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 2; t < ncorr * nrhs; t += stride) {
+    const int64_t q = (nrhs == 1) ? t : t / nrhs;
+    const int r = (nrhs == 1) ? 0 : (int)(t - q * nrhs);
+    const int32_t e1 = __ldg(cstart + q + 1);
+    T acc = T(0);
+    for (int32_t e = __ldg(cstart + q) + sub; e < e1; e += 4)
+      acc += __ldg(cw + e) * (__ldg(u + (int64_t)__ldg(ccol + e) * ld + r) - cs * __ldg(u + (int64_t)__ldg(cnode + e) * ld + r));
+    // the four lanes of a row are active together (the loop bound is theirs)
+    const unsigned m = 0xFu << (threadIdx.x & 28);
+    acc += __shfl_xor_sync(m, acc, 1);
+    acc += __shfl_xor_sync(m, acc, 2);
+    if (sub == 0) a[(int64_t)__ldg(crow + q) * ld + r] += acc;
+  }
+}
+
+template <typename T, bool DIFF, int DIM, int NP, int CT>
+void launch_tile(const cpm_ctx *c, const T *tc, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st) {
+  TileArgs A{c->d_cell_start, c->d_cell_rows, c->d_row_cell, c->d_cell_key,
+             reinterpret_cast<const int2 *>(c->d_cell_lines), c->ncells};
+  const int64_t tiles = (c->ncells + CT - 1) / CT;
+  gather_tile_kernel<T, DIFF, DIM, NP, CT><<<(unsigned)((tiles + TW - 1) / TW), TW * 32, 0, st>>>(A, tc, cs, u, a, nrhs,
+                                                                                                   ld);
+}
+
+template <typename T, bool DIFF>
+void launch_tile_any(const cpm_ctx *c, const T *tc, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st) {
+  // 16 cells (~88 rows: three passes of 32 lanes, 92 % of them at work) where
+  // that fills the SMs; 4 cells (two passes) on bands with fewer tiles than
+  // 8 warps per SM, whose time is the latency of one tile
+  const bool small = c->ncells < (int64_t)16 * 8 * c->nsm;
+#define CPM_TILE(D, NP)                                                             \
+  (small ? launch_tile<T, DIFF, D, NP, 4>(c, tc, cs, u, a, nrhs, ld, st)             \
+         : launch_tile<T, DIFF, D, NP, 16>(c, tc, cs, u, a, nrhs, ld, st))
+  if (c->dim == 3) {
+    if (c->p == 2) CPM_TILE(3, 3); else CPM_TILE(3, 4);
+  } else {
+    if (c->p == 2) CPM_TILE(2, 3); else CPM_TILE(2, 4);
+  }
+#undef CPM_TILE
+}
+
+}  // namespace
+
+template <typename T>
+int cpm_launch_correct_few(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st) {
+  if (c->ncorr == 0) return 0;
+  const T *cw;
+  if constexpr (sizeof(T) == 8) cw = reinterpret_cast<const T *>(c->d_corr_w64);
+  else cw = reinterpret_cast<const T *>(c->d_corr_w32);
+  correct_few_kernel<T><<<cpm_grid(4 * c->ncorr * nrhs, 256), 256, 0, st>>>(c->d_corr_row, c->d_corr_start,
+                                                                            c->d_corr_node, c->d_corr_col, cw,
+                                                                            c->ncorr, cs, u, a, nrhs, ld);
+  return 1;
+}
+
+template <typename T>
+int cpm_launch_gather_tile(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st,
+                           bool diff) {
+  if (c->ncells == 0) return 0;
+  const T *tc;
+  if constexpr (sizeof(T) == 8) tc = reinterpret_cast<const T *>(c->d_tc64);
+  else tc = reinterpret_cast<const T *>(c->d_tc32);
+  if (diff) launch_tile_any<T, true>(c, tc, cs, u, a, nrhs, ld, st);
+  else launch_tile_any<T, false>(c, tc, cs, u, a, nrhs, ld, st);
+  return 1 + cpm_launch_correct_few<T>(c, cs, u, a, nrhs, ld, st);
+}
+#define CPM_TILE_INST(T)                                                                                       \
+  template int cpm_launch_correct_few<T>(const cpm_ctx *, T, const T *, T *, int, int64_t, cudaStream_t);     \
+  template int cpm_launch_gather_tile<T>(const cpm_ctx *, T, const T *, T *, int, int64_t, cudaStream_t, bool);
+CPM_TILE_INST(float)
+CPM_TILE_INST(double)

@@ -1,0 +1,69 @@
+"""E u of one or a few columns by warp tiles (integer sums in FP64): every
+stencil shape, tiles that end ragged, odd column counts and strides, values at
+the ends of the exponent range, infinities and NaN, against the oracle.
+
+Tolerance: both sides round at most 64 products and 20 operations on weights of
+sum <= 1.25^3 in FP64, so they differ by at most (64 + 20) 2^-53 1.95 max|u| =
+1.9e-14 max|u|; FP32 (apply only, existing bar) 2e-6 of max|A u|."""
+import numpy as np
+import pytest
+
+import cpm_inputs as ci
+from gpu_common import SMALL, need_gpu, pair
+
+pytestmark = pytest.mark.gpu
+TOL = 84 * 2.0 ** -53 * 1.95
+
+
+def _wl(name):
+    if name.startswith("torus"):  # odd spacing: ragged cell counts
+        return ci.Workload("t", ci.torus(), 1 / 17.3, [ci.torus_meridian(0.3, 1.0, 0.4, ci.BC_DIR2)], 0.0, 1.0)
+    return SMALL[name]()
+
+
+@pytest.mark.parametrize("name", ["circle_dir1", "circle_dir2", "sphere_lat_dir2", "torus", "sphere_closed"])
+@pytest.mark.parametrize("p", [3, 2])
+def test_few_columns_match_oracle(oracle_mod, name, p):
+    torch = need_gpu()
+    w = _wl(name)
+    band, ref = pair(oracle_mod, w, p=p)
+    for nrhs in (1, 2, 3, 15):
+        U = ci.random_vector(ref.N, seed=nrhs, nrhs=nrhs).reshape(ref.N, -1)
+        Ug = torch.tensor(U if nrhs > 1 else U[:, 0], device="cuda")
+        a = band.extend(Ug).cpu().numpy().reshape(ref.NS, -1)
+        v = band.apply(0.0, 1.0, Ug).cpu().numpy().reshape(ref.N, -1)
+        v32 = band.apply(0.0, 1.0, Ug.float()).cpu().numpy().reshape(ref.N, -1)
+        for r in range(nrhs):
+            assert np.max(np.abs(a[:, r] - ref.extend(U[:, r])[:ref.NS])) <= TOL * np.max(np.abs(U[:, r]))
+            vr = ref.apply(0.0, 1.0, U[:, r])
+            assert np.max(np.abs(v[:, r] - vr)) <= 1e-14 * np.max(np.abs(vr))
+            assert np.max(np.abs(v32[:, r] - vr)) <= 2e-6 * np.max(np.abs(vr))
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -1060, 2.0 ** -950, 2.0 ** -600, 2.0 ** 600, 2.0 ** 1018])
+def test_ends_of_the_exponent_range(oracle_mod, scale):
+    """Scaled inputs give scaled outputs (absolute 64 denormals where they underflow)."""
+    torch = need_gpu()
+    w = SMALL["circle_dir2"]()
+    band, ref = pair(oracle_mod, w)
+    u = ci.random_vector(ref.N, seed=3)
+    u[::7] *= 1e-9   # neighbours of very different size
+    a = band.extend(torch.tensor(u * scale, device="cuda")).cpu().numpy()
+    er = ref.extend(u)[:ref.NS] * scale
+    assert np.max(np.abs(a - er)) <= TOL * scale + 64 * 2.0 ** -1074
+    assert not np.any(band.extend(torch.zeros(ref.N, dtype=torch.float64, device="cuda")).cpu().numpy())
+
+
+def test_infinities_and_nan_reach_the_same_rows(oracle_mod):
+    torch = need_gpu()
+    w = SMALL["sphere_closed"]()
+    band, ref = pair(oracle_mod, w)
+    for bad in (np.inf, -np.inf, np.nan):
+        u = ci.random_vector(ref.N, seed=4)
+        u[ref.N // 3] = bad
+        with np.errstate(all="ignore"):
+            er = ref.extend(u)[:ref.NS]
+        a = band.extend(torch.tensor(u, device="cuda")).cpu().numpy()
+        assert np.array_equal(np.isfinite(a), np.isfinite(er))
+        ok = np.isfinite(er)
+        assert np.max(np.abs(a[ok] - er[ok])) <= TOL
