@@ -251,8 +251,6 @@ cpm_status cpm_solve_adjoint(cpm_ctx *c, double m, double n, const double *g, do
                              const cpm_solve_opts *o, cpm_solve_stats *stats, void *stream) {
   cpm_status rc = check_solve(c, g, lam, nrhs, ld, o);
   if (rc) return rc;
-  rc = cpm_build_transpose(c);
-  if (rc) return rc;
   return cpm_internal_solve(c, true, m, n, g, lam, nrhs, ld, o, stats, as_stream(stream));
 }
 

@@ -4,172 +4,148 @@
 //   a = E u;  b = (L - diag L) a;  a = diag(L) u;  v = m u + n a + n b.
 // Here E and L are never stored for the bulk of the rows: each PDE row keeps
 // only the packed location of its interpolation stencil's base node and the
-// fractional position t (FP64 and FP32 copies); the cubic Lagrange weights are
-// formed in registers and the separable 4x4x4 gather runs along x-lines whose
-// DOFs are consecutive in the canonical order (a line crossing a brick face is
-// split in two runs).  Rows within 2 r of an interior boundary carry explicit
-// stencils with the crossing-test flips (Eq. 10).  Two kernels per product:
-//   gather : a_i = (E u)_i for PDE rows
-//   combine: v_i = (m + n diagL) u_i + (n/h^2) sum_nbr a_sigma(nbr)   (PDE rows)
-//            v_alpha = sum_beta B_alpha,beta u_beta                   (BC rows)
+// fractional position t (FP64 and FP32 copies).  Two steps per product:
+//   gather : a_i = (E u - u)_i for PDE rows (tile.cu up to 15 columns, cells.cu
+//            from 16), rows near an interior boundary with the crossing-test
+//            flips (Eq. 10) added as a sparse correction;
+//   combine: the FD stencil of the PDE rows and the BC rows
+//            v_alpha = sum_beta B_alpha,beta u_beta,
 // where a neighbour flipped to a BC DOF reads u of that DOF (E rows of BC DOFs
 // are the identity).
 #include <mutex>
 
 #include "apply.cuh"
 #include "cpm_internal.cuh"
+#include "fixed.cuh"
 
 namespace {
 
-template <typename T, bool DIFF, int NP>
-__device__ __forceinline__ T line_sum(const T *u, int64_t ld, int r, int32_t s0, int32_t s1, int split, const T *w,
-                                      T ui) {
-  // nodes 0..split-1 are consecutive from s0, nodes split..NP-1 consecutive from
-  // s1; a negative start (a node outside the band, excluded at set-up) reads
-  // nothing
-  T acc = T(0);
-#pragma unroll
-  for (int cx = 0; cx < NP; ++cx) {
-    int32_t st = (cx < split) ? s0 : s1;
-    int32_t idx = (cx < split) ? (s0 + cx) : (s1 + (cx - split));
-    if (st >= 0) {
-      T val = __ldg(u + (int64_t)idx * ld + r);
-      acc += w[cx] * (DIFF ? (val - ui) : val);
-    }
-  }
-  return acc;
+// ---- combine -----------------------------------------------------------------
+// With a holding the extension defects cs sum_j w_j (u_j - u_k) (the gather's
+// difference form), a PDE row is
+//   v_i = R { m cs u_i + (n/h^2) [ sum_{k PDE} (a_k + cs u_k - cs u_i)
+//             + sum_{k BC} (u_k - cs u_i) - n_missing cs u_i ] }.
+// FP32 sums the terms as they stand.  In FP64 the dozen additions a row are 12 of
+// the FP64 pipe's clocks per SM, which held the kernel at 82 % of that pipe (126 us
+// on the sphere at h = 1/128); there the u and the a differences are summed as
+// integers of one exponent each (fixed.cuh).  Neighbouring u within 6 binary
+// orders are represented exactly, so sum (u_k - u_i) is exact on smooth fields
+// and otherwise off by 2^-58 of the largest value, where each FP64 difference is
+// rounded at 2^-53 of itself.
+struct CombineArgs {
+  int64_t NS, N;
+  int nfd;
+  const int32_t *nbr8;  // [NS][8] FD neighbour columns, flipped near curves
+  const int32_t *bc_cnt, *bc_col;
+};
+
+template <typename T>
+struct CombineScale {
+  T m, c;    // R m cs, R n / h^2
+  T cs;
+};
+
+__device__ __forceinline__ void load_nbrs(const int32_t *nbr8, int64_t i, int32_t (&nb)[6]) {
+  const int4 n0 = __ldg(reinterpret_cast<const int4 *>(nbr8 + i * 8));
+  const int2 n1 = __ldg(reinterpret_cast<const int2 *>(nbr8 + i * 8 + 4));
+  nb[0] = n0.x; nb[1] = n0.y; nb[2] = n0.z; nb[3] = n0.w; nb[4] = n1.x; nb[5] = n1.y;
 }
 
-// DIFF: a_i = sum_j w_j (u_j - u_i), the extension's defect, instead of
-// sum_j w_j u_j.  Subtracting neighbouring values first keeps the rounding
-// error relative to the differences (exact when close, Sterbenz), which FP32
-// needs on smooth fields where the Laplacian cancels O(1) values to O(h^2).
-// cs scales the values of PDE DOFs on input (a right diagonal factor C: the
-// product is then E C u); BC DOFs enter unscaled.
-template <typename T, bool DIFF, int NP>
-__global__ void __launch_bounds__(256) gather_kernel(ApplyArgs<T> A, T cs, const T *__restrict__ u,
-                                                     T *__restrict__ a, int nrhs, int64_t ld) {
-  const int64_t NS = A.v.NS;
-  CPM_ROWS_COLS_LOOP(A.v.NS, nrhs, i, r) {
-    uint32_t rb = __ldg(A.rbase + i);
-    T acc = T(0);
-    const T ui = DIFF ? __ldg(u + i * ld + r) : T(0);
-    if (rb & CPM_SPECIAL_BIT) {
-      int64_t s = __ldg(A.spec_of + i);
-      const int32_t *ec = A.ecol + s * 64;
-      const T *ew = A.ew + s * 64;
-      for (int e = 0; e < 64; ++e) {
-        int32_t c = __ldg(ec + e);
-        if (c >= 0) {
-          const T val = __ldg(u + (int64_t)c * ld + r) * ((c < NS) ? cs : T(1));
-          acc += __ldg(ew + e) * (DIFF ? (val - cs * ui) : val);
-        }
-      }
-    } else {
-      int32_t b = (int32_t)((rb >> 9) & 0x3FFFFFu);
-      int l = (int)(rb & 511u);
-      int lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
-      T wx[4], wy[4], wz[4];
-      cpm_lagrange<NP, T>(__ldg(A.t + 3 * i), wx);
-      cpm_lagrange<NP, T>(__ldg(A.t + 3 * i + 1), wy);
-      const int nz = (A.v.dim == 3) ? NP : 1;
-      if (A.v.dim == 3) cpm_lagrange<NP, T>(__ldg(A.t + 3 * i + 2), wz);
-      else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
-      const int split = (lx + NP - 1 < 8) ? NP : 8 - lx;
-      for (int cz = 0; cz < nz; ++cz) {
-        T pz = T(0);
+// one row, one column: u0 = u_i; uk, ak the values at the neighbours nb (anything
+// where nb < 0, ak anything where the neighbour is a BC DOF)
+__device__ __forceinline__ float combine_row(const CombineScale<float> &S, int64_t NS, int nfd, const int32_t (&nb)[6],
+                                             float u0, const float (&uk)[6], const float (&ak)[6]) {
+  const float ui = S.cs * u0;
+  float s = 0.0f;
+  int present = 0;
 #pragma unroll
-        for (int cy = 0; cy < NP; ++cy) {
-          int32_t s0 = cpm_node_index(A.v, b, lx, ly + cy, lz + cz);
-          int32_t s1 = (split < NP) ? cpm_node_index(A.v, b, 8, ly + cy, lz + cz) : 0;
-          pz += wy[cy] * line_sum<T, DIFF, NP>(u, ld, r, s0, s1, split, wx, ui);
-        }
-        acc += wz[cz] * pz;
-      }
-      acc *= cs;
-    }
-    a[i * ld + r] = acc;
+  for (int k = 0; k < 6; ++k) {
+    if (nb[k] < 0) continue;
+    ++present;
+    s += (nb[k] < NS) ? ak[k] + (S.cs * uk[k] - ui) : uk[k] - ui;
   }
+  return S.m * u0 + S.c * (s - (float)(nfd - present) * ui);
 }
 
-// DIFF: a holds the extension defects sum_j w_j (u_j - u_k), and the row is
-// m u_i + (n/h^2) [ sum_present (a_k + (u_k - u_i)) - n_missing u_i ],
-// the same value as m u_i + n [diag(L) u_i + (1/h^2) sum_present (E u)_k].
-template <typename T, bool DIFF>
-__global__ void __launch_bounds__(256) combine_kernel(ApplyArgs<T> A, T m, T n, T rowscale, T cs,
+__device__ __forceinline__ double combine_row_plain(const CombineScale<double> &S, int64_t NS, int nfd,
+                                                 const int32_t (&nb)[6], double u0, const double (&uk)[6],
+                                                 const double (&ak)[6]) {
+  const double ui = S.cs * u0;
+  double s = 0.0;
+  int present = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    if (nb[k] < 0) continue;
+    ++present;
+    s += (nb[k] < NS) ? ak[k] + (S.cs * uk[k] - ui) : uk[k] - ui;
+  }
+  return S.m * u0 + S.c * (s - (nfd - present) * ui);
+}
+
+__device__ __forceinline__ double combine_row(const CombineScale<double> &S, int64_t NS, int nfd,
+                                              const int32_t (&nb)[6], double u0, const double (&uk)[6],
+                                              const double (&ak)[6]) {
+  unsigned tu = fx_key(u0), ta = 0;
+  int npde = 0, nbc = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    if (nb[k] >= 0 && nb[k] < NS) {
+      ++npde;
+      tu = max(tu, fx_key(uk[k]));
+      ta = max(ta, fx_key(ak[k]));
+    }
+    nbc += nb[k] >= NS;
+  }
+  const int eu = (int)(tu >> 20), ea = (int)(ta >> 20);
+  const int ecs = ((__double2hiint(S.cs) >> 20) & 0x7FF) + eu - 1081;
+  if (fx_ok(tu) && fx_ok(ta) && (tu == 0u || (ecs >= 1 && ecs <= 2046))) {
+    // 12 values below 2^59: no overflow
+    long long su = 0, sa = 0;
+    const long long x0 = fx_of(u0, eu, 6);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      if (nb[k] >= 0 && nb[k] < NS) {
+        su += fx_of(uk[k], eu, 6) - x0;
+        sa += fx_of(ak[k], ea, 6);
+      }
+    double s = (ta == 0u) ? 0.0 : (double)sa * fx_scale(1.0, ea - 1081);
+    if (tu != 0u) s = fma((double)su, fx_scale(S.cs, eu - 1081), s);
+    if (nbc) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (nb[k] >= NS) s += uk[k] - S.cs * u0;
+    }
+    const int miss = nfd - npde - nbc;
+    if (miss) s -= miss * (S.cs * u0);
+    return fma(S.c, s, S.m * u0);
+  }
+  return combine_row_plain(S, NS, nfd, nb, u0, uk, ak);
+}
+
+// a few columns: one thread per element
+template <typename T>
+__global__ void __launch_bounds__(256) combine_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val,
                                                       const T *__restrict__ u, const T *__restrict__ a,
                                                       T *__restrict__ v, int nrhs, int64_t ld) {
-  const int64_t NS = A.v.NS, N = NS + A.v.NC;
-  const T inv_h2 = T(A.v.inv_h * A.v.inv_h);
-  const T diag = m + n * T(-2.0 * A.v.dim * A.v.inv_h * A.v.inv_h);
-  const int nfd = 2 * A.v.dim;
-  CPM_ROWS_COLS_LOOP(N, nrhs, i, r) {
-    if (i < NS) {
-      uint32_t rb = __ldg(A.rbase + i);
-      const T ui = cs * __ldg(u + i * ld + r);
-      T s = T(0);
-      int present = 0;
-      if (A.nbr8) {
-        // the precomputed neighbour table (flipped columns included)
-        const int4 n0 = __ldg(reinterpret_cast<const int4 *>(A.nbr8 + i * 8));
-        const int2 n1 = __ldg(reinterpret_cast<const int2 *>(A.nbr8 + i * 8 + 4));
-        const int32_t nb[6] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y};
+  CPM_ROWS_COLS_LOOP(A.N, nrhs, i, r) {
+    if (i < A.NS) {
+      int32_t nb[6];
+      load_nbrs(A.nbr8, i, nb);
+      T uk[6], ak[6];
+      const T u0 = __ldg(u + i * ld + r);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          const int32_t c = nb[k];
-          if (c < 0) continue;
-          ++present;
-          if (c < NS) {
-            const T ac = __ldg(a + (int64_t)c * ld + r);
-            s += DIFF ? ac + (cs * __ldg(u + (int64_t)c * ld + r) - ui) : ac;
-          } else {
-            const T uc = __ldg(u + (int64_t)c * ld + r);
-            s += DIFF ? (uc - ui) : uc;
-          }
-        }
-      } else if (rb & CPM_SPECIAL_BIT) {
-        int64_t sp = __ldg(A.spec_of + i);
-        for (int k = 0; k < 6; ++k) {
-          int32_t c = __ldg(A.fcol + sp * 6 + k);
-          if (c < 0) continue;
-          ++present;
-          const T uc = __ldg(u + (int64_t)c * ld + r) * ((c < NS) ? cs : T(1));
-          if (DIFF) s += (c < NS) ? (__ldg(a + (int64_t)c * ld + r) + (uc - ui)) : (uc - ui);
-          else s += (c < NS) ? __ldg(a + (int64_t)c * ld + r) : uc;
-        }
-      } else {
-        uint32_t rs = __ldg(A.rself + i);
-        int32_t b = (int32_t)(rs >> 9);
-        int l = (int)(rs & 511u);
-        int lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
-        int32_t nbr[6];
-        nbr[0] = cpm_node_index(A.v, b, lx - 1, ly, lz);
-        nbr[1] = cpm_node_index(A.v, b, lx + 1, ly, lz);
-        nbr[2] = cpm_node_index(A.v, b, lx, ly - 1, lz);
-        nbr[3] = cpm_node_index(A.v, b, lx, ly + 1, lz);
-        nbr[4] = (A.v.dim == 3) ? cpm_node_index(A.v, b, lx, ly, lz - 1) : -1;
-        nbr[5] = (A.v.dim == 3) ? cpm_node_index(A.v, b, lx, ly, lz + 1) : -1;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-          int32_t j = nbr[k];
-          if (j < 0) continue;
-          ++present;
-          T aj = __ldg(a + (int64_t)j * ld + r);
-          if (DIFF) s += aj + (cs * __ldg(u + (int64_t)j * ld + r) - ui);
-          else s += aj;
-        }
+      for (int k = 0; k < 6; ++k) {
+        uk[k] = (nb[k] >= 0) ? __ldg(u + (int64_t)nb[k] * ld + r) : T(0);
+        ak[k] = (nb[k] >= 0 && nb[k] < A.NS) ? __ldg(a + (int64_t)nb[k] * ld + r) : T(0);
       }
-      T val;
-      if (DIFF) val = m * ui + (n * inv_h2) * (s - T(nfd - present) * ui);
-      else val = diag * ui + (n * inv_h2) * s;
-      v[i * ld + r] = rowscale * val;
+      v[i * ld + r] = combine_row(S, A.NS, A.nfd, nb, u0, uk, ak);
     } else {
-      int64_t al = i - NS;
-      int cnt = __ldg(A.bc_cnt + al);
+      const int64_t al = i - A.NS;
+      const int cnt = __ldg(A.bc_cnt + al);
       T s = T(0);
       for (int e = 0; e < cnt; ++e) {
         const int32_t c = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
-        s += __ldg(A.bc_val + al * CPM_BC_STRIDE + e) * (__ldg(u + (int64_t)c * ld + r) * ((c < NS) ? cs : T(1)));
+        s += __ldg(bc_val + al * CPM_BC_STRIDE + e) * (__ldg(u + (int64_t)c * ld + r) * ((c < A.NS) ? S.cs : T(1)));
       }
       v[i * ld + r] = s;
     }
@@ -178,15 +154,13 @@ __global__ void __launch_bounds__(256) combine_kernel(ApplyArgs<T> A, T m, T n, 
 
 // ---- batched combine: one warp per row, lanes over right-hand sides ---------
 // With many right-hand sides the FD stencil is the same for every column, so
-// one warp reads it once per row and each lane carries RPL columns
-// (r = lane * RPL + k): every neighbour is one coalesced load of 32 * RPL
-// contiguous values ([N][ld] layout, ld a multiple of RPL).  The extension
-// values a = E u come from the cell-bucketed gather (cells.cu).
+// one warp reads it once per row and each lane carries RPL adjacent columns per
+// group of 32 RPL: every neighbour is one coalesced load ([N][ld] layout, ld a
+// multiple of RPL).
 template <typename T, int RPL>
 struct Vec;
 template <> struct Vec<float, 1> { typedef float t; };
 template <> struct Vec<float, 2> { typedef float2 t; };
-template <> struct Vec<float, 4> { typedef float4 t; };
 template <> struct Vec<double, 1> { typedef double t; };
 template <> struct Vec<double, 2> { typedef double2 t; };
 
@@ -209,105 +183,94 @@ __device__ __forceinline__ void stv(T *p, const T in[RPL]) {
   *reinterpret_cast<V *>(p) = v;
 }
 
-template <typename T, bool DIFF, int RPL>
-__global__ void __launch_bounds__(256) combine_batched_kernel(ApplyArgs<T> A, T m, T n, T rowscale, T cs,
-                                                              const T *__restrict__ u, const T *__restrict__ a,
-                                                              T *__restrict__ v, int nrhs, int64_t ld) {
+// A block takes `chunk` consecutive rows, its 8 warps 8 of them at a time, so
+// that the y neighbours (8 rows away inside a brick) are still in L1.
+template <typename T, int RPL>
+__global__ void __launch_bounds__(256) combine_batched_kernel(CombineArgs A, CombineScale<T> S,
+                                                              const T *__restrict__ bc_val, const T *__restrict__ u,
+                                                              const T *__restrict__ a, T *__restrict__ v, int nrhs,
+                                                              int64_t ld, int chunk) {
   const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int col = lane * RPL;
-  const bool on = col < nrhs;
-  const int64_t NS = A.v.NS, N = NS + A.v.NC;
-  const T inv_h2 = T(A.v.inv_h * A.v.inv_h);
-  const T diag = m + n * T(-2.0 * A.v.dim * A.v.inv_h * A.v.inv_h);
-  const int nfd = 2 * A.v.dim;
-  for (int64_t i = warp; i < N; i += nwarps) {
-    T out[RPL];
-    if (i < NS) {
-      int32_t nbr[6];
-      if (A.nbr8) {
-        const int4 n0 = __ldg(reinterpret_cast<const int4 *>(A.nbr8 + i * 8));
-        const int2 n1 = __ldg(reinterpret_cast<const int2 *>(A.nbr8 + i * 8 + 4));
-        nbr[0] = n0.x; nbr[1] = n0.y; nbr[2] = n0.z; nbr[3] = n0.w; nbr[4] = n1.x; nbr[5] = n1.y;
-      } else if (__ldg(A.rbase + i) & CPM_SPECIAL_BIT) {
-        int64_t sp = __ldg(A.spec_of + i);
+  for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < A.N; c0 += (int64_t)gridDim.x * chunk) {
+    const int64_t c1 = (c0 + chunk < A.N) ? c0 + chunk : A.N;
+    for (int64_t i = c0 + (threadIdx.x >> 5); i < c1; i += 8) {
+      int32_t nb[6];
+      if (i < A.NS) load_nbrs(A.nbr8, i, nb);
+      for (int col = lane * RPL; col < nrhs; col += 32 * RPL) {
+        T out[RPL];
+        if (i < A.NS) {
+          T u0[RPL], uk[6][RPL], ak[6][RPL];
+          ldv<T, RPL>(u + i * ld + col, u0);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) nbr[k] = __ldg(A.fcol + sp * 6 + k);
-      } else {
-        uint32_t rs = __ldg(A.rself + i);
-        int32_t b = (int32_t)(rs >> 9);
-        int l = (int)(rs & 511u);
-        int lx = l & 7, ly = (l >> 3) & 7, lz = l >> 6;
-        nbr[0] = cpm_node_index(A.v, b, lx - 1, ly, lz);
-        nbr[1] = cpm_node_index(A.v, b, lx + 1, ly, lz);
-        nbr[2] = cpm_node_index(A.v, b, lx, ly - 1, lz);
-        nbr[3] = cpm_node_index(A.v, b, lx, ly + 1, lz);
-        nbr[4] = (A.v.dim == 3) ? cpm_node_index(A.v, b, lx, ly, lz - 1) : -1;
-        nbr[5] = (A.v.dim == 3) ? cpm_node_index(A.v, b, lx, ly, lz + 1) : -1;
-      }
-      if (!on) continue;
-      T ui[RPL], s[RPL];
-      ldv<T, RPL>(u + i * ld + col, ui);
+          for (int q = 0; q < 6; ++q) {
 #pragma unroll
-      for (int k = 0; k < RPL; ++k) {
-        ui[k] *= cs;
-        s[k] = T(0);
-      }
-      int present = 0;
+            for (int k = 0; k < RPL; ++k) uk[q][k] = ak[q][k] = T(0);
+            if (nb[q] >= 0) ldv<T, RPL>(u + (int64_t)nb[q] * ld + col, uk[q]);
+            if (nb[q] >= 0 && nb[q] < A.NS) ldv<T, RPL>(a + (int64_t)nb[q] * ld + col, ak[q]);
+          }
 #pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        int32_t c = nbr[q];
-        if (c < 0) continue;
-        ++present;
-        T uc[RPL], ac[RPL];
-        if (DIFF || c >= NS) ldv<T, RPL>(u + (int64_t)c * ld + col, uc);
-        if (c < NS) ldv<T, RPL>(a + (int64_t)c * ld + col, ac);
-        const T sc_c = (c < NS) ? cs : T(1);
+          for (int k = 0; k < RPL; ++k) {
+            T x[6], y[6];
 #pragma unroll
-        for (int k = 0; k < RPL; ++k) {
-          uc[k] *= sc_c;
-          if (DIFF) s[k] += (c < NS) ? (ac[k] + (uc[k] - ui[k])) : (uc[k] - ui[k]);
-          else s[k] += (c < NS) ? ac[k] : uc[k];
+            for (int q = 0; q < 6; ++q) { x[q] = uk[q][k]; y[q] = ak[q][k]; }
+            out[k] = combine_row(S, A.NS, A.nfd, nb, u0[k], x, y);
+          }
+        } else {
+          const int64_t al = i - A.NS;
+          const int cnt = __ldg(A.bc_cnt + al);
+#pragma unroll
+          for (int k = 0; k < RPL; ++k) out[k] = T(0);
+          for (int e = 0; e < cnt; ++e) {
+            const int32_t cc = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
+            const T w = __ldg(bc_val + al * CPM_BC_STRIDE + e) * ((cc < A.NS) ? S.cs : T(1));
+            T val[RPL];
+            ldv<T, RPL>(u + (int64_t)cc * ld + col, val);
+#pragma unroll
+            for (int k = 0; k < RPL; ++k) out[k] += w * val[k];
+          }
         }
-      }
-#pragma unroll
-      for (int k = 0; k < RPL; ++k) {
-        T val = DIFF ? (m * ui[k] + (n * inv_h2) * (s[k] - T(nfd - present) * ui[k]))
-                     : (diag * ui[k] + (n * inv_h2) * s[k]);
-        out[k] = rowscale * val;
-      }
-    } else {
-      if (!on) continue;
-      int64_t al = i - NS;
-      int cnt = __ldg(A.bc_cnt + al);
-#pragma unroll
-      for (int k = 0; k < RPL; ++k) out[k] = T(0);
-      for (int e = 0; e < cnt; ++e) {
-        const int32_t cc = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
-        const T w = __ldg(A.bc_val + al * CPM_BC_STRIDE + e) * ((cc < NS) ? cs : T(1));
-        T val[RPL];
-        ldv<T, RPL>(u + (int64_t)cc * ld + col, val);
-#pragma unroll
-        for (int k = 0; k < RPL; ++k) out[k] += w * val[k];
+        stv<T, RPL>(v + i * ld + col, out);
       }
     }
-    stv<T, RPL>(v + i * ld + col, out);
   }
+}
+
+template <typename T>
+void combine_args(const cpm_ctx *c, T m, T n, T rowscale, T cs, CombineArgs *A, CombineScale<T> *S, const T **bc_val) {
+  *A = CombineArgs{c->NS, c->NS + c->NC, 2 * c->dim, c->d_nbr8, c->d_bc_cnt, c->d_bc_col};
+  const double inv_h = 1.0 / c->h;
+  *S = CombineScale<T>{(T)((double)rowscale * (double)m * (double)cs),
+                       (T)((double)rowscale * (double)n * (inv_h * inv_h)), cs};
+  if constexpr (sizeof(T) == 8) *bc_val = reinterpret_cast<const T *>(c->d_bc_val);
+  else *bc_val = reinterpret_cast<const T *>(c->d_bc_val32);
+}
+
+template <typename T>
+void launch_combine(const cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, const T *a, T *v, int nrhs, int64_t ld,
+                    cudaStream_t st) {
+  CombineArgs A;
+  CombineScale<T> S;
+  const T *bv;
+  combine_args<T>(c, m, n, rowscale, cs, &A, &S, &bv);
+  combine_kernel<T><<<cpm_grid(A.N * nrhs, 256), 256, 0, st>>>(A, S, bv, u, a, v, nrhs, ld);
 }
 
 // batched product: E u for all PDE rows through the cell-bucketed gather
 // (cells.cu), then the warp-per-row combine
 template <typename T, int RPL>
-static int launch_batched(const cpm_ctx *c, const ApplyArgs<T> &A, T m, T n, T rowscale, T cs, const T *u, T *a,
-                          T *v, int nrhs, int64_t ld, cudaStream_t st, bool diff) {
+int launch_batched(const cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T *a, T *v, int nrhs, int64_t ld,
+                   cudaStream_t st) {
+  CombineArgs A;
+  CombineScale<T> S;
+  const T *bv;
+  combine_args<T>(c, m, n, rowscale, cs, &A, &S, &bv);
   // 8 warps per block; by default 8 blocks per SM
   const int64_t warps = (int64_t)c->nsm * (c->tune.combine_warps_per_sm > 0 ? c->tune.combine_warps_per_sm : 64);
-  unsigned g = (unsigned)std::min<int64_t>((A.v.NS + A.v.NC + 7) / 8, warps / 8);
+  const int chunk = 64;
+  unsigned g = (unsigned)std::min<int64_t>((A.N + chunk - 1) / chunk, warps / 8);
   if (g < 1) g = 1;
-  int launched = 1 + cpm_launch_gather_cells<T>(c, A, cs, u, a, nrhs, ld, st, diff, RPL);
-  if (diff) combine_batched_kernel<T, true, RPL><<<g, 256, 0, st>>>(A, m, n, rowscale, cs, u, a, v, nrhs, ld);
-  else combine_batched_kernel<T, false, RPL><<<g, 256, 0, st>>>(A, m, n, rowscale, cs, u, a, v, nrhs, ld);
+  const int launched = 1 + cpm_launch_gather_cells<T>(c, cs, u, a, nrhs, ld, st, true, RPL);
+  combine_batched_kernel<T, RPL><<<g, 256, 0, st>>>(A, S, bv, u, a, v, nrhs, ld, chunk);
   return launched;
 }
 
@@ -423,68 +386,34 @@ ApplyArgs<T> cpm_apply_args(const cpm_ctx *c) {
   return A;
 }
 
-template <typename T>
-void cpm_launch_gather(const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st,
-                       bool diff) {
-  const unsigned g = cpm_grid(A.v.NS * nrhs, 256);
-  if (A.v.np1 == 3) {
-    if (diff) gather_kernel<T, true, 3><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
-    else gather_kernel<T, false, 3><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
-  } else {
-    if (diff) gather_kernel<T, true, 4><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
-    else gather_kernel<T, false, 4><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
-  }
-}
-
-template <typename T>
-void cpm_launch_combine(const ApplyArgs<T> &A, T m, T n, T rowscale, T cs, const T *u, const T *a, T *v, int nrhs,
-                        int64_t ld, cudaStream_t st, bool diff) {
-  unsigned g = cpm_grid((A.v.NS + A.v.NC) * nrhs, 256);
-  if (diff) combine_kernel<T, true><<<g, 256, 0, st>>>(A, m, n, rowscale, cs, u, a, v, nrhs, ld);
-  else combine_kernel<T, false><<<g, 256, 0, st>>>(A, m, n, rowscale, cs, u, a, v, nrhs, ld);
-}
-
 template ApplyArgs<double> cpm_apply_args<double>(const cpm_ctx *);
 template ApplyArgs<float> cpm_apply_args<float>(const cpm_ctx *);
-template void cpm_launch_gather<double>(const ApplyArgs<double> &, double, const double *, double *, int, int64_t,
-                                        cudaStream_t, bool);
-template void cpm_launch_gather<float>(const ApplyArgs<float> &, float, const float *, float *, int, int64_t,
-                                       cudaStream_t, bool);
-template void cpm_launch_combine<double>(const ApplyArgs<double> &, double, double, double, double, const double *,
-                                         const double *, double *, int, int64_t, cudaStream_t, bool);
-template void cpm_launch_combine<float>(const ApplyArgs<float> &, float, float, float, float, const float *,
-                                        const float *, float *, int, int64_t, cudaStream_t, bool);
 
 // the kernels of one product v = R A C u with the intermediate a ([N_S][ld]);
 // returns the number of launches
 template <typename T>
 static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T *a, T *v, int nrhs, int64_t ld,
                           cudaStream_t st) {
-  ApplyArgs<T> A = cpm_apply_args<T>(c);
-  const bool diff = true;
-  // batched layouts whose columns fill whole warps use the warp-per-row kernels;
-  // two adjacent columns per lane need an even column count and 2-element alignment
+  // from 16 columns on a warp holds a cell for a group of columns; two adjacent
+  // columns per lane need an even column count and 2-element alignment
   const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
                                            reinterpret_cast<uintptr_t>(a)) % (2 * sizeof(T)) == 0);
-  if (nrhs > 32 && nrhs <= 64 && nrhs % 2 == 0 && aligned2)
-    return launch_batched<T, 2>(c, A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
-  if (nrhs >= 16 && nrhs <= 32)
-    return launch_batched<T, 1>(c, A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
+  if (nrhs > 32 && nrhs % 2 == 0 && aligned2)
+    return launch_batched<T, 2>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);
+  if (nrhs >= 16) return launch_batched<T, 1>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);
   int launched = 0;
-  if (nrhs == 1 && c->ncells > 0 && c->tune.single_mode == 2) {
-    launched = cpm_launch_fused1<T>(c, A, m, n, rowscale, cs, u, a, v, st);
-    if (launched) return launched;
+  if (nrhs == 1 && c->ncells > 0 && c->tune.single_mode != 0) {
+    ApplyArgs<T> A = cpm_apply_args<T>(c);
+    if (c->tune.single_mode == 2) {
+      launched = cpm_launch_fused1<T>(c, A, m, n, rowscale, cs, u, a, v, st);
+      if (launched) return launched;
+    } else {
+      cpm_launch_gather1<T>(c, A, cs, u, a, st);
+      launched = 1 + cpm_launch_correct_few<T>(c, cs, u, a, 1, ld, st);
+    }
   }
-  if (nrhs == 1 && c->ncells > 0 && c->tune.single_mode == 1) {
-    cpm_launch_gather1<T>(c, A, cs, u, a, st);
-    launched = 1 + cpm_launch_correct_few<T>(c, cs, u, a, 1, ld, st);
-  } else if (nrhs < 16) {
-    launched = cpm_launch_gather_tile<T>(c, cs, u, a, nrhs, ld, st, diff);
-  } else {
-    cpm_launch_gather<T>(A, cs, u, a, nrhs, ld, st, diff);
-    launched = 1;
-  }
-  cpm_launch_combine<T>(A, m, n, rowscale, cs, u, a, v, nrhs, ld, st, diff);
+  if (launched == 0) launched = cpm_launch_gather_tile<T>(c, cs, u, a, nrhs, ld, st, true);
+  launch_combine<T>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);
   return launched + 1;
 }
 
@@ -543,7 +472,7 @@ void cpm_prof_end(cpm_ctx *c, cudaStream_t st, int64_t row_rhs) {
 
 cpm_status cpm_internal_extend(cpm_ctx *c, const double *u, double *a, int nrhs, int64_t ld, cudaStream_t st) {
   if (nrhs < 16) cpm_launch_gather_tile<double>(c, 1.0, u, a, nrhs, ld, st, false);
-  else cpm_launch_gather<double>(cpm_apply_args<double>(c), 1.0, u, a, nrhs, ld, st, false);
+  else cpm_launch_gather_cells<double>(c, 1.0, u, a, nrhs, ld, st, false, 1);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }

@@ -24,12 +24,6 @@ struct ApplyArgs {
 
 template <typename T>
 ApplyArgs<T> cpm_apply_args(const cpm_ctx *c);
-template <typename T>
-void cpm_launch_gather(const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st,
-                       bool diff);
-template <typename T>
-void cpm_launch_combine(const ApplyArgs<T> &A, T m, T n, T rowscale, T cs, const T *u, const T *a, T *v, int nrhs,
-                        int64_t ld, cudaStream_t st, bool diff);
 // v = R A C u: R scales the PDE rows of the result, C the PDE entries of the
 // input (diagonal row scaling and right preconditioning without extra vectors)
 template <typename T>
@@ -52,8 +46,8 @@ cpm_status cpm_apply_transpose_T(cpm_ctx *c, double m, double n, const T *u, T *
 // cell-bucketed E u for all PDE rows plus the flipped-entry correction of the
 // rows near curves (batched layouts); returns the number of kernels launched
 template <typename T>
-int cpm_launch_gather_cells(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
-                            cudaStream_t st, bool diff, int rpl);
+int cpm_launch_gather_cells(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st, bool diff,
+                            int rpl);
 
 cpm_status cpm_internal_surface_gradient(cpm_ctx *c, const double *u, double *X, int normalize, cudaStream_t st);
 cpm_status cpm_internal_surface_divergence(cpm_ctx *c, const double *X, double *b, cudaStream_t st);

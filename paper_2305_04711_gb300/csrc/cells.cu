@@ -20,6 +20,7 @@
 
 #include "apply.cuh"
 #include "cpm_internal.cuh"
+#include "fixed.cuh"
 #include "util.cuh"
 
 namespace {
@@ -135,6 +136,13 @@ __global__ void corr_fill_kernel(BandView v, const int32_t *spec_row, int64_t ns
 constexpr int CHUNK = 8;   // rows of a cell whose weights are staged together
 constexpr int WARPS = 8;   // warps per block
 
+struct CellArgs {
+  const int32_t *cstart, *crows;
+  const uint32_t *ckey;
+  const int2 *lines;
+  int64_t ncells;
+};
+
 template <typename T, int R>
 struct VecT;
 template <> struct VecT<float, 1> { typedef float t; };
@@ -187,55 +195,81 @@ __device__ __forceinline__ void sub_v<float, 2>(float (&d)[2], const float (&c)[
   d[1] = o.y;
 }
 
+// what a cell's warp reads before its node values: the stencil line starts (lane
+// ln < 16) and the brick-face split; the index of node x of line ln is
+// x < split ? s0 + x : s1 + x - split
+struct CellHead {
+  int2 line;
+  int split;
+  int32_t r0, r1;
+};
+
+template <int NP>
+__device__ __forceinline__ CellHead cell_head(const CellArgs &A, int64_t cid, int lane) {
+  CellHead h;
+  const int lx = (int)(__ldg(A.ckey + cid) & 7u);
+  h.split = (lx + NP - 1 < 8) ? NP : 8 - lx;
+  h.line = __ldg(A.lines + cid * 16 + (lane & 15));
+  h.r0 = __ldg(A.cstart + cid);
+  h.r1 = __ldg(A.cstart + cid + 1);
+  return h;
+}
+
 // One warp per cell; each lane takes R adjacent columns (32 R per group).  For
 // a group the lane loads the cell's node values (NX x positions per pass, XH
 // passes) into registers and applies each row of the cell: the y-z weights
 // along each x position (P[cx] = sum_{cy,cz} w_y w_z u), then the x weights.
-// Partial sums of the passes wait in shared memory.
+// Partial sums of the passes wait in shared memory.  A block's warps take
+// neighbouring cells, which share most of their nodes in L1, and a warp reads
+// the head and the fractions of its next cell while it works on this one.
 //
-// DIFF (the FP32 form): the node values enter as differences to the cell's
-// base-node value u_c and each row adds u_c - u_i, which equals
-// sum_n w_n (u_n - u_i) since sum_n w_n = 1; rounding then stays relative to
-// local differences.
-template <typename T, bool DIFF, int DIM, int NP, int XH, int R>
-__global__ void __launch_bounds__(WARPS * 32, 2)
-    gather_cells_kernel(ApplyArgs<T> A, const int32_t *__restrict__ cstart, const uint32_t *__restrict__ ckey,
-                        const int32_t *__restrict__ crows, int64_t ncells, T cs, const T *__restrict__ u,
-                        T *__restrict__ a, int nrhs, int64_t ld_) {
+// The node values enter as differences to the cell's base-node value u_c and
+// each row adds u_c - u_i, which equals sum_n w_n (u_n - u_i) since
+// sum_n w_n = 1; rounding then stays relative to local differences.
+template <int DIM, int NP, int XH, int R>
+__global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
+    gather_cells_kernel(CellArgs A, const float *__restrict__ tc, float cs, const float *__restrict__ u,
+                        float *__restrict__ a, int nrhs, int64_t ld_) {
+  typedef float T;
   constexpr int NZ = (DIM == 3) ? NP : 1;
   constexpr int NL = NP * NZ;  // stencil lines along x
-  constexpr int NN = NP * NL;  // stencil nodes
   constexpr int NX = NP / XH;  // x positions per pass
   static_assert(NX * XH == NP, "passes must split the stencil's x positions");
   typedef typename VecT<T, R>::t V;
   __shared__ __align__(16) T s_wyz[WARPS][CHUNK][NL];
   __shared__ __align__(16) T s_wx[WARPS][CHUNK][4];
   __shared__ int32_t s_row[WARPS][CHUNK];
-  __shared__ __align__(16) int32_t s_idx[WARPS][NN];
+  __shared__ __align__(16) int32_t s_idx[WARPS][16 * 4];
   __shared__ V s_acc[(XH > 1) ? WARPS : 1][CHUNK][32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int ngroups = (nrhs + 32 * R - 1) / (32 * R);
-  for (int64_t cid = warp; cid < ncells; cid += nwarps) {
-    const uint32_t key = __ldg(ckey + cid);
-    // node (x, line) at s_idx[line * NP + x], line = cz * NP + cy
-    for (int e = lane; e < NN; e += 32) {
-      const int x = e % NP, ln = e / NP;
-      s_idx[wib][e] = entry_node(A.v, key, x + 4 * (ln % NP) + 16 * (ln / NP));
+  if (warp >= A.ncells) return;
+  CellHead h = cell_head<NP>(A, warp, lane);
+  for (int64_t cid = warp; cid < A.ncells; cid += nwarps) {
+    // node x of line cz * 4 + cy at s_idx[line * 4 + x]
+    if (lane < 16) {
+      int4 o;
+      o.x = h.line.x;
+      o.y = (1 < h.split) ? h.line.x + 1 : h.line.y + (1 - h.split);
+      o.z = (2 < h.split) ? h.line.x + 2 : h.line.y + (2 - h.split);
+      o.w = (3 < h.split) ? h.line.x + 3 : h.line.y + (3 - h.split);
+      *reinterpret_cast<int4 *>(&s_idx[wib][lane * 4]) = o;
     }
+    const int32_t r0 = h.r0, r1 = h.r1;
+    if (cid + nwarps < A.ncells) h = cell_head<NP>(A, cid + nwarps, lane);
     __syncwarp();
     const int32_t base = s_idx[wib][0];
-    const int32_t r0 = __ldg(cstart + cid), r1 = __ldg(cstart + cid + 1);
     for (int32_t c0 = r0; c0 < r1; c0 += CHUNK) {
       const int k = min(CHUNK, r1 - c0);
       if (lane < k) {
-        const int32_t row = __ldg(crows + c0 + lane);
-        s_row[wib][lane] = row;
+        s_row[wib][lane] = __ldg(A.crows + c0 + lane);
+        const T *tq = tc + 3 * (int64_t)(c0 + lane);
         T wx[4], wy[4], wz[4];
-        cpm_lagrange<NP, T>(__ldg(A.t + 3 * (int64_t)row), wx);
-        cpm_lagrange<NP, T>(__ldg(A.t + 3 * (int64_t)row + 1), wy);
-        if (DIM == 3) cpm_lagrange<NP, T>(__ldg(A.t + 3 * (int64_t)row + 2), wz);
+        cpm_lagrange<NP, T>(__ldg(tq), wx);
+        cpm_lagrange<NP, T>(__ldg(tq + 1), wy);
+        if (DIM == 3) cpm_lagrange<NP, T>(__ldg(tq + 2), wz);
         else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
 #pragma unroll
         for (int q = 0; q < NP; ++q) s_wx[wib][lane][q] = wx[q];
@@ -249,7 +283,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2)
         T uc[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) uc[q] = T(0);
-        if (DIFF && on) vld<T, R>(u + (int64_t)base * ld_ + col, uc);
+        if (on) vld<T, R>(u + (int64_t)base * ld_ + col, uc);
 #pragma unroll 1
         for (int xp = 0; xp < XH; ++xp) {
           T d[NL][NX][R];
@@ -257,16 +291,16 @@ __global__ void __launch_bounds__(WARPS * 32, 2)
           for (int ln = 0; ln < NL; ++ln) {
 #pragma unroll
             for (int q = 0; q < NX; ++q) {
-              const int32_t idx = s_idx[wib][ln * NP + xp * NX + q];
-              if (on) {
-                vld<T, R>(u + (int64_t)idx * ld_ + col, d[ln][q]);
-                if (DIFF) sub_v<T, R>(d[ln][q], uc);
-              } else {
+              const int32_t idx = s_idx[wib][((ln / NP) * 4 + ln % NP) * 4 + xp * NX + q];
 #pragma unroll
-                for (int r = 0; r < R; ++r) d[ln][q][r] = T(0);
-              }
+              for (int r = 0; r < R; ++r) d[ln][q][r] = T(0);
+              if (on) vld<T, R>(u + (int64_t)idx * ld_ + col, d[ln][q]);
             }
           }
+#pragma unroll
+          for (int ln = 0; ln < NL; ++ln)
+#pragma unroll
+            for (int q = 0; q < NX; ++q) sub_v<T, R>(d[ln][q], uc);
 #pragma unroll 1
           for (int j = 0; j < k; ++j) {
             T P[NX][R];
@@ -299,16 +333,128 @@ __global__ void __launch_bounds__(WARPS * 32, 2)
               s_acc[(XH > 1) ? wib : 0][j][lane] = pv;
             } else if (on) {
               const int64_t row = s_row[wib][j];
-              if (DIFF) {
-                T ui[R];
-                vld<T, R>(u + row * ld_ + col, ui);
+              T ui[R];
+              vld<T, R>(u + row * ld_ + col, ui);
 #pragma unroll
-                for (int r = 0; r < R; ++r) part[r] += uc[r] - ui[r];
-              }
-#pragma unroll
-              for (int r = 0; r < R; ++r) part[r] *= cs;
+              for (int r = 0; r < R; ++r) part[r] = cs * (part[r] + (uc[r] - ui[r]));
               vst<T, R>(a + row * ld_ + col, part);
             }
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// FP64, one column per lane: the sums of fixed.cuh, with an exponent per column
+// and cell.  The lane holds its column's 64 node differences as integer halves
+// (128 registers) and takes the weights of each row from shared memory, where one
+// lane per row formed them.  On the torus at h = 1/64, 64 columns (34M row columns):
+// the FP64 pipe needed 5.8 ms for this.
+template <bool DIFF, int DIM, int NP>
+__global__ void __launch_bounds__(WARPS * 16, 2)
+    gather_cells_fx_kernel(CellArgs A, const double *__restrict__ tc, double cs, const double *__restrict__ u,
+                           double *__restrict__ a, int nrhs, int64_t ld) {
+  constexpr int NZ = (DIM == 3) ? NP : 1;
+  constexpr int NL = NP * NZ;
+  constexpr int W = WARPS / 2;
+  __shared__ __align__(16) int2 s_w[W][CHUNK][3][4];
+  __shared__ int32_t s_row[W][CHUNK];
+  __shared__ __align__(16) int32_t s_idx[W][16 * 4];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  if (warp >= A.ncells) return;
+  CellHead h = cell_head<NP>(A, warp, lane);
+  for (int64_t cid = warp; cid < A.ncells; cid += nwarps) {
+    const int split = h.split;
+    if (lane < 16) {
+      int4 o;
+      o.x = h.line.x;
+      o.y = (1 < split) ? h.line.x + 1 : h.line.y + (1 - split);
+      o.z = (2 < split) ? h.line.x + 2 : h.line.y + (2 - split);
+      o.w = (3 < split) ? h.line.x + 3 : h.line.y + (3 - split);
+      *reinterpret_cast<int4 *>(&s_idx[wib][lane * 4]) = o;
+    }
+    const int32_t r0 = h.r0, r1 = h.r1;
+    if (cid + nwarps < A.ncells) h = cell_head<NP>(A, cid + nwarps, lane);
+    __syncwarp();
+    for (int32_t c0 = r0; c0 < r1; c0 += CHUNK) {
+      const int k = min(CHUNK, r1 - c0);
+      if (lane < 3 * k) {  // lane j + k axis forms the weights of one axis of row j
+        const int ax = lane / k, j = lane - ax * k;
+        int32_t wh[4] = {0, 0, 0, 0}, wl[4] = {0, 0, 0, 0};
+        if (ax < DIM) fixed_weights<NP>(__ldg(tc + 3 * (int64_t)(c0 + j) + ax), wh, wl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s_w[wib][j][ax][q] = make_int2(wh[q], wl[q]);
+      }
+      if (lane < k) s_row[wib][lane] = __ldg(A.crows + c0 + lane);
+      __syncwarp();
+      for (int col = lane; col - lane < nrhs; col += 32) {
+        const bool on = col < nrhs;
+        double d[NL][NP];
+#pragma unroll
+        for (int ln = 0; ln < NL; ++ln)
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            const int32_t idx = s_idx[wib][((ln / NP) * 4 + ln % NP) * 4 + q];
+            d[ln][q] = on ? __ldg(u + (int64_t)idx * ld + col) : 0.0;
+          }
+        const double uc = d[0][0];
+        unsigned top = 0;
+#pragma unroll
+        for (int ln = 0; ln < NL; ++ln)
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            d[ln][q] -= uc;
+            top = max(top, fx_key(d[ln][q]));
+          }
+        const double sc = fx_cell_scale<DIM>(top);
+        int32_t dh[NL][NP], dl[NL][NP];
+#pragma unroll
+        for (int ln = 0; ln < NL; ++ln)
+#pragma unroll
+          for (int q = 0; q < NP; ++q) halves(fx_of(d[ln][q], (int)(top >> 20), 8), dh[ln][q], dl[ln][q]);
+#pragma unroll 1
+        for (int j = 0; j < k; ++j) {
+          const int4 *wp = reinterpret_cast<const int4 *>(&s_w[wib][j][0][0]);
+          const int4 x0 = wp[0], x1 = wp[1];
+          long long zh = 0, zr = 0;
+#pragma unroll
+          for (int cz = 0; cz < NZ; ++cz) {
+            long long yh = 0, yr = 0;
+#pragma unroll
+            for (int cy = 0; cy < NP; ++cy) {
+              const int ln = cz * NP + cy;
+              long long xh = 0, xr = 0;
+              mac(xh, xr, x0.x, x0.y, dh[ln][0], dl[ln][0]);
+              mac(xh, xr, x0.z, x0.w, dh[ln][1], dl[ln][1]);
+              mac(xh, xr, x1.x, x1.y, dh[ln][2], dl[ln][2]);
+              if (NP == 4) mac(xh, xr, x1.z, x1.w, dh[ln][NP - 1], dl[ln][NP - 1]);
+              int32_t lh, ll;
+              halves(xh + high_word(xr), lh, ll);
+              const int2 wy = s_w[wib][j][1][cy];
+              mac(yh, yr, wy.x, wy.y, lh, ll);
+            }
+            if constexpr (DIM == 3) {
+              int32_t mh, ml;
+              halves(yh + high_word(yr), mh, ml);
+              const int2 wz = s_w[wib][j][2][cz];
+              mac(zh, zr, wz.x, wz.y, mh, ml);
+            } else {
+              zh = yh;
+              zr = yr;
+            }
+          }
+          if (on) {
+            const int64_t row = s_row[wib][j];
+            const double b = DIFF ? uc - __ldg(u + row * ld + col) : uc;
+            double acc;
+            if (sc > 0.0) acc = fma(sc, (double)(zh + high_word(zr)), b);
+            else acc = slow_row<DIM, NP>(tc + 3 * (int64_t)(c0 + j), A.lines + cid * 16, split, u + col, ld, uc) + b;
+            if (cs != 1.0) acc *= cs;
+            a[row * ld + col] = acc;
           }
         }
       }
@@ -550,86 +696,100 @@ done:
   return rc;
 }
 
-// x passes of the cell gather that keep the node values of one pass in
-// registers: a divisor of NP; FP64 pairs of columns are not held four x wide
-template <typename T, int NP, int R>
-__host__ __device__ constexpr bool xh_ok(int xh) {
-  return (NP % xh == 0) && !(sizeof(T) == 8 && R == 2 && NP / xh > 2) && !(sizeof(T) == 8 && NP / xh > 2);
-}
-
-template <typename T, int DIM, int NP, int R, int XH>
-static void launch_cells_xh(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
-                            cudaStream_t st, unsigned g) {
-  if constexpr (xh_ok<T, NP, R>(XH))
-    gather_cells_kernel<T, true, DIM, NP, XH, R><<<g, WARPS * 32, 0, st>>>(
-        A, c->d_cell_start, c->d_cell_key, c->d_cell_rows, c->ncells, cs, u, a, nrhs, ld);
-}
-
 // the default number of x passes (node values of one pass near 64 registers)
-template <typename T, int NP, int R>
-constexpr int default_xh() {
-  return (NP == 3) ? ((sizeof(T) == 8 && R == 2) ? 3 : 1) : ((sizeof(T) == 8) ? ((R == 2) ? 4 : 2) : 2);
+int cpm_cells_default_xh(int np1, bool fp64, int /*rpl*/) { return (np1 == 3 || fp64) ? 1 : 2; }
+
+static CellArgs cell_args(const cpm_ctx *c) {
+  return CellArgs{c->d_cell_start, c->d_cell_rows, c->d_cell_key, reinterpret_cast<const int2 *>(c->d_cell_lines),
+                  c->ncells};
 }
 
-int cpm_cells_default_xh(int np1, bool fp64, int rpl) {
-  if (np1 == 3) return fp64 ? (rpl == 2 ? default_xh<double, 3, 2>() : default_xh<double, 3, 1>())
-                            : (rpl == 2 ? default_xh<float, 3, 2>() : default_xh<float, 3, 1>());
-  return fp64 ? (rpl == 2 ? default_xh<double, 4, 2>() : default_xh<double, 4, 1>())
-              : (rpl == 2 ? default_xh<float, 4, 2>() : default_xh<float, 4, 1>());
+template <int DIM, int NP, int R, int XH>
+static void launch_cells_xh(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
+                            cudaStream_t st, unsigned g) {
+  if constexpr (NP % XH == 0)
+    gather_cells_kernel<DIM, NP, XH, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, ld);
 }
 
-template <typename T, int DIM, int NP, int R>
-static void launch_cells_k(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
+template <int DIM, int NP, int R>
+static void launch_cells_k(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
                            cudaStream_t st) {
-  int xh = c->tune.cells_xh[sizeof(T) == 8 ? 1 : 0][R - 1];
-  if (xh <= 0 || xh > 4 || !xh_ok<T, NP, R>(xh)) xh = default_xh<T, NP, R>();
+  int xh = c->tune.cells_xh[0][R - 1];
+  if (xh <= 0 || xh > 4 || NP % xh != 0) xh = cpm_cells_default_xh(NP, false, R);
   const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : 16;
   unsigned g = (unsigned)std::min<int64_t>((c->ncells + WARPS - 1) / WARPS, (int64_t)c->nsm * per_sm);
   if (g < 1) g = 1;
   switch (xh) {
-    case 1: launch_cells_xh<T, DIM, NP, R, 1>(c, A, cs, u, a, nrhs, ld, st, g); break;
-    case 2: launch_cells_xh<T, DIM, NP, R, 2>(c, A, cs, u, a, nrhs, ld, st, g); break;
-    case 3: launch_cells_xh<T, DIM, NP, R, 3>(c, A, cs, u, a, nrhs, ld, st, g); break;
-    default: launch_cells_xh<T, DIM, NP, R, 4>(c, A, cs, u, a, nrhs, ld, st, g); break;
+    case 1: launch_cells_xh<DIM, NP, R, 1>(c, cs, u, a, nrhs, ld, st, g); break;
+    case 2: launch_cells_xh<DIM, NP, R, 2>(c, cs, u, a, nrhs, ld, st, g); break;
+    case 3: launch_cells_xh<DIM, NP, R, 3>(c, cs, u, a, nrhs, ld, st, g); break;
+    default: launch_cells_xh<DIM, NP, R, 4>(c, cs, u, a, nrhs, ld, st, g); break;
   }
 }
 
-template <typename T, int NP, int R>
-static void launch_cells_np(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
+template <int R>
+static void launch_cells(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld, cudaStream_t st) {
+  if (c->dim == 3) {
+    if (c->p == 2) launch_cells_k<3, 3, R>(c, cs, u, a, nrhs, ld, st);
+    else launch_cells_k<3, 4, R>(c, cs, u, a, nrhs, ld, st);
+  } else {
+    if (c->p == 2) launch_cells_k<2, 3, R>(c, cs, u, a, nrhs, ld, st);
+    else launch_cells_k<2, 4, R>(c, cs, u, a, nrhs, ld, st);
+  }
+}
+
+template <bool DIFF>
+static void launch_cells_fx(const cpm_ctx *c, double cs, const double *u, double *a, int nrhs, int64_t ld,
                             cudaStream_t st) {
-  if (c->dim == 3) launch_cells_k<T, 3, NP, R>(c, A, cs, u, a, nrhs, ld, st);
-  else launch_cells_k<T, 2, NP, R>(c, A, cs, u, a, nrhs, ld, st);
-}
-
-// the cell gather always takes the difference form (the batched products are
-// only used in it)
-template <typename T, int R>
-static void launch_cells_r(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
-                           cudaStream_t st, bool /*diff*/) {
-  if (c->p == 2) launch_cells_np<T, 3, R>(c, A, cs, u, a, nrhs, ld, st);
-  else launch_cells_np<T, 4, R>(c, A, cs, u, a, nrhs, ld, st);
-  if (c->ncorr > 0) {
-    const T *cw;
-    if constexpr (sizeof(T) == 8) cw = reinterpret_cast<const T *>(c->d_corr_w64);
-    else cw = reinterpret_cast<const T *>(c->d_corr_w32);
-    unsigned gc = (unsigned)std::min<int64_t>((c->ncorr + 7) / 8, (int64_t)c->nsm * 16);
-    correct_kernel<T, R><<<gc, 256, 0, st>>>(c->d_corr_row, c->d_corr_start, c->d_corr_node, c->d_corr_col, cw,
-                                             c->ncorr, cs, u, a, nrhs, ld);
+  const int W = WARPS / 2;
+  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : 16;
+  unsigned g = (unsigned)std::min<int64_t>((c->ncells + W - 1) / W, (int64_t)c->nsm * per_sm);
+  if (g < 1) g = 1;
+  const CellArgs A = cell_args(c);
+#define CPM_FX(D, NP) gather_cells_fx_kernel<DIFF, D, NP><<<g, W * 32, 0, st>>>(A, c->d_tc64, cs, u, a, nrhs, ld)
+  if (c->dim == 3) {
+    if (c->p == 2) CPM_FX(3, 3); else CPM_FX(3, 4);
+  } else {
+    if (c->p == 2) CPM_FX(2, 3); else CPM_FX(2, 4);
   }
+#undef CPM_FX
 }
 
-template <typename T>
-int cpm_launch_gather_cells(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, int nrhs, int64_t ld,
-                            cudaStream_t st, bool diff, int rpl) {
-  if (c->ncells == 0) return 0;
-  if (rpl == 2) launch_cells_r<T, 2>(c, A, cs, u, a, nrhs, ld, st, diff);
-  else launch_cells_r<T, 1>(c, A, cs, u, a, nrhs, ld, st, diff);
-  return (c->ncorr > 0) ? 2 : 1;
+// the flipped entries of a batch
+template <typename T, int R>
+static int launch_correct(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, int64_t ld, cudaStream_t st) {
+  if (c->ncorr == 0) return 0;
+  const T *cw;
+  if constexpr (sizeof(T) == 8) cw = reinterpret_cast<const T *>(c->d_corr_w64);
+  else cw = reinterpret_cast<const T *>(c->d_corr_w32);
+  unsigned gc = (unsigned)std::min<int64_t>((c->ncorr + 7) / 8, (int64_t)c->nsm * 16);
+  correct_kernel<T, R><<<gc, 256, 0, st>>>(c->d_corr_row, c->d_corr_start, c->d_corr_node, c->d_corr_col, cw,
+                                           c->ncorr, cs, u, a, nrhs, ld);
+  return 1;
 }
-template int cpm_launch_gather_cells<float>(const cpm_ctx *, const ApplyArgs<float> &, float, const float *, float *,
-                                            int, int64_t, cudaStream_t, bool, int);
-template int cpm_launch_gather_cells<double>(const cpm_ctx *, const ApplyArgs<double> &, double, const double *,
-                                             double *, int, int64_t, cudaStream_t, bool, int);
+
+// FP32 takes the difference form only (no caller wants E u itself in FP32)
+template <>
+int cpm_launch_gather_cells<float>(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
+                                   cudaStream_t st, bool /*diff*/, int rpl) {
+  if (c->ncells == 0) return 0;
+  if (rpl == 2) {
+    launch_cells<2>(c, cs, u, a, nrhs, ld, st);
+    return 1 + launch_correct<float, 2>(c, cs, u, a, nrhs, ld, st);
+  }
+  launch_cells<1>(c, cs, u, a, nrhs, ld, st);
+  return 1 + launch_correct<float, 1>(c, cs, u, a, nrhs, ld, st);
+}
+
+template <>
+int cpm_launch_gather_cells<double>(const cpm_ctx *c, double cs, const double *u, double *a, int nrhs, int64_t ld,
+                                    cudaStream_t st, bool diff, int rpl) {
+  if (c->ncells == 0) return 0;
+  if (diff) launch_cells_fx<true>(c, cs, u, a, nrhs, ld, st);
+  else launch_cells_fx<false>(c, cs, u, a, nrhs, ld, st);
+  return 1 + (rpl == 2 ? launch_correct<double, 2>(c, cs, u, a, nrhs, ld, st)
+                       : launch_correct<double, 1>(c, cs, u, a, nrhs, ld, st));
+}
 
 template <typename T>
 void cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st) {

@@ -983,11 +983,13 @@ cpm_status fp64_passes(cpm_ctx *c, ApplyFn<double> ap64, bool left, double dS, d
       all = all && d;
       if (!d) fmin = std::min(fmin, floors[q]);
     }
-    // a further pass while the last one still gained 10 %; its recursion need
-    // not go below the rounding floor, where the true residual cannot follow
-    // a breakdown ends the pass, not the solve: the next pass restarts from x
+    // a further pass while the last one still gained 10 %; it aims at half the
+    // tolerance (one that starts just above tol would otherwise stop at once,
+    // gain nothing and end the solve), but need not go below the rounding floor,
+    // where the true residual cannot follow.  A breakdown ends the pass, not the
+    // solve: the next pass restarts from x
     if (all || *iters >= maxit || !(worst < 0.9 * prev_worst)) break;
-    if (std::isfinite(fmin)) cv.tol = std::max(tol, 0.5 * fmin);
+    cv.tol = 0.5 * (std::isfinite(fmin) ? std::max(tol, fmin) : tol);
     prev_worst = worst;
   }
   return CPM_OK;

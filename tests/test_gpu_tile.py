@@ -67,3 +67,33 @@ def test_infinities_and_nan_reach_the_same_rows(oracle_mod):
         assert np.array_equal(np.isfinite(a), np.isfinite(er))
         ok = np.isfinite(er)
         assert np.max(np.abs(a[ok] - er[ok])) <= TOL
+
+
+@pytest.mark.parametrize("name", ["circle_dir2", "sphere_lat_dir2", "torus"])
+@pytest.mark.parametrize("p", [3, 2])
+def test_batches_of_every_width_match_oracle(oracle_mod, name, p):
+    """Column groups that end ragged, odd widths and more than 64 columns; columns
+    of very different size, one of zeros and one holding an infinity."""
+    torch = need_gpu()
+    w = _wl(name)
+    band, ref = pair(oracle_mod, w, p=p)
+    A = ref.A(0.0, 1.0)
+    for nrhs in (16, 31, 33, 34, 65, 66, 130):
+        U = ci.random_vector(ref.N, seed=nrhs, nrhs=nrhs)
+        VR = A @ U
+        U32 = torch.tensor(U, device="cuda").float()
+        V32 = band.apply(0.0, 1.0, U32).cpu().numpy()
+        assert np.max(np.abs(V32 - VR)) <= 2e-6 * np.max(np.abs(VR))
+        scale = np.ones(nrhs)
+        scale[0], scale[1], scale[2] = 2.0 ** -800, 2.0 ** 800, 0.0
+        Ug = torch.tensor(U * scale, device="cuda")
+        Ug[ref.N // 2, 3] = float("inf")
+        V = band.apply(0.0, 1.0, Ug).cpu().numpy()
+        E = band.extend(Ug).cpu().numpy()
+        for r in range(nrhs):
+            if r == 3:
+                assert not np.all(np.isfinite(V[:, r])) and np.any(np.isfinite(V[:, r]))
+                continue
+            assert np.max(np.abs(V[:, r] - VR[:, r] * scale[r])) <= 1e-14 * np.max(np.abs(VR[:, r])) * scale[r]
+            er = ref.extend(U[:, r])[:ref.NS] * scale[r]
+            assert np.max(np.abs(E[:, r] - er)) <= TOL * np.max(np.abs(U[:, r])) * scale[r]
