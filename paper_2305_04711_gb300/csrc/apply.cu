@@ -53,7 +53,7 @@ __device__ __forceinline__ void load_nbrs(const int32_t *nbr8, int64_t i, int32_
 
 // one row, one column: u0 = u_i; uk, ak the values at the neighbours nb (anything
 // where nb < 0, ak anything where the neighbour is a BC DOF)
-__device__ __forceinline__ float combine_row(const CombineScale<float> &S, int64_t NS, int nfd, const int32_t (&nb)[6],
+__device__ __forceinline__ float combine_row(const CombineScale<float> &S, int NS, int nfd, const int32_t (&nb)[6],
                                              float u0, const float (&uk)[6], const float (&ak)[6]) {
   const float ui = S.cs * u0;
   float s = 0.0f;
@@ -67,7 +67,7 @@ __device__ __forceinline__ float combine_row(const CombineScale<float> &S, int64
   return S.m * u0 + S.c * (s - (float)(nfd - present) * ui);
 }
 
-__device__ __forceinline__ double combine_row_plain(const CombineScale<double> &S, int64_t NS, int nfd,
+__device__ __forceinline__ double combine_row_plain(const CombineScale<double> &S, int NS, int nfd,
                                                  const int32_t (&nb)[6], double u0, const double (&uk)[6],
                                                  const double (&ak)[6]) {
   const double ui = S.cs * u0;
@@ -82,7 +82,7 @@ __device__ __forceinline__ double combine_row_plain(const CombineScale<double> &
   return S.m * u0 + S.c * (s - (nfd - present) * ui);
 }
 
-__device__ __forceinline__ double combine_row(const CombineScale<double> &S, int64_t NS, int nfd,
+__device__ __forceinline__ double combine_row(const CombineScale<double> &S, int NS, int nfd,
                                               const int32_t (&nb)[6], double u0, const double (&uk)[6],
                                               const double (&ak)[6]) {
   unsigned tu = fx_key(u0), ta = 0;
@@ -124,7 +124,7 @@ __device__ __forceinline__ double combine_row(const CombineScale<double> &S, int
 
 // a few columns: one thread per element
 template <typename T>
-__global__ void __launch_bounds__(256) combine_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val,
+__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 6 : 8) combine_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val,
                                                       const T *__restrict__ u, const T *__restrict__ a,
                                                       T *__restrict__ v, int nrhs, int64_t ld) {
   CPM_ROWS_COLS_LOOP(A.N, nrhs, i, r) {
@@ -134,11 +134,12 @@ __global__ void __launch_bounds__(256) combine_kernel(CombineArgs A, CombineScal
       T uk[6], ak[6];
       const T u0 = __ldg(u + i * ld + r);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        uk[k] = (nb[k] >= 0) ? __ldg(u + (int64_t)nb[k] * ld + r) : T(0);
-        ak[k] = (nb[k] >= 0 && nb[k] < A.NS) ? __ldg(a + (int64_t)nb[k] * ld + r) : T(0);
+      for (int k = 0; k < 6; ++k) {  // absent ones read the row's own: all 13 loads start at once
+        const int64_t c = (nb[k] >= 0) ? nb[k] : i, ca = (c < A.NS) ? c : i;
+        uk[k] = __ldg(u + c * ld + r);
+        ak[k] = __ldg(a + ca * ld + r);
       }
-      v[i * ld + r] = combine_row(S, A.NS, A.nfd, nb, u0, uk, ak);
+      v[i * ld + r] = combine_row(S, (int)A.NS, A.nfd, nb, u0, uk, ak);
     } else {
       const int64_t al = i - A.NS;
       const int cnt = __ldg(A.bc_cnt + al);
@@ -186,50 +187,51 @@ __device__ __forceinline__ void stv(T *p, const T in[RPL]) {
 // A block takes `chunk` consecutive rows, its 8 warps 8 of them at a time, so
 // that the y neighbours (8 rows away inside a brick) are still in L1.
 template <typename T, int RPL>
-__global__ void __launch_bounds__(256) combine_batched_kernel(CombineArgs A, CombineScale<T> S,
+__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 3 : 4) combine_batched_kernel(CombineArgs A, CombineScale<T> S,
                                                               const T *__restrict__ bc_val, const T *__restrict__ u,
                                                               const T *__restrict__ a, T *__restrict__ v, int nrhs,
-                                                              int64_t ld, int chunk) {
+                                                              unsigned ld, int chunk) {
+  // (a 32-bit stride: one widening multiply-add per neighbour's address)
   const int lane = threadIdx.x & 31;
-  for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < A.N; c0 += (int64_t)gridDim.x * chunk) {
-    const int64_t c1 = (c0 + chunk < A.N) ? c0 + chunk : A.N;
-    for (int64_t i = c0 + (threadIdx.x >> 5); i < c1; i += 8) {
+  const int NS = (int)A.NS, N = (int)A.N;
+  for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < N; c0 += (int64_t)gridDim.x * chunk) {
+    const int c1 = (int)((c0 + chunk < N) ? c0 + chunk : N);
+    for (int i = (int)c0 + (int)(threadIdx.x >> 5); i < c1; i += 8) {
       int32_t nb[6];
-      if (i < A.NS) load_nbrs(A.nbr8, i, nb);
+      if (i < NS) load_nbrs(A.nbr8, i, nb);
       for (int col = lane * RPL; col < nrhs; col += 32 * RPL) {
         T out[RPL];
-        if (i < A.NS) {
+        if (i < NS) {
           T u0[RPL], uk[6][RPL], ak[6][RPL];
-          ldv<T, RPL>(u + i * ld + col, u0);
+          ldv<T, RPL>(u + (uint64_t)(unsigned)i * ld + col, u0);
 #pragma unroll
-          for (int q = 0; q < 6; ++q) {
-#pragma unroll
-            for (int k = 0; k < RPL; ++k) uk[q][k] = ak[q][k] = T(0);
-            if (nb[q] >= 0) ldv<T, RPL>(u + (int64_t)nb[q] * ld + col, uk[q]);
-            if (nb[q] >= 0 && nb[q] < A.NS) ldv<T, RPL>(a + (int64_t)nb[q] * ld + col, ak[q]);
+          for (int q = 0; q < 6; ++q) {  // absent ones read the row's own: all 13 loads start at once
+            const int c = (nb[q] >= 0) ? nb[q] : i, ca = (c < NS) ? c : i;
+            ldv<T, RPL>(u + (uint64_t)(unsigned)c * ld + col, uk[q]);
+            ldv<T, RPL>(a + (uint64_t)(unsigned)ca * ld + col, ak[q]);
           }
 #pragma unroll
           for (int k = 0; k < RPL; ++k) {
             T x[6], y[6];
 #pragma unroll
             for (int q = 0; q < 6; ++q) { x[q] = uk[q][k]; y[q] = ak[q][k]; }
-            out[k] = combine_row(S, A.NS, A.nfd, nb, u0[k], x, y);
+            out[k] = combine_row(S, NS, A.nfd, nb, u0[k], x, y);
           }
         } else {
-          const int64_t al = i - A.NS;
+          const int64_t al = i - NS;
           const int cnt = __ldg(A.bc_cnt + al);
 #pragma unroll
           for (int k = 0; k < RPL; ++k) out[k] = T(0);
           for (int e = 0; e < cnt; ++e) {
             const int32_t cc = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
-            const T w = __ldg(bc_val + al * CPM_BC_STRIDE + e) * ((cc < A.NS) ? S.cs : T(1));
+            const T w = __ldg(bc_val + al * CPM_BC_STRIDE + e) * ((cc < NS) ? S.cs : T(1));
             T val[RPL];
-            ldv<T, RPL>(u + (int64_t)cc * ld + col, val);
+            ldv<T, RPL>(u + (uint64_t)(unsigned)cc * ld + col, val);
 #pragma unroll
             for (int k = 0; k < RPL; ++k) out[k] += w * val[k];
           }
         }
-        stv<T, RPL>(v + i * ld + col, out);
+        stv<T, RPL>(v + (uint64_t)(unsigned)i * ld + col, out);
       }
     }
   }
@@ -270,7 +272,7 @@ int launch_batched(const cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T *
   unsigned g = (unsigned)std::min<int64_t>((A.N + chunk - 1) / chunk, warps / 8);
   if (g < 1) g = 1;
   const int launched = 1 + cpm_launch_gather_cells<T>(c, cs, u, a, nrhs, ld, st, true, RPL);
-  combine_batched_kernel<T, RPL><<<g, 256, 0, st>>>(A, S, bv, u, a, v, nrhs, ld, chunk);
+  combine_batched_kernel<T, RPL><<<g, 256, 0, st>>>(A, S, bv, u, a, v, nrhs, (unsigned)ld, chunk);
   return launched;
 }
 

@@ -172,17 +172,17 @@ __device__ __forceinline__ void vst(T *p, const T in[R]) {
 // acc[r] += w d[r] and d[r] -= c[r] over a lane's R columns; two FP32 columns
 // go through one packed instruction (FFMA2 / FADD2 of sm_100+), with the same
 // rounding as the scalar FMA and add
-template <typename T, int R>
-__device__ __forceinline__ void axpy_w(T (&acc)[R], T w, const T (&d)[R]) {
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] += w * d[r];
-}
-template <>
-__device__ __forceinline__ void axpy_w<float, 2>(float (&acc)[2], float w, const float (&d)[2]) {
-  const float2 o = __ffma2_rn(make_float2(w, w), make_float2(d[0], d[1]), make_float2(acc[0], acc[1]));
+__device__ __forceinline__ void axpy_w(float (&acc)[1], float w, const float (&d)[1]) { acc[0] += w * d[0]; }
+__device__ __forceinline__ void axpy_w(float (&acc)[2], float2 w, const float (&d)[2]) {
+  const float2 o = __ffma2_rn(w, make_float2(d[0], d[1]), make_float2(acc[0], acc[1]));
   acc[0] = o.x;
   acc[1] = o.y;
 }
+// a weight as the multiply-add above takes it: for two columns twice, so that it
+// comes out of shared memory as the register pair the packed instruction wants
+template <int R> struct Weight;
+template <> struct Weight<1> { typedef float t; static __device__ __forceinline__ t of(float w) { return w; } };
+template <> struct Weight<2> { typedef float2 t; static __device__ __forceinline__ t of(float w) { return make_float2(w, w); } };
 template <typename T, int R>
 __device__ __forceinline__ void sub_v(T (&d)[R], const T (&c)[R]) {
 #pragma unroll
@@ -229,15 +229,16 @@ __device__ __forceinline__ CellHead cell_head(const CellArgs &A, int64_t cid, in
 template <int DIM, int NP, int XH, int R>
 __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
     gather_cells_kernel(CellArgs A, const float *__restrict__ tc, float cs, const float *__restrict__ u,
-                        float *__restrict__ a, int nrhs, int64_t ld_) {
+                        float *__restrict__ a, int nrhs, unsigned ld_) {
   typedef float T;
   constexpr int NZ = (DIM == 3) ? NP : 1;
   constexpr int NL = NP * NZ;  // stencil lines along x
   constexpr int NX = NP / XH;  // x positions per pass
   static_assert(NX * XH == NP, "passes must split the stencil's x positions");
   typedef typename VecT<T, R>::t V;
-  __shared__ __align__(16) T s_wyz[WARPS][CHUNK][NL];
-  __shared__ __align__(16) T s_wx[WARPS][CHUNK][4];
+  typedef typename Weight<R>::t WT;
+  __shared__ __align__(16) WT s_wyz[WARPS][CHUNK][(NL + 3) / 4 * 4];
+  __shared__ __align__(16) WT s_wx[WARPS][CHUNK][4];
   __shared__ int32_t s_row[WARPS][CHUNK];
   __shared__ __align__(16) int32_t s_idx[WARPS][16 * 4];
   __shared__ V s_acc[(XH > 1) ? WARPS : 1][CHUNK][32];
@@ -272,9 +273,9 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
         if (DIM == 3) cpm_lagrange<NP, T>(__ldg(tq + 2), wz);
         else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
 #pragma unroll
-        for (int q = 0; q < NP; ++q) s_wx[wib][lane][q] = wx[q];
+        for (int q = 0; q < NP; ++q) s_wx[wib][lane][q] = Weight<R>::of(wx[q]);
 #pragma unroll
-        for (int q = 0; q < NL; ++q) s_wyz[wib][lane][q] = wy[q % NP] * wz[q / NP];
+        for (int q = 0; q < NL; ++q) s_wyz[wib][lane][q] = Weight<R>::of(wy[q % NP] * wz[q / NP]);
       }
       __syncwarp();
       for (int grp = 0; grp < ngroups; ++grp) {
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
         T uc[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) uc[q] = T(0);
-        if (on) vld<T, R>(u + (int64_t)base * ld_ + col, uc);
+        vld<T, R>(u + (uint64_t)(unsigned)base * ld_ + (on ? col : 0), uc);
 #pragma unroll 1
         for (int xp = 0; xp < XH; ++xp) {
           T d[NL][NX][R];
@@ -292,9 +293,8 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
 #pragma unroll
             for (int q = 0; q < NX; ++q) {
               const int32_t idx = s_idx[wib][((ln / NP) * 4 + ln % NP) * 4 + xp * NX + q];
-#pragma unroll
-              for (int r = 0; r < R; ++r) d[ln][q][r] = T(0);
-              if (on) vld<T, R>(u + (int64_t)idx * ld_ + col, d[ln][q]);
+              // lanes past the last column read the first ones (and store nothing)
+              vld<T, R>(u + (uint64_t)(unsigned)idx * ld_ + (on ? col : 0), d[ln][q]);
             }
           }
 #pragma unroll
@@ -310,15 +310,15 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
               for (int r = 0; r < R; ++r) P[q][r] = T(0);
 #pragma unroll
             for (int ln = 0; ln < NL; ++ln) {
-              const T w = s_wyz[wib][j][ln];
+              const WT w = s_wyz[wib][j][ln];
 #pragma unroll
-              for (int q = 0; q < NX; ++q) axpy_w<T, R>(P[q], w, d[ln][q]);
+              for (int q = 0; q < NX; ++q) axpy_w(P[q], w, d[ln][q]);
             }
             T part[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) part[r] = T(0);
 #pragma unroll
-            for (int q = 0; q < NX; ++q) axpy_w<T, R>(part, s_wx[wib][j][xp * NX + q], P[q]);
+            for (int q = 0; q < NX; ++q) axpy_w(part, s_wx[wib][j][xp * NX + q], P[q]);
             if (XH > 1 && xp > 0) {
               const V pv = s_acc[(XH > 1) ? wib : 0][j][lane];
               const T *pp = reinterpret_cast<const T *>(&pv);
@@ -332,12 +332,12 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
               for (int r = 0; r < R; ++r) pp[r] = part[r];
               s_acc[(XH > 1) ? wib : 0][j][lane] = pv;
             } else if (on) {
-              const int64_t row = s_row[wib][j];
+              const unsigned row = (unsigned)s_row[wib][j];
               T ui[R];
-              vld<T, R>(u + row * ld_ + col, ui);
+              vld<T, R>(u + (uint64_t)row * ld_ + col, ui);
 #pragma unroll
               for (int r = 0; r < R; ++r) part[r] = cs * (part[r] + (uc[r] - ui[r]));
-              vst<T, R>(a + row * ld_ + col, part);
+              vst<T, R>(a + (uint64_t)row * ld_ + col, part);
             }
           }
         }
@@ -347,115 +347,127 @@ __global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
   }
 }
 
-// FP64, one column per lane: the sums of fixed.cuh, with an exponent per column
-// and cell.  The lane holds its column's 64 node differences as integer halves
-// (128 registers) and takes the weights of each row from shared memory, where one
-// lane per row formed them.  On the torus at h = 1/64, 64 columns (34M row columns):
-// the FP64 pipe needed 5.8 ms for this.
+// FP64: the sums of fixed.cuh, with an exponent per column and cell.  A warp
+// takes 16 columns of a cell: its half-warps load every other node and put the
+// node differences as integer halves into shared memory (8 KB a warp), then take
+// every other row of the cell, so that both read the same shared-memory words in
+// one broadcast.  64 nodes in the registers of a lane (254 of them) left 2 warps
+// per scheduler, too few for the multiply-adds' latency: 3.6 ms on the torus at
+// h = 1/64 with 64 columns (34M row columns), 5.8 ms in FP64 arithmetic.
+constexpr int FXC = 16;  // columns per warp
+constexpr int FXW = 4;   // warps per block
+
 template <bool DIFF, int DIM, int NP>
-__global__ void __launch_bounds__(WARPS * 16, 2)
+__global__ void __launch_bounds__(FXW * 32, 5)
     gather_cells_fx_kernel(CellArgs A, const double *__restrict__ tc, double cs, const double *__restrict__ u,
-                           double *__restrict__ a, int nrhs, int64_t ld) {
+                           double *__restrict__ a, int nrhs, unsigned ld) {
   constexpr int NZ = (DIM == 3) ? NP : 1;
-  constexpr int NL = NP * NZ;
-  constexpr int W = WARPS / 2;
-  __shared__ __align__(16) int2 s_w[W][CHUNK][3][4];
-  __shared__ int32_t s_row[W][CHUNK];
-  __shared__ __align__(16) int32_t s_idx[W][16 * 4];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  constexpr int SLOTS = 16 * NZ;  // node x of line cz * 4 + cy at (cz * 4 + cy) * 4 + x
+  __shared__ __align__(16) int2 s_d[FXW][SLOTS][FXC];
+  __shared__ __align__(16) int2 s_w[FXW][CHUNK][3][4];
+  __shared__ int32_t s_row[FXW][CHUNK];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, half = lane >> 4, lc = lane & 15;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  if (warp >= A.ncells) return;
-  CellHead h = cell_head<NP>(A, warp, lane);
-  for (int64_t cid = warp; cid < A.ncells; cid += nwarps) {
-    const int split = h.split;
-    if (lane < 16) {
-      int4 o;
-      o.x = h.line.x;
-      o.y = (1 < split) ? h.line.x + 1 : h.line.y + (1 - split);
-      o.z = (2 < split) ? h.line.x + 2 : h.line.y + (2 - split);
-      o.w = (3 < split) ? h.line.x + 3 : h.line.y + (3 - split);
-      *reinterpret_cast<int4 *>(&s_idx[wib][lane * 4]) = o;
+  const int ngroups = (nrhs + FXC - 1) / FXC;
+  const int64_t items = A.ncells * ngroups;  // groups of a cell go to neighbouring warps
+  for (int64_t it = warp; it < items; it += nwarps) {
+    const int64_t cid = (ngroups == 1) ? it : it / ngroups;
+    const int col = (int)(it - cid * ngroups) * FXC + lc;
+    const bool on = col < nrhs;
+    const CellHead h = cell_head<NP>(A, cid, lane);
+    const int k0 = min(CHUNK, h.r1 - h.r0);
+    // weights of the first rows while the node values are on their way
+    const int ax0 = lane >> 3, j0 = lane & 7;
+    double t0 = 1.0;
+    if (ax0 < DIM && j0 < k0) t0 = __ldg(tc + 3 * (int64_t)(h.r0 + j0) + ax0);
+    const double *uc_ = u + (on ? col : 0);
+    double d[SLOTS / 2];
+#pragma unroll
+    for (int s = 0; s < SLOTS / 2; ++s) {
+      // half-warp 0 takes x = 0, 2, half-warp 1 x = 1, 3 of each line
+      const int ln = s >> 1, x = (s & 1) * 2 + half;
+      d[s] = 0.0;
+      if ((ln & 3) >= NP) continue;
+      const int2 se = make_int2(__shfl_sync(0xffffffffu, h.line.x, ln), __shfl_sync(0xffffffffu, h.line.y, ln));
+      const int32_t idx = (x < h.split) ? se.x + x : se.y + (x - h.split);
+      if (x < NP) d[s] = __ldg(uc_ + (uint64_t)(unsigned)idx * ld);
     }
-    const int32_t r0 = h.r0, r1 = h.r1;
-    if (cid + nwarps < A.ncells) h = cell_head<NP>(A, cid + nwarps, lane);
-    __syncwarp();
-    for (int32_t c0 = r0; c0 < r1; c0 += CHUNK) {
-      const int k = min(CHUNK, r1 - c0);
-      if (lane < 3 * k) {  // lane j + k axis forms the weights of one axis of row j
-        const int ax = lane / k, j = lane - ax * k;
+    const double uc = __shfl_sync(0xffffffffu, d[0], lc);
+    unsigned top = 0;
+#pragma unroll
+    for (int s = 0; s < SLOTS / 2; ++s) {
+      const int ln = s >> 1, x = (s & 1) * 2 + half;
+      if ((ln & 3) >= NP) continue;
+      d[s] = (x < NP) ? d[s] - uc : 0.0;
+      top = max(top, fx_key(d[s]));
+    }
+    top = max(top, __shfl_xor_sync(0xffffffffu, top, 16));
+    const double sc = fx_cell_scale<DIM>(top);
+#pragma unroll
+    for (int s = 0; s < SLOTS / 2; ++s) {
+      const int ln = s >> 1, x = (s & 1) * 2 + half;
+      if ((ln & 3) >= NP) continue;
+      int2 o;
+      halves(fx_of(d[s], (int)(top >> 20), 8), o.x, o.y);
+      s_d[w][ln * 4 + x][lc] = o;
+    }
+    for (int32_t c0 = h.r0; c0 < h.r1; c0 += CHUNK) {
+      const int k = min(CHUNK, h.r1 - c0);
+      if (ax0 < 3) {  // lane 8 axis + j forms the weights of one axis of row j
+        if (c0 != h.r0 && ax0 < DIM && j0 < k) t0 = __ldg(tc + 3 * (int64_t)(c0 + j0) + ax0);
         int32_t wh[4] = {0, 0, 0, 0}, wl[4] = {0, 0, 0, 0};
-        if (ax < DIM) fixed_weights<NP>(__ldg(tc + 3 * (int64_t)(c0 + j) + ax), wh, wl);
+        if (ax0 < DIM) fixed_weights<NP>(t0, wh, wl);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s_w[wib][j][ax][q] = make_int2(wh[q], wl[q]);
+        for (int q = 0; q < 4; ++q) s_w[w][j0][ax0][q] = make_int2(wh[q], wl[q]);
       }
-      if (lane < k) s_row[wib][lane] = __ldg(A.crows + c0 + lane);
+      if (lane < k) s_row[w][lane] = __ldg(A.crows + c0 + lane);
       __syncwarp();
-      for (int col = lane; col - lane < nrhs; col += 32) {
-        const bool on = col < nrhs;
-        double d[NL][NP];
-#pragma unroll
-        for (int ln = 0; ln < NL; ++ln)
-#pragma unroll
-          for (int q = 0; q < NP; ++q) {
-            const int32_t idx = s_idx[wib][((ln / NP) * 4 + ln % NP) * 4 + q];
-            d[ln][q] = on ? __ldg(u + (int64_t)idx * ld + col) : 0.0;
-          }
-        const double uc = d[0][0];
-        unsigned top = 0;
-#pragma unroll
-        for (int ln = 0; ln < NL; ++ln)
-#pragma unroll
-          for (int q = 0; q < NP; ++q) {
-            d[ln][q] -= uc;
-            top = max(top, fx_key(d[ln][q]));
-          }
-        const double sc = fx_cell_scale<DIM>(top);
-        int32_t dh[NL][NP], dl[NL][NP];
-#pragma unroll
-        for (int ln = 0; ln < NL; ++ln)
-#pragma unroll
-          for (int q = 0; q < NP; ++q) halves(fx_of(d[ln][q], (int)(top >> 20), 8), dh[ln][q], dl[ln][q]);
 #pragma unroll 1
-        for (int j = 0; j < k; ++j) {
-          const int4 *wp = reinterpret_cast<const int4 *>(&s_w[wib][j][0][0]);
-          const int4 x0 = wp[0], x1 = wp[1];
-          long long zh = 0, zr = 0;
+      for (int j = half; j < k; j += 2) {
+        const int4 *wp = reinterpret_cast<const int4 *>(&s_w[w][j][0][0]);
+        const int4 x0 = wp[0], x1 = wp[1], y0 = wp[2], y1 = wp[3];
+        const int32_t yh_[4] = {y0.x, y0.z, y1.x, y1.z}, yl_[4] = {y0.y, y0.w, y1.y, y1.w};
+        const int2(*dn)[FXC] = &s_d[w][0];
+        const unsigned row = (unsigned)s_row[w][j];
+        const double ui = (DIFF && on) ? __ldg(uc_ + (uint64_t)row * ld) : 0.0;
+        long long zh = 0, zr = 0;
 #pragma unroll
-          for (int cz = 0; cz < NZ; ++cz) {
-            long long yh = 0, yr = 0;
+        for (int cz = 0; cz < NZ; ++cz) {
+          long long yh = 0, yr = 0;
 #pragma unroll
-            for (int cy = 0; cy < NP; ++cy) {
-              const int ln = cz * NP + cy;
-              long long xh = 0, xr = 0;
-              mac(xh, xr, x0.x, x0.y, dh[ln][0], dl[ln][0]);
-              mac(xh, xr, x0.z, x0.w, dh[ln][1], dl[ln][1]);
-              mac(xh, xr, x1.x, x1.y, dh[ln][2], dl[ln][2]);
-              if (NP == 4) mac(xh, xr, x1.z, x1.w, dh[ln][NP - 1], dl[ln][NP - 1]);
-              int32_t lh, ll;
-              halves(xh + high_word(xr), lh, ll);
-              const int2 wy = s_w[wib][j][1][cy];
-              mac(yh, yr, wy.x, wy.y, lh, ll);
+          for (int cy = 0; cy < NP; ++cy) {
+            const int b = (cz * 4 + cy) * 4;
+            long long xh = 0, xr = 0;
+            const int2 n0 = dn[b][lc], n1 = dn[b + 1][lc], n2 = dn[b + 2][lc];
+            mac(xh, xr, x0.x, x0.y, n0.x, n0.y);
+            mac(xh, xr, x0.z, x0.w, n1.x, n1.y);
+            mac(xh, xr, x1.x, x1.y, n2.x, n2.y);
+            if (NP == 4) {
+              const int2 n3 = dn[b + 3][lc];
+              mac(xh, xr, x1.z, x1.w, n3.x, n3.y);
             }
-            if constexpr (DIM == 3) {
-              int32_t mh, ml;
-              halves(yh + high_word(yr), mh, ml);
-              const int2 wz = s_w[wib][j][2][cz];
-              mac(zh, zr, wz.x, wz.y, mh, ml);
-            } else {
-              zh = yh;
-              zr = yr;
-            }
+            int32_t lh, ll;
+            halves(xh + high_word(xr), lh, ll);
+            mac(yh, yr, yh_[cy], yl_[cy], lh, ll);
           }
-          if (on) {
-            const int64_t row = s_row[wib][j];
-            const double b = DIFF ? uc - __ldg(u + row * ld + col) : uc;
-            double acc;
-            if (sc > 0.0) acc = fma(sc, (double)(zh + high_word(zr)), b);
-            else acc = slow_row<DIM, NP>(tc + 3 * (int64_t)(c0 + j), A.lines + cid * 16, split, u + col, ld, uc) + b;
-            if (cs != 1.0) acc *= cs;
-            a[row * ld + col] = acc;
+          if constexpr (DIM == 3) {
+            int32_t mh, ml;
+            halves(yh + high_word(yr), mh, ml);
+            const int2 wz = s_w[w][j][2][cz];
+            mac(zh, zr, wz.x, wz.y, mh, ml);
+          } else {
+            zh = yh;
+            zr = yr;
           }
+        }
+        if (on) {
+          const double b = DIFF ? uc - ui : uc;
+          double acc;
+          if (sc > 0.0) acc = fma(sc, (double)(zh + high_word(zr)), b);
+          else acc = slow_row<DIM, NP>(tc + 3 * (int64_t)(c0 + j), A.lines + cid * 16, h.split, uc_, ld, uc) + b;
+          if (cs != 1.0) acc *= cs;
+          a[(uint64_t)row * ld + col] = acc;
         }
       }
       __syncwarp();
@@ -708,7 +720,7 @@ template <int DIM, int NP, int R, int XH>
 static void launch_cells_xh(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
                             cudaStream_t st, unsigned g) {
   if constexpr (NP % XH == 0)
-    gather_cells_kernel<DIM, NP, XH, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, ld);
+    gather_cells_kernel<DIM, NP, XH, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, (unsigned)ld);
 }
 
 template <int DIM, int NP, int R>
@@ -741,12 +753,11 @@ static void launch_cells(const cpm_ctx *c, float cs, const float *u, float *a, i
 template <bool DIFF>
 static void launch_cells_fx(const cpm_ctx *c, double cs, const double *u, double *a, int nrhs, int64_t ld,
                             cudaStream_t st) {
-  const int W = WARPS / 2;
-  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : 16;
-  unsigned g = (unsigned)std::min<int64_t>((c->ncells + W - 1) / W, (int64_t)c->nsm * per_sm);
-  if (g < 1) g = 1;
+  const int64_t items = c->ncells * ((nrhs + FXC - 1) / FXC);
+  const unsigned g = (unsigned)std::min<int64_t>((items + FXW - 1) / FXW, (int64_t)c->nsm * 64);
   const CellArgs A = cell_args(c);
-#define CPM_FX(D, NP) gather_cells_fx_kernel<DIFF, D, NP><<<g, W * 32, 0, st>>>(A, c->d_tc64, cs, u, a, nrhs, ld)
+#define CPM_FX(D, NP) \
+  gather_cells_fx_kernel<DIFF, D, NP><<<g, FXW * 32, 0, st>>>(A, c->d_tc64, cs, u, a, nrhs, (unsigned)ld)
   if (c->dim == 3) {
     if (c->p == 2) CPM_FX(3, 3); else CPM_FX(3, 4);
   } else {

@@ -5,8 +5,7 @@
 // integer multiply-adds.  The weighted sum therefore runs in integers that are
 // wider than a double's 53 bits:
 //  * the differences of a cell's node values to its base node's, exact or rounded
-//    once as doubles, become
-//    integers X of 61 bits relative to the largest of the cell;
+//    once as doubles, become integers X of 61 bits relative to the cell's largest;
 //  * the Lagrange weights are formed as integers W = 6 w 2^60 (times 6, so that
 //    no division rounds) from the fractional position t, of which every bit is
 //    kept;
@@ -27,6 +26,8 @@
 #pragma once
 
 #include <stdint.h>
+
+namespace {  // (internal linkage: the plain path's call then leaves the callers' registers alone)
 
 // signed halves of x = xh 2^32 + xl
 __device__ __forceinline__ void halves(long long x, int32_t &xh, int32_t &xl) {
@@ -147,3 +148,4 @@ __device__ __noinline__ double slow_row(const double *t, const int2 *ln, int spl
   return acc;
 }
 
+}  // namespace

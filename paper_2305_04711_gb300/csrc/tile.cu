@@ -88,11 +88,12 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
 #pragma unroll
       for (int k = 0; k < PER; ++k) d[k] = on[k] ? v[k] - uc : T(0);
       if constexpr (FX) {
-        // exponent of the cell's largest difference
+        // exponent of the cell's largest difference (fx_key, fx_of and fx_cell_scale
+        // written out: as calls they cost this unrolled loop 38 of 215 us a product)
         unsigned top = 0;
 #pragma unroll
         for (int k = 0; k < PER; ++k)
-          top = max(top, fx_key(d[k]));
+          top = max(top, ((unsigned)__double2hiint(d[k]) & 0x7FFFFFFFu) | (unsigned)(__double2loint(d[k]) != 0));
         if (CPI > 1) {
 #pragma unroll
           for (int o = SLOTS / 2; o; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
@@ -104,7 +105,12 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
           const int slot = (CPI > 1) ? (lane & (SLOTS - 1)) : lane + 32 * k;
-          const long long X = fx_of(d[k], em, 8);
+          const int hi = __double2hiint(d[k]);
+          const int e = (hi >> 20) & 0x7FF;
+          unsigned long long m = ((unsigned long long)(((unsigned)hi & 0xFFFFFu) | 0x100000u) << 32) |
+                                 (unsigned)__double2loint(d[k]);
+          m = (e == 0) ? 0ull : ((m << 8) >> min(em - e, 63));
+          const long long X = (hi < 0) ? -(long long)m : (long long)m;
           if (SLOTS % 32 == 0 || slot < SLOTS) {
             int2 o;
             halves(X, o.x, o.y);
@@ -112,7 +118,10 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
           }
         }
         if (live && (lane & (SLOTS - 1 < 31 ? SLOTS - 1 : 31)) == 0) {
-          s_sc[w][c] = fx_cell_scale<DIM>(top);
+          constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;
+          const bool plain = em >= 2040 || (em < 83 && top != 0u);
+          const double sc = __hiloint2double(__double2hiint(back) + ((em - 1083) * (1 << 20)), __double2loint(back));
+          s_sc[w][c] = plain ? -1.0 : (top == 0u ? 1.0 : sc);
           s_uc[w][c] = uc;
         }
       } else {
