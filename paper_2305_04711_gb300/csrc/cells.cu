@@ -431,14 +431,14 @@ __global__ void __launch_bounds__(FXW * 32, 5)
         const int2(*dn)[FXC] = &s_d[w][0];
         const unsigned row = (unsigned)s_row[w][j];
         const double ui = (DIFF && on) ? __ldg(uc_ + (uint64_t)row * ld) : 0.0;
-        long long zh = 0, zr = 0;
+        long long zh = 0, zr = HALF;
 #pragma unroll
         for (int cz = 0; cz < NZ; ++cz) {
-          long long yh = 0, yr = 0;
+          long long yh = 0, yr = HALF;
 #pragma unroll
           for (int cy = 0; cy < NP; ++cy) {
             const int b = (cz * 4 + cy) * 4;
-            long long xh = 0, xr = 0;
+            long long xh = 0, xr = HALF;
             const int2 n0 = dn[b][lc], n1 = dn[b + 1][lc], n2 = dn[b + 2][lc];
             mac(xh, xr, x0.x, x0.y, n0.x, n0.y);
             mac(xh, xr, x0.z, x0.w, n1.x, n1.y);
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(FXW * 32, 5)
         if (on) {
           const double b = DIFF ? uc - ui : uc;
           double acc;
-          if (sc > 0.0) acc = fma(sc, (double)(zh + high_word(zr)), b);
+          if (sc > 0.0) acc = scaled_sum(sc, zh + high_word(zr), b);
           else acc = slow_row<DIM, NP>(tc + 3 * (int64_t)(c0 + j), A.lines + cid * 16, h.split, uc_, ld, uc) + b;
           if (cs != 1.0) acc *= cs;
           a[(uint64_t)row * ld + col] = acc;
@@ -497,6 +497,7 @@ __global__ void __launch_bounds__(256) correct_kernel(const int32_t *__restrict_
       T acc[R];
 #pragma unroll
       for (int r = 0; r < R; ++r) acc[r] = T(0);
+#pragma unroll 4
       for (int32_t e = e0; e < e1; ++e) {
         const T w = __ldg(cw + e);
         T ut[R], un[R];

@@ -21,7 +21,7 @@
 // The sum is converted back once, exactly scaled, with one FP64 rounding: its
 // error is a few 2^-56 of the largest difference in the cell, where 84 rounded
 // FP64 operations leave a few 2^-53 of the partial sums.  A cell whose
-// differences are not finite or whose largest one is below 2^-940 goes through
+// differences are not finite or whose largest one is below 2^-883 goes through
 // plain FP64.
 #pragma once
 
@@ -35,6 +35,8 @@ __device__ __forceinline__ void halves(long long x, int32_t &xh, int32_t &xl) {
   xh = (int32_t)((unsigned long long)x >> 32) + (int32_t)((uint32_t)xl >> 31);
 }
 
+// cross sums start at half a unit of the word they lose, so that they round
+constexpr long long HALF = 0x80000000ll;
 __device__ __forceinline__ long long high_word(long long cr) { return (long long)(int32_t)(cr >> 32); }
 
 // a b + c, one instruction
@@ -55,7 +57,7 @@ __device__ __forceinline__ long long mul_high(long long a, long long b) {
   int32_t ah, al, bh, bl;
   halves(a, ah, al);
   halves(b, bh, bl);
-  return mad_wide(ah, bh, high_word(mad_wide(al, bh, mad_wide(ah, bl, 0))));
+  return mad_wide(ah, bh, high_word(mad_wide(al, bh, mad_wide(ah, bl, HALF))));
 }
 
 // 6 2^60 times the Lagrange weights of one axis, in halves.  With tau = t - 1 (exact):
@@ -99,7 +101,7 @@ __device__ __forceinline__ unsigned fx_key(double d) {
 // (finite, and no scale factor leaves the normal range), or is all zero
 __device__ __forceinline__ bool fx_ok(unsigned top) {
   const int em = (int)(top >> 20);
-  return em < 2040 && (em >= 83 || top == 0u);
+  return em < 2040 && (em >= 140 || top == 0u);
 }
 
 // d as an integer in units of 2^(em - 1075 - K), em the largest exponent field of
@@ -119,12 +121,18 @@ __device__ __forceinline__ double fx_scale(double c, int k) {
 }
 
 // what a cell's sum over DIM axes (operands fx_of(d, em, 8)) is multiplied with;
-// negative where the cell needs plain FP64
+// negative where the cell needs plain FP64.  512/27 and 64/9 both lie half a unit
+// above the double next to them, 2^-54 of themselves, which scaled_sum adds.
 template <int DIM>
 __device__ __forceinline__ double fx_cell_scale(unsigned top) {
   constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
   if (!fx_ok(top)) return -1.0;
   return (top == 0u) ? 1.0 : fx_scale(back, (int)(top >> 20) - 1083);
+}
+
+// sc z + b, z with the scale's missing half unit
+__device__ __forceinline__ double scaled_sum(double sc, long long z, double b) {
+  return fma(sc, (double)(z + (z >> 54)), b);
 }
 
 // E u - u_c of one row in plain FP64 (the rare cells outside the integer range)

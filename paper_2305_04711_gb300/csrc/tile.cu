@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
         }
         if (live && (lane & (SLOTS - 1 < 31 ? SLOTS - 1 : 31)) == 0) {
           constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;
-          const bool plain = em >= 2040 || (em < 83 && top != 0u);
+          const bool plain = em >= 2040 || (em < 140 && top != 0u);
           const double sc = __hiloint2double(__double2hiint(back) + ((em - 1083) * (1 << 20)), __double2loint(back));
           s_sc[w][c] = plain ? -1.0 : (top == 0u ? 1.0 : sc);
           s_uc[w][c] = uc;
@@ -148,14 +148,14 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
         fixed_weights<NP>(__ldg(tq + 1), wyh, wyl);
         if (DIM == 3) fixed_weights<NP>(__ldg(tq + 2), wzh, wzl);
         const int4 *dn = reinterpret_cast<const int4 *>(&s_d[w][c][0]);
-        long long zh = 0, zr = 0;
+        long long zh = 0, zr = HALF;
 #pragma unroll
         for (int cz = 0; cz < NZ; ++cz) {
-          long long yh = 0, yr = 0;
+          long long yh = 0, yr = HALF;
 #pragma unroll
           for (int cy = 0; cy < NP; ++cy) {
             const int4 p = dn[(cz * 4 + cy) * 2], s = dn[(cz * 4 + cy) * 2 + 1];
-            long long xh = 0, xr = 0;
+            long long xh = 0, xr = HALF;
             mac(xh, xr, wxh[0], wxl[0], p.x, p.y);
             mac(xh, xr, wxh[1], wxl[1], p.z, p.w);
             mac(xh, xr, wxh[2], wxl[2], s.x, s.y);
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
         const double sc = s_sc[w][c];
         const double base = DIFF ? uc - ui : uc;
         if (sc > 0.0) {
-          acc = fma(sc, (double)(zh + high_word(zr)), base);
+          acc = scaled_sum(sc, zh + high_word(zr), base);
         } else {
           const int64_t cid = c0 + c;
           const int lx = (int)(__ldg(A.ckey + cid) & 7u);
