@@ -122,35 +122,64 @@ __device__ __forceinline__ double combine_row(const CombineScale<double> &S, int
   return combine_row_plain(S, NS, nfd, nb, u0, uk, ak);
 }
 
+template <typename T>
+__device__ __forceinline__ T combine_element(const CombineArgs &A, const CombineScale<T> &S,
+                                             const T *__restrict__ bc_val, const T *__restrict__ u,
+                                             const T *__restrict__ a, int64_t i, int r, int64_t ld) {
+  if (i < A.NS) {
+    int32_t nb[6];
+    load_nbrs(A.nbr8, i, nb);
+    T uk[6], ak[6];
+    const T u0 = __ldg(u + i * ld + r);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {  // absent ones read the row's own: all 13 loads start at once
+      const int64_t c = (nb[k] >= 0) ? nb[k] : i, ca = (c < A.NS) ? c : i;
+      uk[k] = __ldg(u + c * ld + r);
+      ak[k] = __ldg(a + ca * ld + r);
+    }
+    return combine_row(S, (int)A.NS, A.nfd, nb, u0, uk, ak);
+  }
+  const int64_t al = i - A.NS;
+  const int cnt = __ldg(A.bc_cnt + al);
+  T s = T(0);
+  for (int e = 0; e < cnt; ++e) {
+    const int32_t c = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
+    s += __ldg(bc_val + al * CPM_BC_STRIDE + e) * (__ldg(u + (int64_t)c * ld + r) * ((c < A.NS) ? S.cs : T(1)));
+  }
+  return s;
+}
+
 // a few columns: one thread per element
 template <typename T>
-__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 6 : 8) combine_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val,
-                                                      const T *__restrict__ u, const T *__restrict__ a,
-                                                      T *__restrict__ v, int nrhs, int64_t ld) {
-  CPM_ROWS_COLS_LOOP(A.N, nrhs, i, r) {
-    if (i < A.NS) {
-      int32_t nb[6];
-      load_nbrs(A.nbr8, i, nb);
-      T uk[6], ak[6];
-      const T u0 = __ldg(u + i * ld + r);
+__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 6 : 8)
+    combine_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val, const T *__restrict__ u,
+                   const T *__restrict__ a, T *__restrict__ v, int nrhs, int64_t ld) {
+  CPM_ROWS_COLS_LOOP(A.N, nrhs, i, r) v[i * ld + r] = combine_element<T>(A, S, bc_val, u, a, i, r, ld);
+}
+
+// one column with the iteration's dot products of v: (w, v), or (v, u) and (v, v)
+// (STAGE); reading v back for them was a launch and a pass over two vectors
+template <typename T, int STAGE>
+__global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 6 : 8)
+    combine_dot_kernel(CombineArgs A, CombineScale<T> S, const T *__restrict__ bc_val, const T *__restrict__ u,
+                       const T *__restrict__ a, T *__restrict__ v, Red R, Conv cv, const T *__restrict__ w) {
+  constexpr int NQ = (STAGE == ST_OMEGA) ? 2 : 1;
+  double acc[NQ] = {};
+  T run[NQ] = {};
+  int k = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.N; i += (int64_t)gridDim.x * blockDim.x) {
+    const T o = (STAGE == ST_OMEGA) ? u[i] : w[i];
+    const T x = combine_element<T>(A, S, bc_val, u, a, i, 0, 1);
+    v[i] = x;
+    run[0] += x * o;
+    if (NQ > 1) run[NQ - 1] += x * x;
+    if (sizeof(T) == 4 && (++k & 15) == 0)  // FP32 runs of 16, the runs in FP64
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {  // absent ones read the row's own: all 13 loads start at once
-        const int64_t c = (nb[k] >= 0) ? nb[k] : i, ca = (c < A.NS) ? c : i;
-        uk[k] = __ldg(u + c * ld + r);
-        ak[k] = __ldg(a + ca * ld + r);
-      }
-      v[i * ld + r] = combine_row(S, (int)A.NS, A.nfd, nb, u0, uk, ak);
-    } else {
-      const int64_t al = i - A.NS;
-      const int cnt = __ldg(A.bc_cnt + al);
-      T s = T(0);
-      for (int e = 0; e < cnt; ++e) {
-        const int32_t c = __ldg(A.bc_col + al * CPM_BC_STRIDE + e);
-        s += __ldg(bc_val + al * CPM_BC_STRIDE + e) * (__ldg(u + (int64_t)c * ld + r) * ((c < A.NS) ? S.cs : T(1)));
-      }
-      v[i * ld + r] = s;
-    }
+      for (int q = 0; q < NQ; ++q) { acc[q] += (double)run[q]; run[q] = T(0); }
   }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) acc[q] += (double)run[q];
+  if (block_publish<NQ, 256>(acc, R)) finish_reduce<NQ, 256>(STAGE, R, cv);
 }
 
 // ---- batched combine: one warp per row, lanes over right-hand sides ---------
@@ -249,11 +278,21 @@ void combine_args(const cpm_ctx *c, T m, T n, T rowscale, T cs, CombineArgs *A, 
 
 template <typename T>
 void launch_combine(const cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, const T *a, T *v, int nrhs, int64_t ld,
-                    cudaStream_t st) {
+                    cudaStream_t st, FusedDot<T> *dot) {
   CombineArgs A;
   CombineScale<T> S;
   const T *bv;
   combine_args<T>(c, m, n, rowscale, cs, &A, &S, &bv);
+  if (dot && nrhs == 1 && ld == 1) {
+    // (the partials hold 4 blocks per SM)
+    const unsigned g = (unsigned)std::min<int64_t>((A.N + 255) / 256, (int64_t)c->nsm * 4);
+    if (dot->stage == ST_ALPHA)
+      combine_dot_kernel<T, ST_ALPHA><<<g, 256, 0, st>>>(A, S, bv, u, a, v, dot->R, dot->cv, dot->w);
+    else
+      combine_dot_kernel<T, ST_OMEGA><<<g, 256, 0, st>>>(A, S, bv, u, a, v, dot->R, dot->cv, dot->w);
+    dot->done = true;
+    return;
+  }
   combine_kernel<T><<<cpm_grid(A.N * nrhs, 256), 256, 0, st>>>(A, S, bv, u, a, v, nrhs, ld);
 }
 
@@ -395,7 +434,7 @@ template ApplyArgs<float> cpm_apply_args<float>(const cpm_ctx *);
 // returns the number of launches
 template <typename T>
 static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T *a, T *v, int nrhs, int64_t ld,
-                          cudaStream_t st) {
+                          cudaStream_t st, FusedDot<T> *dot) {
   // from 16 columns on a warp holds a cell for a group of columns; two adjacent
   // columns per lane need an even column count and 2-element alignment
   const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
@@ -415,7 +454,7 @@ static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T 
     }
   }
   if (launched == 0) launched = cpm_launch_gather_tile<T>(c, cs, u, a, nrhs, ld, st, true);
-  launch_combine<T>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);
+  launch_combine<T>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st, dot);
   return launched + 1;
 }
 
@@ -426,20 +465,20 @@ static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T 
 // keeps the rounding of smooth fields relative to local differences.
 template <typename T>
 cpm_status cpm_apply_rc_T(cpm_ctx *c, double m, double n, double rowscale, double colscale, const T *u, T *v,
-                          int nrhs, int64_t ld, cudaStream_t st) {
+                          int nrhs, int64_t ld, cudaStream_t st, FusedDot<T> *dot) {
   if (sizeof(T) * (size_t)c->NS * (size_t)ld > c->a_scratch.bytes) return CPM_ERR_CAPACITY;
   T *a = reinterpret_cast<T *>(c->a_scratch.p);
   cpm_prof_begin(c, st);
-  const int launched = launch_product<T>(c, (T)m, (T)n, (T)rowscale, (T)colscale, u, a, v, nrhs, ld, st);
+  const int launched = launch_product<T>(c, (T)m, (T)n, (T)rowscale, (T)colscale, u, a, v, nrhs, ld, st, dot);
   cpm_prof_end(c, st, c->NS * (int64_t)nrhs);
   cpm_count_launches(c, launched);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }
 template cpm_status cpm_apply_rc_T<double>(cpm_ctx *, double, double, double, double, const double *, double *, int,
-                                           int64_t, cudaStream_t);
+                                           int64_t, cudaStream_t, FusedDot<double> *);
 template cpm_status cpm_apply_rc_T<float>(cpm_ctx *, double, double, double, double, const float *, float *, int,
-                                          int64_t, cudaStream_t);
+                                          int64_t, cudaStream_t, FusedDot<float> *);
 
 template <typename T>
 cpm_status cpm_apply_T(cpm_ctx *c, double m, double n, const T *u, T *v, int nrhs, int64_t ld, cudaStream_t st) {
@@ -543,7 +582,8 @@ cpm_status cpm_apply_noalloc_T(cpm_ctx *c, double m, double n, const T *u, T *v,
   cpm_status rc = noalloc_scratch(&p);
   if (rc) return rc;
   // the same kernels as cpm_apply
-  const int launched = launch_product<T>(c, (T)m, (T)n, T(1), T(1), u, reinterpret_cast<T *>(p), v, nrhs, ld, st);
+  const int launched = launch_product<T>(c, (T)m, (T)n, T(1), T(1), u, reinterpret_cast<T *>(p), v, nrhs, ld, st,
+                                         nullptr);
   cpm_count_launches(c, launched);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;

@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "cpm_internal.cuh"
+#include "reduce.cuh"
 
 template <typename T>
 struct ApplyArgs {
@@ -28,10 +29,10 @@ ApplyArgs<T> cpm_apply_args(const cpm_ctx *c);
 // input (diagonal row scaling and right preconditioning without extra vectors)
 template <typename T>
 cpm_status cpm_apply_rc_T(cpm_ctx *c, double m, double n, double rowscale, double colscale, const T *u, T *v,
-                          int nrhs, int64_t ld, cudaStream_t st);
+                          int nrhs, int64_t ld, cudaStream_t st, FusedDot<T> *dot = nullptr);
 template <typename T>
 cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowscale, double colscale, const T *u,
-                                    T *v, int nrhs, int64_t ld, cudaStream_t st);
+                                    T *v, int nrhs, int64_t ld, cudaStream_t st, FusedDot<T> *dot = nullptr);
 // the product with the intermediate in a fixed module array (no allocation)
 template <typename T>
 cpm_status cpm_apply_noalloc_T(cpm_ctx *c, double m, double n, const T *u, T *v, int nrhs, int64_t ld,

@@ -11,13 +11,14 @@
 // D never becomes a vector pass: the operator applies it as a column (right)
 // or row (left) factor of the PDE entries, and the solution update folds it in.
 //
-// One iteration is five vector kernels and two operator products:
+// One iteration is five vector kernels and two operator products (three with one
+// right-hand side, whose forward products take their dot products along):
 //   p  = r + beta (p - omega v)            (shadow restart: rhat = w r, p = r)
 //   v  = A D p;  (rhat, v) -> alpha        (dot kernel, last block finishes)
 //   s  = r - alpha v
 //   t  = A D s;  (t, s), (t, t) -> omega
 //   x += D (alpha p + omega s);  r = s - omega t;
-//        (r, r), (rhat, r), (rhat, rhat), (w r, r) -> convergence, rho, beta
+//        (r, r), (rhat, r), (rhat', r) -> convergence, rho, beta
 // Every dot product is reduced deterministically: a fixed grid of blocks, each
 // reducing its rows in a fixed order (warp shuffles, then shared memory) to a
 // partial per right-hand side, and the last block to arrive (atomic ticket)
@@ -48,194 +49,14 @@
 #include "apply.cuh"
 #include "cpm_internal.cuh"
 #include "krylov.cuh"
+#include "reduce.cuh"
 
 namespace {
 
 constexpr int KT = 512;    // threads per block of the vector kernels
-constexpr int NQMAX = 4;   // dot products reduced by one kernel at most
 // elements per thread in flight in the vector loops (16 bytes of each vector)
 template <typename T>
 constexpr int unroll_of() { return (sizeof(T) == 8) ? 2 : 4; }
-
-// per right-hand side scalar slots
-enum {
-  S_RHO_OLD = 0, S_ALPHA, S_OMEGA, S_RHO, S_BETA, S_ACTIVE, S_RESTART, S_NRESTART, S_FN2, S_RN2, S_BROKE,
-  S_BEST, S_STALL, S_STOPPED, S_RN2_0, S_ITERS, NSC
-};
-
-enum { ST_OUT = 0, ST_INIT, ST_ALPHA, ST_OMEGA, ST_XR };
-
-struct Red {
-  double *part;      // [G][NQMAX][nrhs] block partials
-  unsigned *ticket;  // arrival counter (reset by the last block)
-  double *sc;        // [nrhs][NSC]
-  double *out;       // [NQMAX][nrhs] reduced dot products (ST_OUT / ST_INIT)
-  int nrhs;
-};
-
-struct Conv {
-  double tol;     // relative tolerance on the iterated system's residual
-  double stall;   // iterations without the residual halving before giving up
-  float mix;      // shadow = r o (1 + mix u) (shadow 0; mix 0: the classical rhat = r)
-  int shadow;     // 0: rhat from r as above; 1: rhat = u, independent of r
-  unsigned seed;  // of the hash u
-};
-
-// a fixed hash u(i, c, seed) in [-1, 1]
-__device__ __forceinline__ float hash_unit(int64_t i, int c, unsigned seed) {
-  uint64_t k = (uint64_t)i * 0x9E3779B97F4A7C15ull + (uint64_t)c * 0xD1B54A32D192ED03ull +
-               (uint64_t)seed * 0x94D049BB133111EBull;
-  k ^= k >> 31; k *= 0xBF58476D1CE4E5B9ull; k ^= k >> 29;
-  return (float)((k >> 40) & 0xFFFFFF) * (2.0f / 16777215.0f) - 1.0f;
-}
-
-// The shadow residual rhat of a (re)start, given the residual r there.
-// rhat = r is the classical choice, but when r is supported on few rows (a
-// right-hand side on the BC rows only) A r lives elsewhere and (rhat, A r) = 0:
-// the first step breaks down.  A random rhat (shadow 1) meets every row; its
-// (rhat, r) ~ |rhat| |r| / sqrt(N) is still far above the rounding of the dot
-// products.  `restarts` selects a fresh hash after a near-breakdown.
-__device__ __forceinline__ float shadow_of(const Conv &cv, int64_t i, int c, float r, unsigned restarts) {
-  if (cv.shadow == 1) return hash_unit(i, c, cv.seed + restarts);
-  if (cv.mix == 0.0f) return r;
-  return r * (1.0f + cv.mix * hash_unit(i, c, 0u));
-}
-__device__ __forceinline__ double shadow_of(const Conv &cv, int64_t i, int c, double r, unsigned restarts) {
-  if (cv.shadow == 1) return (double)hash_unit(i, c, cv.seed + restarts);
-  if (cv.mix == 0.0f) return r;
-  return r * (1.0 + (double)cv.mix * (double)hash_unit(i, c, 0u));
-}
-
-// ---- deterministic block reduction -----------------------------------------
-// Thread t of a block owns column c = t % nrhs and rows sub, sub + rows_per,
-// ... of the block's share (sub = t / nrhs, rows_per = KT / nrhs).
-template <int NQ>
-__device__ __forceinline__ bool block_publish(const double (&acc)[NQ], const Red &R) {
-  __shared__ double sh[NQ][KT];
-  __shared__ bool s_last;
-  const int t = threadIdx.x, nrhs = R.nrhs;
-  if (nrhs < 32 && (32 % nrhs) == 0) {
-    // lanes with equal column combine by xor shuffles, then the warps in order
-    double v[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) v[q] = acc[q];
-    for (int off = 16; off >= nrhs; off >>= 1)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    const int lane = t & 31, w = t >> 5;
-    if (lane < nrhs)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) sh[q][w * nrhs + lane] = v[q];
-    __syncthreads();
-    if (t < nrhs)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        double s = 0.0;
-        for (int k = 0; k < KT / 32; ++k) s += sh[q][k * nrhs + t];
-        R.part[((int64_t)blockIdx.x * NQMAX + q) * nrhs + t] = s;
-      }
-  } else {
-    const int rows_per = KT / nrhs;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) sh[q][t] = acc[q];
-    __syncthreads();
-    if (t < nrhs)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        double s = 0.0;
-        for (int k = 0; k < rows_per; ++k) s += sh[q][k * nrhs + t];
-        R.part[((int64_t)blockIdx.x * NQMAX + q) * nrhs + t] = s;
-      }
-  }
-  __threadfence();
-  __syncthreads();
-  if (t == 0) s_last = (atomicAdd(R.ticket, 1u) == gridDim.x - 1);
-  __syncthreads();
-  return s_last;
-}
-
-__device__ void stage_finish(int stage, const Red &R, const Conv &cv, int c, const double *d) {
-  double *s = R.sc + c * NSC;
-  if (stage == ST_OUT) return;
-  if (stage == ST_INIT) {
-    const double fn2 = d[1] > 0.0 ? d[1] : 1.0;
-    s[S_FN2] = fn2;
-    s[S_RN2] = d[0]; s[S_BEST] = d[0]; s[S_RN2_0] = d[0];
-    s[S_RHO] = d[2]; s[S_RHO_OLD] = 1.0; s[S_ALPHA] = 1.0; s[S_OMEGA] = 1.0; s[S_BETA] = 0.0;
-    s[S_RESTART] = 0.0; s[S_NRESTART] = 0.0; s[S_BROKE] = 0.0; s[S_STALL] = 0.0; s[S_STOPPED] = 0.0;
-    s[S_ITERS] = 0.0;
-    const bool fin = isfinite(d[0]);
-    s[S_ACTIVE] = (!fin || sqrt(d[0]) <= cv.tol * sqrt(fn2)) ? 0.0 : 1.0;
-    if (!fin) s[S_STOPPED] = 1.0;
-    return;
-  }
-  if (s[S_ACTIVE] == 0.0) return;
-  if (stage == ST_ALPHA) {
-    if (d[0] == 0.0 || !isfinite(d[0])) { s[S_BROKE] = 1.0; s[S_ACTIVE] = 0.0; return; }
-    s[S_ALPHA] = s[S_RHO] / d[0];
-    return;
-  }
-  if (stage == ST_OMEGA) {
-    const double om = (d[1] > 0.0) ? d[0] / d[1] : 0.0;
-    s[S_OMEGA] = om;
-    if (om == 0.0 || !isfinite(om)) { s[S_BROKE] = 1.0; s[S_ACTIVE] = 0.0; }
-    return;
-  }
-  // ST_XR: residual bookkeeping, then rho and beta of the next iteration
-  s[S_ITERS] += 1.0;
-  const double rn2 = d[0];
-  s[S_RN2] = rn2;
-  if (!isfinite(rn2) || rn2 > 1e16 * s[S_BEST]) { s[S_STOPPED] = 1.0; s[S_ACTIVE] = 0.0; return; }
-  if (sqrt(rn2) <= cv.tol * sqrt(s[S_FN2])) { s[S_ACTIVE] = 0.0; return; }
-  if (rn2 < 0.25 * s[S_BEST]) { s[S_BEST] = rn2; s[S_STALL] = 0.0; }
-  else {
-    s[S_STALL] += 1.0;
-    if (s[S_STALL] > cv.stall) { s[S_STOPPED] = 1.0; s[S_ACTIVE] = 0.0; return; }
-  }
-  double rho = d[1];
-  s[S_RESTART] = 0.0;
-  if (fabs(rho) <= 1e-28 * sqrt(d[2]) * sqrt(rn2) || rho == 0.0) {
-    // restart from a new shadow residual (the one the XR pass dotted with r
-    // as d[3]): p = r, rho = (rhat', r)
-    s[S_RESTART] = 1.0;
-    s[S_NRESTART] += 1.0;
-    if (s[S_NRESTART] > 20.0) { s[S_BROKE] = 1.0; s[S_ACTIVE] = 0.0; return; }
-    rho = d[3];
-    s[S_RHO] = 1.0; s[S_ALPHA] = 1.0; s[S_OMEGA] = 1.0;
-  }
-  s[S_BETA] = (rho / s[S_RHO]) * (s[S_ALPHA] / s[S_OMEGA]);
-  s[S_RHO_OLD] = s[S_RHO];
-  s[S_RHO] = rho;
-}
-
-// the last block: sum the partials in block order (a warp per (q, c), lanes
-// strided over the blocks, then an xor-shuffle tree, identical in every lane)
-template <int NQ>
-__device__ void finish_reduce(int stage, const Red &R, const Conv &cv) {
-  __shared__ double sd[NQMAX][256];
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, nrhs = R.nrhs;
-  const int G = gridDim.x;
-  __threadfence();
-  for (int pr = w; pr < NQ * nrhs; pr += KT / 32) {
-    const int q = pr / nrhs, c = pr - q * nrhs;
-    double s = 0.0;
-    for (int b = lane; b < G; b += 32) s += __ldcg(R.part + ((int64_t)b * NQMAX + q) * nrhs + c);
-#pragma unroll
-    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) sd[q][c] = s;
-  }
-  __syncthreads();
-  if (t < nrhs) {
-    double d[NQMAX] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) d[q] = sd[q][t];
-    if (stage == ST_OUT || stage == ST_INIT)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) R.out[q * nrhs + t] = d[q];
-    stage_finish(stage, R, cv, t, d);
-  }
-  if (t == 0) *R.ticket = 0u;
-}
 
 // grid-stride element loop with UNR elements per thread in flight; the body
 // functor loads into its element state, then updates and accumulates.  Runs
@@ -355,7 +176,7 @@ __global__ void __launch_bounds__(KT, 2) dot_kernel(Red R, Conv cv, int stage, i
   DotBody<T, NQ> body{R.sc, a, b};
   double acc[NQ];
   vloop<T, NQ>(body, N, R.nrhs, ld, acc);
-  if (block_publish<NQ>(acc, R)) finish_reduce<NQ>(stage, R, cv);
+  if (block_publish<NQ, KT>(acc, R)) finish_reduce<NQ, KT>(stage, R, cv);
 }
 
 // x += D (alpha p + omega s);  r = s - omega t;  the XR dot products
@@ -376,16 +197,15 @@ struct XRBody {
   __device__ void load(Elt &e, int64_t, int64_t o) const {
     e.x = x[o]; e.rh = rh[o]; e.p = p[o]; e.s = s[o]; e.t = t[o];
   }
-  __device__ void apply(Elt &e, int64_t i, int64_t o, T (&run)[4]) const {
+  __device__ void apply(Elt &e, int64_t i, int64_t o, T (&run)[3]) const {
     const T d = (i < NS) ? cs : T(1);
     x[o] = e.x + TX(d * (alpha * e.p + omega * e.s));
     const T rn = e.s - omega * e.t;
     r[o] = rn;
     run[0] += rn * rn;
     run[1] += e.rh * rn;
-    run[2] += e.rh * e.rh;
-    // (rhat', r) for the shadow residual a restart would take
-    run[3] += shadow_of(cv, i, c_, rn, nres) * rn;
+    // (rhat', r) for the shadow residual a restart would take, where it is not r
+    if (cv.shadow != 0 || cv.mix != 0.0f) run[2] += shadow_of(cv, i, c_, rn, nres) * rn;
   }
 };
 
@@ -393,13 +213,13 @@ template <typename T, typename TX>
 __global__ void __launch_bounds__(KT, 2) kxr_kernel(Red R, Conv cv, int64_t N, int64_t NS, T cs, int64_t ld, TX *x,
                                                  T *r, const T *rh, const T *p, const T *s, const T *t) {
   XRBody<T, TX> body{R.sc, cv, NS, cs, x, r, rh, p, s, t};
-  double acc[4];
-  vloop<T, 4>(body, N, R.nrhs, ld, acc);
-  if (block_publish<4>(acc, R)) finish_reduce<4>(ST_XR, R, cv);
+  double acc[3];
+  vloop<T, 3>(body, N, R.nrhs, ld, acc);
+  if (block_publish<3, KT>(acc, R)) finish_reduce<3, KT>(ST_XR, R, cv);
 }
 
 // r = f - r (r holds A x, or nothing when x = 0);  rhat = shadow of r;
-// p = v = 0;  (r, r), (f, f), (rhat, r) -> the initial scalars
+// p = v = 0;  (r, r), (f, f), (rhat, r), (rhat, rhat) -> the initial scalars
 template <typename T>
 struct InitBody {
   const T *__restrict__ f; T *__restrict__ r; T *__restrict__ rh; T *__restrict__ p; T *__restrict__ v;
@@ -409,13 +229,14 @@ struct InitBody {
   __device__ bool on(int) const { return true; }
   __device__ void init(int c) const { c_ = c; }
   __device__ void load(Elt &e, int64_t, int64_t o) const { e.f = f[o]; e.r = x_zero ? T(0) : r[o]; }
-  __device__ void apply(Elt &e, int64_t i, int64_t o, T (&run)[3]) const {
+  __device__ void apply(Elt &e, int64_t i, int64_t o, T (&run)[4]) const {
     const T rv = e.f - e.r;
     const T sh = shadow_of(cv, i, c_, rv, 0u);
     r[o] = rv; rh[o] = sh; p[o] = T(0); v[o] = T(0);
     run[0] += rv * rv;
     run[1] += e.f * e.f;
     run[2] += sh * rv;
+    run[3] += sh * sh;
   }
 };
 
@@ -423,9 +244,9 @@ template <typename T>
 __global__ void __launch_bounds__(KT, 2) init_kernel(Red R, Conv cv, int64_t N, int64_t ld, bool x_zero, const T *f,
                                                   T *r, T *rh, T *p, T *v) {
   InitBody<T> body{f, r, rh, p, v, x_zero, cv};
-  double acc[3];
-  vloop<T, 3>(body, N, R.nrhs, ld, acc);
-  if (block_publish<3>(acc, R)) finish_reduce<3>(ST_INIT, R, cv);
+  double acc[4];
+  vloop<T, 4>(body, N, R.nrhs, ld, acc);
+  if (block_publish<4, KT>(acc, R)) finish_reduce<4, KT>(ST_INIT, R, cv);
 }
 
 // ---- FP64 residual -----------------------------------------------------------
@@ -455,7 +276,7 @@ __global__ void __launch_bounds__(KT, 2) resid_kernel(Red R, int64_t N, int64_t 
   double acc[3];
   vloop<double, 3>(body, N, R.nrhs, ld, acc);
   Conv cv{0.0, 0.0, 0.0f, 0, 0u};
-  if (block_publish<3>(acc, R)) finish_reduce<3>(ST_OUT, R, cv);
+  if (block_publish<3, KT>(acc, R)) finish_reduce<3, KT>(ST_OUT, R, cv);
 }
 
 // y = x o xi with xi(i, c) = +-1 from a fixed hash: the model of the rounding
@@ -487,7 +308,7 @@ __global__ void __launch_bounds__(KT, 2) wnorm_kernel(Red R, int64_t N, int64_t 
   double acc[1];
   vloop<double, 1>(body, N, R.nrhs, ld, acc);
   Conv cv{0.0, 0.0, 0.0f, 0, 0u};
-  if (block_publish<1>(acc, R)) finish_reduce<1>(ST_OUT, R, cv);
+  if (block_publish<1, KT>(acc, R)) finish_reduce<1, KT>(ST_OUT, R, cv);
 }
 
 // out = W f (PDE rows scaled by dS)
@@ -619,14 +440,15 @@ namespace {
 // (or R A^T C u)
 template <typename T>
 using ApplyFn = cpm_status (*)(cpm_ctx *, double, double, double, double, const T *, T *, int, int64_t,
-                               cudaStream_t);
+                               cudaStream_t, FusedDot<T> *);
 
 template <typename T>
 struct Op {
   ApplyFn<T> fn;
   double m, n, rowscale, colscale;
-  cpm_status operator()(cpm_ctx *c, const T *u, T *v, int nrhs, int64_t ld, cudaStream_t st, bool plain_cols) const {
-    return fn(c, m, n, rowscale, plain_cols ? 1.0 : colscale, u, v, nrhs, ld, st);
+  cpm_status operator()(cpm_ctx *c, const T *u, T *v, int nrhs, int64_t ld, cudaStream_t st, bool plain_cols,
+                        FusedDot<T> *dot = nullptr) const {
+    return fn(c, m, n, rowscale, plain_cols ? 1.0 : colscale, u, v, nrhs, ld, st, dot);
   }
 };
 
@@ -643,15 +465,16 @@ cpm_status iteration(cpm_ctx *c, const Op<T> &op, TX *x, const Vecs<T> &V, Solve
   const Red R = red_of(w, nrhs);
   const unsigned G = (unsigned)w->G;
   kp_kernel<T><<<G, KT, 0, st>>>(w->sc, cv, N, nrhs, ld, V.r, V.rh, V.p, V.v);
-  cpm_status rc = op(c, V.p, V.v, nrhs, ld, st, false);
+  FusedDot<T> fa{R, cv, ST_ALPHA, V.rh, false}, fo{R, cv, ST_OMEGA, nullptr, false};
+  cpm_status rc = op(c, V.p, V.v, nrhs, ld, st, false, &fa);
   if (rc) return rc;
-  dot_kernel<T, 1><<<G, KT, 0, st>>>(R, cv, ST_ALPHA, N, ld, V.rh, V.v);
+  if (!fa.done) dot_kernel<T, 1><<<G, KT, 0, st>>>(R, cv, ST_ALPHA, N, ld, V.rh, V.v);
   ks_kernel<T><<<G, KT, 0, st>>>(w->sc, N, nrhs, ld, V.r, V.v, V.s);
-  rc = op(c, V.s, V.t, nrhs, ld, st, false);
+  rc = op(c, V.s, V.t, nrhs, ld, st, false, &fo);
   if (rc) return rc;
-  dot_kernel<T, 2><<<G, KT, 0, st>>>(R, cv, ST_OMEGA, N, ld, V.t, V.s);
+  if (!fo.done) dot_kernel<T, 2><<<G, KT, 0, st>>>(R, cv, ST_OMEGA, N, ld, V.t, V.s);
   kxr_kernel<T, TX><<<G, KT, 0, st>>>(R, cv, N, c->NS, T(op.colscale), ld, x, V.r, V.rh, V.p, V.s, V.t);
-  cpm_count_launches(c, 5);
+  cpm_count_launches(c, 5 - (int)fa.done - (int)fo.done);
   return CPM_OK;
 }
 
@@ -771,7 +594,7 @@ cpm_status residual64(cpm_ctx *c, ApplyFn<double> fn, double m, double n, const 
                       std::vector<double> &fn2, cudaStream_t st, double vrow = 1.0,
                       std::vector<double> *rv2 = nullptr) {
   const int64_t N = c->NS + c->NC;
-  cpm_status rc = fn(c, m, n, 1.0, 1.0, x, w->r64, nrhs, ld, st);
+  cpm_status rc = fn(c, m, n, 1.0, 1.0, x, w->r64, nrhs, ld, st, nullptr);
   if (rc) return rc;
   resid_kernel<<<(unsigned)w->G, KT, 0, st>>>(red_of(w, nrhs), N, c->NS, wrow * wrow, vrow * vrow, ld, f, w->r64);
   cpm_count_launches(c, 1);
@@ -802,7 +625,7 @@ cpm_status floor64(cpm_ctx *c, ApplyFn<double> fn, double m, double n, const dou
                    std::vector<double> &floors, cudaStream_t st) {
   const int64_t N = c->NS + c->NC;
   sign_perturb_kernel<<<cpm_grid(N * nrhs, 256), 256, 0, st>>>(N, nrhs, ld, x, y);
-  cpm_status rc = fn(c, m, n, 1.0, 1.0, y, Ay, nrhs, ld, st);
+  cpm_status rc = fn(c, m, n, 1.0, 1.0, y, Ay, nrhs, ld, st, nullptr);
   if (rc) return rc;
   wnorm_kernel<<<(unsigned)w->G, KT, 0, st>>>(red_of(w, nrhs), N, c->NS, wrow * wrow, ld, Ay);
   cpm_count_launches(c, 2);
@@ -1029,7 +852,10 @@ cpm_status solve_impl(cpm_ctx *c, bool adjoint, double m, double n, const double
   // of A^T leaves the BC rows with O(1/h^2) couplings and BiCGSTAB breaks down.
   const bool left = scaled && !adjoint;
   CPM_CUDA_TRY(cudaMemsetAsync(w->ticket, 0, sizeof(unsigned), st));
-  w->G = c->nsm * ((c->tune.vec_blocks_per_sm >= 1 && c->tune.vec_blocks_per_sm <= 4) ? c->tune.vec_blocks_per_sm : 2);
+  // no more blocks than have a row to work on: the last one sums all their partials
+  const int bps = (c->tune.vec_blocks_per_sm >= 1 && c->tune.vec_blocks_per_sm <= 4) ? c->tune.vec_blocks_per_sm : 2;
+  const int64_t rows_per = KT / nrhs > 0 ? KT / nrhs : 1;
+  w->G = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->nsm * bps, (N + rows_per - 1) / rows_per));
   // the initial residual: a right-hand side (or guess) that is not finite is
   // rejected before any iteration
   rc = residual64(c, ap64, m, n, f, x, w, nrhs, ld, wrow, rn2, fn2, st);

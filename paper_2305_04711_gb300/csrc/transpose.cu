@@ -312,7 +312,7 @@ done:
 
 template <typename T>
 cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowscale, double colscale, const T *u,
-                                    T *v, int nrhs, int64_t ld, cudaStream_t st) {
+                                    T *v, int nrhs, int64_t ld, cudaStream_t st, FusedDot<T> * /*dot*/) {
   if (!c->transpose_ready) return CPM_ERR_STATE;
   if (sizeof(T) * (size_t)c->NS * (size_t)ld > c->b_scratch.bytes) return CPM_ERR_CAPACITY;
   TArgs<T> A;
@@ -359,9 +359,9 @@ cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowsc
   return CPM_OK;
 }
 template cpm_status cpm_apply_transpose_rc_T<double>(cpm_ctx *, double, double, double, double, const double *,
-                                                     double *, int, int64_t, cudaStream_t);
+                                                     double *, int, int64_t, cudaStream_t, FusedDot<double> *);
 template cpm_status cpm_apply_transpose_rc_T<float>(cpm_ctx *, double, double, double, double, const float *,
-                                                    float *, int, int64_t, cudaStream_t);
+                                                    float *, int, int64_t, cudaStream_t, FusedDot<float> *);
 
 template <typename T>
 cpm_status cpm_apply_transpose_T(cpm_ctx *c, double m, double n, const T *u, T *v, int nrhs, int64_t ld,
