@@ -188,10 +188,13 @@ struct cpm_ctx {
   bool transpose_ready = false;
   int64_t nT = 0;                   // entries of the per-column remainder lists
   int32_t *d_cellid = nullptr;      // [nb*512] cell index of a packed base location, -1 if none
-  double *d_tblk = nullptr;         // [ncells][64] per-cell blocks of E^T b (one right-hand side; FP32 uses the front half)
+  double *d_tblk = nullptr;         // [ncells][64] per-cell blocks of E^T b (one right-hand side; integers, or FP32 in the
+                                    // front half), then their [ncells] exponents
   double *d_w1d64 = nullptr;        // [NS][12] per-axis Lagrange factors (transposed gather)
   float *d_w1d32 = nullptr;         // [NS][12]
   int32_t *d_T_ptr = nullptr;       // [N+1] CSR over columns
+  int64_t nTcols = 0;
+  int32_t *d_T_cols = nullptr;      // [nTcols] columns with entries, and every BC column
   int32_t *d_T_row = nullptr;       // [nT] source DOF
   int32_t *d_T_kind = nullptr;      // [nT] 0: flipped FD entry, 1: flipped E entry, 2: BC-row entry
   double *d_T_val = nullptr;        // [nT]

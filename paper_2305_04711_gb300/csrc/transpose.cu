@@ -9,15 +9,17 @@
 //   y_j   = d lambda_j + sum_{c, e : col(c,e) = j} w_{c,e} b_c
 //           + s sum_{i : c(i,k) = j >= N_S} lambda_i + sum_{alpha, e : bcol = j} B lambda_alpha.
 // Kernel 1 forms b from the geometric FD neighbours of c, keeping those whose
-// own neighbour slot pointing back at c was not flipped.  Kernel 2 gathers E^T b
-// at each node from the (up to 4^dim) stencil cells whose node set contains it,
-// with every row of those cells (the cell buckets of cells.cu), and adds the
-// sparse remainder -- flipped FD entries, flipped E entries (moved from node j to
+// own neighbour slot pointing back at c was not flipped.  E^T b is gathered at
+// each node from the (up to 4^dim) stencil cells whose node set contains it: for
+// one right-hand side from a block of 64 sums per cell that another kernel forms
+// first, for batches from every row of those cells (the cell buckets of cells.cu).
+// To that comes the sparse remainder -- flipped FD entries, flipped E entries (moved from node j to
 // its twin) and BC-row entries -- from a per-column list built at set-up.
 #include <algorithm>
 
 #include "apply.cuh"
 #include "cpm_internal.cuh"
+#include "fixed.cuh"
 #include "util.cuh"
 
 namespace {
@@ -119,6 +121,16 @@ __global__ void tlist_sort_kernel(const int32_t *ptr, int64_t N, int32_t *t_src,
   }
 }
 
+// columns with remainder entries, and every BC column (which has nothing else)
+__global__ void tcol_flag_kernel(const int32_t *ptr, int64_t NS, int64_t N, int32_t *flag) {
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x)
+    flag[j] = j >= NS || ptr[j + 1] > ptr[j];
+}
+__global__ void tcol_fill_kernel(const int32_t *flag, const int32_t *pos, int64_t N, int32_t *cols) {
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x)
+    if (flag[j]) cols[pos[j]] = (int32_t)j;
+}
+
 template <typename T>
 struct TArgs {
   BandView v;
@@ -132,7 +144,6 @@ struct TArgs {
   const int32_t *T_src;
   const int32_t *T_kind;
   const T *T_val;
-  T *tblk;  // [ncells][64] per-cell blocks (one right-hand side), or nullptr
 };
 
 // b_c = s * sum of lambda over the rows whose unflipped FD slot points at c
@@ -160,49 +171,274 @@ __global__ void __launch_bounds__(256) tb_kernel(TArgs<T> A, T s, const T *__res
   }
 }
 
-// One right-hand side: per stencil cell the block of its E^T b contributions,
-// blk[cz*16 + cy*4 + cx] = sum over the cell's rows of w_x[cx] w_y[cy] w_z[cz] b_row,
-// one thread per cell (the cell's rows share the 4x4x4 node set); the node
-// gather below then reads one value per cell containing the node instead of
-// revisiting every row of it.
-template <typename T, int NP, int NZ>
-__global__ void __launch_bounds__(128) tcell_kernel(TArgs<T> A, int64_t ncells, const T *__restrict__ bv) {
-  for (int64_t cid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; cid < ncells;
-       cid += (int64_t)gridDim.x * blockDim.x) {
-    T blk[NZ][NP][NP];
+// ---- one right-hand side -------------------------------------------------------
+// Per stencil cell the block of its E^T b contributions,
+//   blk[cz*16 + cy*4 + cx] = sum over the cell's rows of w_x[cx] w_y[cy] w_z[cz] b_row,
+// one warp per cell, two nodes per lane.  In FP64 the block is summed in integers
+// (fixed.cuh): b relative to the cell's largest |b|, w_z b and w_y w_z b rounded to
+// 57 bits, the last factor in three multiply-adds; the block is stored as integers
+// below 2^57 of the cell's own exponent, so that the node gather adds them as
+// integers too (up to 64 of them).  One thread per cell with 64 FP64 sums in
+// registers took 872 us on the sphere at h = 1/128, the FP64 node gather 326 us.
+constexpr int TCW = 8;           // warps per block
+constexpr int TCR = 8;           // rows whose weights are staged together
+constexpr int E_NONE = -100000;  // exponent of a block of zeros
+constexpr int E_PLAIN = 100000;  // block of doubles (values outside the integer range)
+
+struct TCellArgs {
+  const int32_t *cstart, *crows;
+  int64_t ncells;
+  const double *tc64;
+  const float *tc32;
+};
+
+template <int DIM, int NP>
+__global__ void __launch_bounds__(TCW * 32)
+    tcell_fx_kernel(TCellArgs A, const double *__restrict__ bv, long long *__restrict__ blk, int32_t *__restrict__ bexp) {
+  constexpr int SLOTS = (DIM == 3) ? 64 : 16;
+  __shared__ __align__(16) int2 s_w[TCW][TCR][3][4];
+  __shared__ int2 s_b[TCW][TCR];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  // the lane's nodes: x = x0, x0 + 1 of line cy, cz
+  const int x0 = (lane & 1) * 2, cy = (lane >> 1) & 3, cz = (DIM == 3) ? lane >> 3 : 0;
+  const bool mine = 2 * lane < SLOTS;
+  const int ax = lane >> 3, j0 = lane & 7;
+  for (int64_t cid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; cid < A.ncells; cid += nwarps) {
+    const int32_t r0 = __ldg(A.cstart + cid), r1 = __ldg(A.cstart + cid + 1);
+    unsigned top = 0;
+    for (int32_t q = r0 + lane; q < r1; q += 32) top = max(top, fx_key(__ldg(bv + __ldg(A.crows + q))));
+    top = __reduce_max_sync(0xffffffffu, top);
+    const int em = (int)(top >> 20);
+    // an axis multiplies by 6 / 16, so a row adds less than 2^56.8 to a sum; more
+    // than 64 rows take fewer bits each
+    const int K = 8 - max(0, 32 - __clz((r1 - r0 - 1) >> 6));
+    // (the exponent limits leave room for the scale factors of the node gather)
+    const bool ok = top == 0u || (em >= 300 && em < 2040 && K >= 0);
+    long long a0 = 0, a1 = 0;
+    if (top != 0u && ok) {
+      for (int32_t c0 = r0; c0 < r1; c0 += TCR) {
+        const int k = min(TCR, r1 - c0);
+        if (ax < 3) {
+          int32_t wh[4] = {0, 0, 0, 0}, wl[4] = {0, 0, 0, 0};
+          if (ax < DIM && j0 < k) fixed_weights<NP>(__ldg(A.tc64 + 3 * (int64_t)(c0 + j0) + ax), wh, wl);
 #pragma unroll
-    for (int cz = 0; cz < NZ; ++cz)
+          for (int q = 0; q < 4; ++q) s_w[w][j0][ax][q] = make_int2(wh[q], (q < NP) ? wl[q] : 0);
+        } else if (j0 < k) {
+          int2 o;
+          halves(fx_of(__ldg(bv + __ldg(A.crows + c0 + j0)), em, K), o.x, o.y);
+          s_b[w][j0] = o;
+        }
+        __syncwarp();
+        for (int j = 0; j < k; ++j) {
+          const int2 b = s_b[w][j], wy = s_w[w][j][1][cy];
+          const int4 wx = *reinterpret_cast<const int4 *>(&s_w[w][j][0][x0]);
+          int32_t qh = b.x, ql = b.y;
+          if (DIM == 3) {
+            const int2 wz = s_w[w][j][2][cz];
+            halves(mad_wide(wz.x, qh, high_word(mad_wide(wz.x, ql, mad_wide(wz.y, qh, HALF)))), qh, ql);
+          }
+          halves(mad_wide(wy.x, qh, high_word(mad_wide(wy.x, ql, mad_wide(wy.y, qh, HALF)))), qh, ql);
+          a0 = mad_wide(wx.x, qh, a0 + high_word(mad_wide(wx.x, ql, mad_wide(wx.y, qh, HALF))));
+          a1 = mad_wide(wx.z, qh, a1 + high_word(mad_wide(wx.z, ql, mad_wide(wx.w, qh, HALF))));
+        }
+        __syncwarp();
+      }
+      // the block's largest sum moved to 57 bits
+      const unsigned long long m0 = (unsigned long long)(a0 < 0 ? -a0 : a0), m1 = (unsigned long long)(a1 < 0 ? -a1 : a1);
+      const int bits = (int)__reduce_max_sync(0xffffffffu, mine ? 64u - (unsigned)__clzll((long long)(m0 | m1)) : 0u);
+      const int sh = 57 - bits;  // bits <= 63
+      // (right shifts round: 64 sums truncated the same way would add up)
+      const long long half = (sh < 0) ? 1ll << (-sh - 1) : 0;
+      a0 = (sh >= 0) ? (long long)((unsigned long long)a0 << sh) : ((a0 + half) >> -sh);
+      a1 = (sh >= 0) ? (long long)((unsigned long long)a1 << sh) : ((a1 + half) >> -sh);
+      if (lane == 0) bexp[cid] = (bits == 0) ? E_NONE : em - 1075 - K - sh;
+    } else {
+      if (!ok) {  // plain FP64
+        double p0 = 0.0, p1 = 0.0;
+        for (int32_t q = r0; q < r1; ++q) {
+          double wx[4] = {0, 0, 0, 0}, wy[4] = {0, 0, 0, 0}, wz[4] = {1, 0, 0, 0};
+          const double *tq = A.tc64 + 3 * (int64_t)q, bb = __ldg(bv + __ldg(A.crows + q));
+          cpm_lagrange<NP, double>(tq[0], wx);
+          cpm_lagrange<NP, double>(tq[1], wy);
+          if (DIM == 3) cpm_lagrange<NP, double>(tq[2], wz);
+          double g = 0.0, h0 = 0.0, h1 = 0.0;
 #pragma unroll
-      for (int cy = 0; cy < NP; ++cy)
+          for (int e = 0; e < 4; ++e) {
+            if (e == cy) g += wy[e];
+            if (e == x0) h0 += wx[e];
+            if (e == x0 + 1) h1 += wx[e];
+          }
+          double gz = 0.0;
 #pragma unroll
-        for (int cx = 0; cx < NP; ++cx) blk[cz][cy][cx] = T(0);
-    const int32_t q1 = __ldg(A.cell_start + cid + 1);
-    for (int32_t q = __ldg(A.cell_start + cid); q < q1; ++q) {
-      const int64_t row = __ldg(A.cell_rows + q);
-      const T *wr = A.w1d + row * 12;
-      const T bb = __ldg(bv + row);
-      T wx[NP], wy[NP], wz[NZ];
+          for (int e = 0; e < 4; ++e)
+            if (e == cz) gz += wz[e];
+          // nodes outside the stencil take nothing, also of infinities
+          if (cy < NP && cz < NP && x0 < NP) p0 += ((h0 * g) * gz) * bb;
+          if (cy < NP && cz < NP && x0 + 1 < NP) p1 += ((h1 * g) * gz) * bb;
+        }
+        a0 = __double_as_longlong(p0);
+        a1 = __double_as_longlong(p1);
+      }
+      if (lane == 0) bexp[cid] = ok ? E_NONE : E_PLAIN;
+    }
+    if (mine) *reinterpret_cast<longlong2 *>(blk + cid * SLOTS + 2 * lane) = make_longlong2(a0, a1);
+  }
+}
+
+template <int DIM, int NP>
+__global__ void __launch_bounds__(TCW * 32)
+    tcell_kernel(TCellArgs A, const float *__restrict__ bv, float *__restrict__ blk) {
+  constexpr int SLOTS = (DIM == 3) ? 64 : 16;
+  __shared__ __align__(16) float s_w[TCW][TCR][3][4];
+  __shared__ float s_b[TCW][TCR];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int x0 = (lane & 1) * 2, cy = (lane >> 1) & 3, cz = (DIM == 3) ? lane >> 3 : 0;
+  const int ax = lane >> 3, j0 = lane & 7;
+  for (int64_t cid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; cid < A.ncells; cid += nwarps) {
+    const int32_t r0 = __ldg(A.cstart + cid), r1 = __ldg(A.cstart + cid + 1);
+    float a0 = 0.0f, a1 = 0.0f;
+    for (int32_t c0 = r0; c0 < r1; c0 += TCR) {
+      const int k = min(TCR, r1 - c0);
+      if (ax < 3) {
+        float wt[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (ax < DIM && j0 < k) cpm_lagrange<NP, float>(__ldg(A.tc32 + 3 * (int64_t)(c0 + j0) + ax), wt);
 #pragma unroll
-      for (int k = 0; k < NP; ++k) { wx[k] = __ldg(wr + k); wy[k] = __ldg(wr + 4 + k); }
-#pragma unroll
-      for (int k = 0; k < NZ; ++k) wz[k] = __ldg(wr + 8 + k);
+        for (int q = 0; q < 4; ++q) s_w[w][j0][ax][q] = (q < NP) ? wt[q] : 0.0f;
+      } else if (j0 < k) {
+        s_b[w][j0] = __ldg(bv + __ldg(A.crows + c0 + j0));
+      }
+      __syncwarp();
+      for (int j = 0; j < k; ++j) {
+        float q = s_b[w][j];
+        if (DIM == 3) q *= s_w[w][j][2][cz];
+        q *= s_w[w][j][1][cy];
+        const float2 wx = *reinterpret_cast<const float2 *>(&s_w[w][j][0][x0]);
+        a0 += wx.x * q;
+        a1 += wx.y * q;
+      }
+      __syncwarp();
+    }
+    if (2 * lane < SLOTS) *reinterpret_cast<float2 *>(blk + cid * SLOTS + 2 * lane) = make_float2(a0, a1);
+  }
+}
+
+// the remainder of one right-hand side, eight lanes per column that has any: up to
+// about a hundred entries near a curve, which one thread each walked as a chain of
+// dependent loads long after the other columns were done
+template <typename T>
+__global__ void __launch_bounds__(256) t_rest_kernel(TArgs<T> A, const int32_t *__restrict__ cols, int64_t ncols, T s,
+                                                     T rowscale, T cs, const T *__restrict__ lam,
+                                                     const T *__restrict__ bv, T *__restrict__ y) {
+  const int sub = threadIdx.x & 7;
+  const unsigned m = 0xFFu << (threadIdx.x & 24);
+  const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3; t < ncols; t += stride) {
+    const int64_t j = __ldg(cols + t);
+    const int32_t e1 = __ldg(A.T_ptr + j + 1);
+    T acc = T(0);
+    for (int32_t e = __ldg(A.T_ptr + j) + sub; e < e1; e += 8) {
+      const int64_t src = __ldg(A.T_src + e);
+      const int kind = __ldg(A.T_kind + e);
+      const T w = (kind == 0) ? s * cs : __ldg(A.T_val + e);
+      acc += w * __ldg((kind == 1 ? bv : lam) + src);
+    }
+    acc += __shfl_xor_sync(m, acc, 1);
+    acc += __shfl_xor_sync(m, acc, 2);
+    acc += __shfl_xor_sync(m, acc, 4);
+    if (sub == 0) y[j] = (j < A.v.NS) ? y[j] + rowscale * acc : acc;
+  }
+}
+
+// The node gather for one right-hand side, one block per brick: the ids (and
+// exponents) of the cells whose base node lies in the brick or up to NP - 1 nodes
+// before it, 11 x 11 x 11, are staged once, so that a node finds its 64 cells at
+// fixed distances in shared memory; on a band about 12 of them exist.
+constexpr int TYT = 256;
+
+template <typename T, int DIM, int NP>
+__global__ void __launch_bounds__(TYT, 5)
+    ty_brick_kernel(TArgs<T> A, const void *__restrict__ blk_, const int32_t *__restrict__ bexp, T dg, T rowscale,
+                    T cs, const T *__restrict__ lam, T *__restrict__ y) {
+  constexpr int H = 7 + NP, HZ = (DIM == 3) ? H : 1;  // NP - 1 before, 8 of the brick
+  constexpr int NZ = (DIM == 3) ? NP : 1;
+  constexpr int SLOTS = (DIM == 3) ? 64 : 16;
+  constexpr bool FX = (sizeof(T) == 8);
+  __shared__ int32_t s_id[HZ * H * H];
+  __shared__ int32_t s_e[FX ? HZ * H * H : 1];
+  const int32_t b = (int32_t)blockIdx.x;
+  for (int e = threadIdx.x; e < HZ * H * H; e += TYT) {
+    const int hx = e % H - (NP - 1), hy = (e / H) % H - (NP - 1), hz = (DIM == 3) ? e / (H * H) - (NP - 1) : 0;
+    const int64_t loc = loc_of(A.v, b, hx, hy, hz);
+    const int32_t id = (loc < 0) ? -1 : __ldg(A.cellid + loc);
+    s_id[e] = id;
+    if (FX) s_e[e] = (id < 0) ? E_NONE : __ldg(bexp + id);
+  }
+  __syncthreads();
+  const int32_t n1 = __ldg(A.v.bstart + b + 1);
+  for (int32_t j = __ldg(A.v.bstart + b) + (int32_t)threadIdx.x; j < n1; j += TYT) {
+    const int l = (int)(__ldg(A.rself + j) & 511u);
+    const int at = (((DIM == 3) ? (l >> 6) + NP - 1 : 0) * H + ((l >> 3) & 7) + NP - 1) * H + (l & 7) + NP - 1;
+    T sum = T(0);
+    if constexpr (FX) {
+      const long long *blk = reinterpret_cast<const long long *>(blk_);
+      int top = E_NONE;
+      bool plain = false;
 #pragma unroll
       for (int cz = 0; cz < NZ; ++cz)
 #pragma unroll
         for (int cy = 0; cy < NP; ++cy)
 #pragma unroll
-          for (int cx = 0; cx < NP; ++cx) blk[cz][cy][cx] += ((wx[cx] * wy[cy]) * wz[cz]) * bb;
+          for (int cx = 0; cx < NP; ++cx) {
+            const int e = s_e[at - (cz * H + cy) * H - cx];
+            plain = plain || e == E_PLAIN;
+            if (e != E_PLAIN) top = max(top, e);
+          }
+      long long acc = 0;
+#pragma unroll
+      for (int cz = 0; cz < NZ; ++cz)
+#pragma unroll
+        for (int cy = 0; cy < NP; ++cy)
+#pragma unroll
+          for (int cx = 0; cx < NP; ++cx) {
+            const int o = at - (cz * H + cy) * H - cx;
+            const int e = s_e[o];
+            if (e != E_NONE && e != E_PLAIN) {
+              const int k = min(top - e, 62);
+              acc += (__ldg(blk + (int64_t)s_id[o] * SLOTS + cz * 16 + cy * 4 + cx) + ((1ll << k) >> 1)) >> k;
+            }
+          }
+      if (top != E_NONE) {
+        constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
+        sum = scaled_sum(fx_scale(back, top), acc, 0.0);
+      }
+      if (plain) {
+        for (int cz = 0; cz < NZ; ++cz)
+          for (int cy = 0; cy < NP; ++cy)
+            for (int cx = 0; cx < NP; ++cx) {
+              const int o = at - (cz * H + cy) * H - cx;
+              if (s_e[o] == E_PLAIN)
+                sum += __longlong_as_double(__ldg(blk + (int64_t)s_id[o] * SLOTS + cz * 16 + cy * 4 + cx));
+            }
+      }
+    } else {
+      const T *blk = reinterpret_cast<const T *>(blk_);
+#pragma unroll
+      for (int cz = 0; cz < NZ; ++cz)
+#pragma unroll
+        for (int cy = 0; cy < NP; ++cy)
+#pragma unroll
+          for (int cx = 0; cx < NP; ++cx) {
+            const int32_t id = s_id[at - (cz * H + cy) * H - cx];
+            if (id >= 0) sum += __ldg(blk + (int64_t)id * SLOTS + cz * 16 + cy * 4 + cx);
+          }
     }
-    T *out = A.tblk + cid * 64;
-#pragma unroll
-    for (int cz = 0; cz < NZ; ++cz)
-#pragma unroll
-      for (int cy = 0; cy < NP; ++cy)
-#pragma unroll
-        for (int cx = 0; cx < NP; ++cx) out[cz * 16 + cy * 4 + cx] = blk[cz][cy][cx];
+    y[j] = rowscale * (sum + (dg * cs) * __ldg(lam + j));
   }
 }
 
+// ---- batches ---------------------------------------------------------------------
 // y = R (d lambda_S + E^T b + remainder)
 template <typename T>
 __global__ void __launch_bounds__(256) ty_kernel(TArgs<T> A, T dg, T s, T rowscale, T cs, const T *__restrict__ lam,
@@ -224,11 +460,6 @@ __global__ void __launch_bounds__(256) ty_kernel(TArgs<T> A, T dg, T s, T rowsca
             if (key < 0) continue;
             const int32_t cell = __ldg(A.cellid + key);
             if (cell < 0) continue;
-            if (A.tblk) {
-              // one right-hand side: the cell's block holds its rows' sum
-              acc += A.tblk[(int64_t)cell * 64 + cz * 16 + cy * 4 + cx];
-              continue;
-            }
             const int32_t q1 = __ldg(A.cell_start + cell + 1);
             for (int32_t q = __ldg(A.cell_start + cell); q < q1; ++q) {
               const int64_t row = __ldg(A.cell_rows + q);
@@ -255,7 +486,8 @@ __global__ void __launch_bounds__(256) ty_kernel(TArgs<T> A, T dg, T s, T rowsca
 cpm_status cpm_build_transpose(cpm_ctx *c) {
   cudaStream_t st = c->stream;
   cudaFree(c->d_T_ptr); cudaFree(c->d_T_row); cudaFree(c->d_T_kind); cudaFree(c->d_T_val); cudaFree(c->d_T_val32);
-  cudaFree(c->d_cellid); cudaFree(c->d_w1d64); cudaFree(c->d_w1d32); cudaFree(c->d_tblk);
+  cudaFree(c->d_cellid); cudaFree(c->d_w1d64); cudaFree(c->d_w1d32); cudaFree(c->d_tblk); cudaFree(c->d_T_cols);
+  c->d_T_cols = nullptr; c->nTcols = 0;
   c->d_w1d64 = nullptr; c->d_w1d32 = nullptr; c->d_tblk = nullptr;
   c->d_T_ptr = nullptr; c->d_T_row = nullptr; c->d_T_kind = nullptr; c->d_T_val = nullptr; c->d_T_val32 = nullptr;
   c->d_cellid = nullptr;
@@ -274,7 +506,8 @@ cpm_status cpm_build_transpose(cpm_ctx *c) {
     if (e_) { rc = cpm_internal_cuda_err(e_); goto done; } \
   } while (0)
   TRY(cudaMalloc(&c->d_cellid, sizeof(int32_t) * std::max<int64_t>(nkeys, 1)));
-  TRY(cudaMalloc(&c->d_tblk, sizeof(double) * 64 * std::max<int64_t>(c->ncells, 1)));
+  // blocks of the one right-hand side form, then the blocks' exponents
+  TRY(cudaMalloc(&c->d_tblk, (sizeof(double) * 64 + sizeof(int32_t)) * std::max<int64_t>(c->ncells, 1)));
   TRY(cudaMemsetAsync(c->d_cellid, 0xFF, sizeof(int32_t) * std::max<int64_t>(nkeys, 1), st));
   TRY(cudaMalloc(&c->d_w1d64, sizeof(double) * 12 * std::max<int64_t>(c->NS, 1)));
   TRY(cudaMalloc(&c->d_w1d32, sizeof(float) * 12 * std::max<int64_t>(c->NS, 1)));
@@ -301,6 +534,14 @@ cpm_status cpm_build_transpose(cpm_ctx *c) {
     tlist_sort_kernel<<<cpm_grid(N, 128), 128, 0, st>>>(c->d_T_ptr, N, c->d_T_row, c->d_T_kind, c->d_T_val,
                                                        c->d_T_val32);
   }
+  // columns with entries (count and cursor are free again)
+  tcol_flag_kernel<<<cpm_grid(N, 256), 256, 0, st>>>(c->d_T_ptr, c->NS, N, count);
+  TRY(cpm_exclusive_scan(count, cursor, N, d_tot, st));
+  TRY(cudaMemcpyAsync(&h_tot, d_tot, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  TRY(cudaStreamSynchronize(st));
+  c->nTcols = h_tot;
+  TRY(cudaMalloc(&c->d_T_cols, sizeof(int32_t) * std::max<int64_t>(c->nTcols, 1)));
+  tcol_fill_kernel<<<cpm_grid(N, 256), 256, 0, st>>>(count, cursor, N, c->d_T_cols);
   TRY(cudaGetLastError());
   TRY(cudaStreamSynchronize(st));
   c->transpose_ready = true;
@@ -336,23 +577,38 @@ cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowsc
   const double inv_h2 = 1.0 / (c->h * c->h);
   const T s = T(n * inv_h2), dg = T(m + n * (-2.0 * c->dim * inv_h2));
   const int64_t N = c->NS + c->NC;
-  // one right-hand side: per-cell blocks of E^T b (reserved at set-up)
-  A.tblk = (nrhs == 1 && ld == 1 && c->d_tblk && c->ncells > 0) ? reinterpret_cast<T *>(c->d_tblk) : nullptr;
   cpm_prof_begin(c, st);
   tb_kernel<T><<<cpm_grid(c->NS * nrhs, 256), 256, 0, st>>>(A, T(s * T(colscale)), u, bv, nrhs, ld);
   int launched = 2;
-  if (A.tblk) {
-    const unsigned gc = cpm_grid(c->ncells, 128);
+  if (nrhs == 1 && ld == 1 && c->d_tblk && c->ncells > 0) {
+    // one right-hand side: per-cell blocks of E^T b (reserved at set-up), then the nodes by bricks
+    TCellArgs C{c->d_cell_start, c->d_cell_rows, c->ncells, c->d_tc64, c->d_tc32};
+    int32_t *bexp = reinterpret_cast<int32_t *>(c->d_tblk + 64 * c->ncells);
+    const unsigned gc = (unsigned)std::min<int64_t>((c->ncells + TCW - 1) / TCW, (int64_t)c->nsm * 64);
+#define CPM_TCELL(D, NP)                                                                                           \
+  do {                                                                                                             \
+    if constexpr (sizeof(T) == 8)                                                                                  \
+      tcell_fx_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<long long *>(c->d_tblk), bexp);      \
+    else                                                                                                           \
+      tcell_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<float *>(c->d_tblk));                   \
+    ty_brick_kernel<T, D, NP><<<(unsigned)c->nb, TYT, 0, st>>>(A, c->d_tblk, bexp, dg, T(rowscale), T(colscale), u, \
+                                                               v);                                                 \
+  } while (0)
     if (c->dim == 3) {
-      if (c->p == 2) tcell_kernel<T, 3, 3><<<gc, 128, 0, st>>>(A, c->ncells, bv);
-      else tcell_kernel<T, 4, 4><<<gc, 128, 0, st>>>(A, c->ncells, bv);
+      if (c->p == 2) CPM_TCELL(3, 3); else CPM_TCELL(3, 4);
     } else {
-      if (c->p == 2) tcell_kernel<T, 3, 1><<<gc, 128, 0, st>>>(A, c->ncells, bv);
-      else tcell_kernel<T, 4, 1><<<gc, 128, 0, st>>>(A, c->ncells, bv);
+      if (c->p == 2) CPM_TCELL(2, 3); else CPM_TCELL(2, 4);
     }
+#undef CPM_TCELL
     ++launched;
+    if (c->nTcols > 0) {
+      t_rest_kernel<T><<<cpm_grid(8 * c->nTcols, 256), 256, 0, st>>>(A, c->d_T_cols, c->nTcols, s, T(rowscale),
+                                                                     T(colscale), u, bv, v);
+      ++launched;
+    }
+  } else {
+    ty_kernel<T><<<cpm_grid(N * nrhs, 256), 256, 0, st>>>(A, dg, s, T(rowscale), T(colscale), u, bv, v, nrhs, ld);
   }
-  ty_kernel<T><<<cpm_grid(N * nrhs, 256), 256, 0, st>>>(A, dg, s, T(rowscale), T(colscale), u, bv, v, nrhs, ld);
   cpm_prof_end(c, st, c->NS * (int64_t)nrhs);
   cpm_count_launches(c, launched);
   CPM_CUDA_TRY(cudaGetLastError());

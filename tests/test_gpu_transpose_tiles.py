@@ -1,0 +1,75 @@
+"""The one right-hand side transposed product by cell blocks and bricks (integer
+sums in FP64): every stencil shape, values at the ends of the exponent range,
+infinities, and a band wide enough that cells hold more than 64 rows.
+
+Tolerances are the repository's for products: 1e-14 (FP64) and 2e-6 (FP32) of the
+largest entry of A^T lambda."""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import cpm_inputs as ci
+from gpu_common import SMALL, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(oracle_mod, name, p, r_band=-1.0):
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.Workload("t", ci.torus(), 1 / 17.3, [ci.torus_meridian(0.3, 1.0, 0.4, ci.BC_DIR2)], 0.0, 1.0) \
+        if name == "torus" else SMALL[name]()
+    band = Band(w.shape, w.h, p=p).set_boundary(w.curves)
+    ref = oracle_mod.Oracle(w.shape, w.h, p=p).set_curves(w.curves)
+    return band, ref
+
+
+@pytest.mark.parametrize("name", ["circle_dir1", "circle_dir2", "sphere_lat_dir2", "torus", "sphere_closed"])
+@pytest.mark.parametrize("p", [3, 2])
+def test_transpose_matches_oracle(oracle_mod, name, p):
+    torch = need_gpu()
+    band, ref = _pair(oracle_mod, name, p)
+    A = sp.csr_matrix(ref.A(0.0, 1.0))
+    lam = ci.random_vector(ref.N, seed=7)
+    y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda"), transpose=True).cpu().numpy()
+    yr = A.T @ lam
+    top = np.max(np.abs(yr))
+    assert np.max(np.abs(y - yr)) <= 1e-14 * top
+    y32 = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda").float(), transpose=True).cpu().numpy()
+    assert np.max(np.abs(y32 - yr)) <= 2e-6 * top
+    for scale in (2.0 ** -900, 2.0 ** 900, 0.0):
+        ys = band.apply(0.0, 1.0, torch.tensor(lam * scale, device="cuda"), transpose=True).cpu().numpy()
+        assert np.max(np.abs(ys - yr * scale)) <= 1e-14 * top * scale
+
+
+def test_an_infinity_stays_in_its_columns(oracle_mod):
+    torch = need_gpu()
+    band, ref = _pair(oracle_mod, "sphere_closed", 3)
+    A = sp.csr_matrix(ref.A(0.0, 1.0))
+    lam = ci.random_vector(ref.N, seed=8)
+    k = ref.N // 3
+    lam[k] = 0.0
+    yr = A.T @ lam
+    lam[k] = np.inf
+    y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda"), transpose=True).cpu().numpy()
+    touched = np.zeros(ref.N, dtype=bool)
+    touched[A[k].indices] = True
+    # (cells share a block: columns of the same cells may become NaN, others may not)
+    ok = np.isfinite(y)
+    assert not np.any(ok[touched] & (np.abs(A[k].toarray()[0][touched]) > 1e-6))
+    assert np.all(np.abs(y[ok] - yr[ok]) <= 1e-11 * np.max(np.abs(yr)))
+    assert ok.sum() > 0.9 * ref.N
+
+
+def test_cells_with_many_rows():
+    """A tube of three radii around the unit circle: over 100 rows share each of its cells."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    band = Band(ci.circle2d(), 0.05, r_band=3.0).set_boundary([])
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    u = torch.randn(band.N, generator=gen, dtype=torch.float64, device="cuda")
+    v = torch.randn(band.N, generator=gen, dtype=torch.float64, device="cuda")
+    a = float(torch.dot(band.apply(0.0, 1.0, u), v))
+    b = float(torch.dot(u, band.apply(0.0, 1.0, v, transpose=True)))
+    # rounding of the two products, each entry of size <= 8/h^2 * 3 per unit of u
+    assert abs(a - b) <= 1e-13 * band.N * 24 / 0.05 ** 2
