@@ -380,59 +380,71 @@ __global__ void __launch_bounds__(TYT, 5)
   for (int32_t j = __ldg(A.v.bstart + b) + (int32_t)threadIdx.x; j < n1; j += TYT) {
     const int l = (int)(__ldg(A.rself + j) & 511u);
     const int at = (((DIM == 3) ? (l >> 6) + NP - 1 : 0) * H + ((l >> 3) & 7) + NP - 1) * H + (l & 7) + NP - 1;
-    T sum = T(0);
-    if constexpr (FX) {
-      const long long *blk = reinterpret_cast<const long long *>(blk_);
-      int top = E_NONE;
-      bool plain = false;
+    // which of the node's cells exist (bit cz 16 + cy 4 + cx), then four at a time, so
+    // that their blocks are read together
+    unsigned long long have = 0;
+    int top = E_NONE;
+    bool plain = false;
 #pragma unroll
-      for (int cz = 0; cz < NZ; ++cz)
+    for (int cz = 0; cz < NZ; ++cz)
 #pragma unroll
-        for (int cy = 0; cy < NP; ++cy)
+      for (int cy = 0; cy < NP; ++cy)
 #pragma unroll
-          for (int cx = 0; cx < NP; ++cx) {
-            const int e = s_e[at - (cz * H + cy) * H - cx];
+        for (int cx = 0; cx < NP; ++cx) {
+          const int o = at - (cz * H + cy) * H - cx;
+          bool yes;
+          if constexpr (FX) {
+            const int e = s_e[o];
+            yes = e != E_NONE;
             plain = plain || e == E_PLAIN;
             if (e != E_PLAIN) top = max(top, e);
+          } else {
+            yes = s_id[o] >= 0;
           }
-      long long acc = 0;
+          if (yes) have |= 1ull << (cz * 16 + cy * 4 + cx);
+        }
+    T sum = T(0);
+    long long acc = 0;
+    while (have) {
+      int slot[4], e[4];
+      int64_t src[4];
+      bool on[4];
 #pragma unroll
-      for (int cz = 0; cz < NZ; ++cz)
-#pragma unroll
-        for (int cy = 0; cy < NP; ++cy)
-#pragma unroll
-          for (int cx = 0; cx < NP; ++cx) {
-            const int o = at - (cz * H + cy) * H - cx;
-            const int e = s_e[o];
-            if (e != E_NONE && e != E_PLAIN) {
-              const int k = min(top - e, 62);
-              acc += (__ldg(blk + (int64_t)s_id[o] * SLOTS + cz * 16 + cy * 4 + cx) + ((1ll << k) >> 1)) >> k;
-            }
-          }
-      if (top != E_NONE) {
-        constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
-        sum = scaled_sum(fx_scale(back, top), acc, 0.0);
+      for (int k = 0; k < 4; ++k) {
+        on[k] = have != 0;
+        slot[k] = on[k] ? __ffsll((long long)have) - 1 : slot[0];
+        have &= have - 1;
+        const int o = at - ((slot[k] >> 4) * H + ((slot[k] >> 2) & 3)) * H - (slot[k] & 3);
+        src[k] = (int64_t)s_id[o] * SLOTS + slot[k];
+        e[k] = FX ? s_e[o] : 0;
       }
-      if (plain) {
-        for (int cz = 0; cz < NZ; ++cz)
-          for (int cy = 0; cy < NP; ++cy)
-            for (int cx = 0; cx < NP; ++cx) {
-              const int o = at - (cz * H + cy) * H - cx;
-              if (s_e[o] == E_PLAIN)
-                sum += __longlong_as_double(__ldg(blk + (int64_t)s_id[o] * SLOTS + cz * 16 + cy * 4 + cx));
-            }
-      }
-    } else {
-      const T *blk = reinterpret_cast<const T *>(blk_);
+      if constexpr (FX) {
+        const long long *blk = reinterpret_cast<const long long *>(blk_);
+        long long z[4];
 #pragma unroll
-      for (int cz = 0; cz < NZ; ++cz)
+        for (int k = 0; k < 4; ++k) z[k] = __ldg(blk + src[k]);
 #pragma unroll
-        for (int cy = 0; cy < NP; ++cy)
-#pragma unroll
-          for (int cx = 0; cx < NP; ++cx) {
-            const int32_t id = s_id[at - (cz * H + cy) * H - cx];
-            if (id >= 0) sum += __ldg(blk + (int64_t)id * SLOTS + cz * 16 + cy * 4 + cx);
+        for (int k = 0; k < 4; ++k) {
+          if (on[k] && e[k] != E_PLAIN) {
+            const int sh = min(top - e[k], 62);
+            acc += (z[k] + ((1ll << sh) >> 1)) >> sh;
+          } else if (on[k]) {
+            sum += __longlong_as_double(z[k]);
           }
+        }
+      } else {
+        const T *blk = reinterpret_cast<const T *>(blk_);
+        T z[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[k] = __ldg(blk + src[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (on[k]) sum += z[k];
+      }
+    }
+    if constexpr (FX) {
+      constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
+      if (top != E_NONE) sum = scaled_sum(fx_scale(back, top), acc, plain ? sum : 0.0);
     }
     y[j] = rowscale * (sum + (dg * cs) * __ldg(lam + j));
   }
