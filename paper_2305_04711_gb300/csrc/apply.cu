@@ -52,7 +52,9 @@ __device__ __forceinline__ void load_nbrs(const int32_t *nbr8, int64_t i, int32_
 }
 
 // one row, one column: u0 = u_i; uk, ak the values at the neighbours nb (anything
-// where nb < 0, ak anything where the neighbour is a BC DOF)
+// where nb < 0, ak anything where the neighbour is a BC DOF).  ALL: all six are
+// PDE DOFs, as in every row away from curves and from the band's edge
+template <bool ALL>
 __device__ __forceinline__ float combine_row(const CombineScale<float> &S, int NS, int nfd, const int32_t (&nb)[6],
                                              float u0, const float (&uk)[6], const float (&ak)[6]) {
   const float ui = S.cs * u0;
@@ -60,10 +62,11 @@ __device__ __forceinline__ float combine_row(const CombineScale<float> &S, int N
   int present = 0;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    if (nb[k] < 0) continue;
+    if (!ALL && nb[k] < 0) continue;
     ++present;
-    s += (nb[k] < NS) ? ak[k] + (S.cs * uk[k] - ui) : uk[k] - ui;
+    s += (ALL || nb[k] < NS) ? ak[k] + (S.cs * uk[k] - ui) : uk[k] - ui;
   }
+  if (ALL) return S.m * u0 + S.c * s;
   return S.m * u0 + S.c * (s - (float)(nfd - present) * ui);
 }
 
@@ -82,6 +85,7 @@ __device__ __forceinline__ double combine_row_plain(const CombineScale<double> &
   return S.m * u0 + S.c * (s - (nfd - present) * ui);
 }
 
+template <bool ALL>
 __device__ __forceinline__ double combine_row(const CombineScale<double> &S, int NS, int nfd,
                                               const int32_t (&nb)[6], double u0, const double (&uk)[6],
                                               const double (&ak)[6]) {
@@ -89,12 +93,12 @@ __device__ __forceinline__ double combine_row(const CombineScale<double> &S, int
   int npde = 0, nbc = 0;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    if (nb[k] >= 0 && nb[k] < NS) {
+    if (ALL || (nb[k] >= 0 && nb[k] < NS)) {
       ++npde;
       tu = max(tu, fx_key(uk[k]));
       ta = max(ta, fx_key(ak[k]));
     }
-    nbc += nb[k] >= NS;
+    if (!ALL) nbc += nb[k] >= NS;
   }
   const int eu = (int)(tu >> 20), ea = (int)(ta >> 20);
   const int ecs = ((__double2hiint(S.cs) >> 20) & 0x7FF) + eu - 1081;
@@ -104,18 +108,18 @@ __device__ __forceinline__ double combine_row(const CombineScale<double> &S, int
     const long long x0 = fx_of(u0, eu, 6);
 #pragma unroll
     for (int k = 0; k < 6; ++k)
-      if (nb[k] >= 0 && nb[k] < NS) {
+      if (ALL || (nb[k] >= 0 && nb[k] < NS)) {
         su += fx_of(uk[k], eu, 6) - x0;
         sa += fx_of(ak[k], ea, 6);
       }
     double s = (ta == 0u) ? 0.0 : (double)sa * fx_scale(1.0, ea - 1081);
     if (tu != 0u) s = fma((double)su, fx_scale(S.cs, eu - 1081), s);
-    if (nbc) {
+    if (!ALL && nbc) {
 #pragma unroll
       for (int k = 0; k < 6; ++k)
         if (nb[k] >= NS) s += uk[k] - S.cs * u0;
     }
-    const int miss = nfd - npde - nbc;
+    const int miss = ALL ? 0 : nfd - npde - nbc;
     if (miss) s -= miss * (S.cs * u0);
     return fma(S.c, s, S.m * u0);
   }
@@ -137,7 +141,7 @@ __device__ __forceinline__ T combine_element(const CombineArgs &A, const Combine
       uk[k] = __ldg(u + c * ld + r);
       ak[k] = __ldg(a + ca * ld + r);
     }
-    return combine_row(S, (int)A.NS, A.nfd, nb, u0, uk, ak);
+    return combine_row<false>(S, (int)A.NS, A.nfd, nb, u0, uk, ak);
   }
   const int64_t al = i - A.NS;
   const int cnt = __ldg(A.bc_cnt + al);
@@ -227,10 +231,31 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 3 : 4) combine_batched
     const int c1 = (int)((c0 + chunk < N) ? c0 + chunk : N);
     for (int i = (int)c0 + (int)(threadIdx.x >> 5); i < c1; i += 8) {
       int32_t nb[6];
-      if (i < NS) load_nbrs(A.nbr8, i, nb);
+      bool all = false;  // (the same in the whole warp)
+      if (i < NS) {
+        load_nbrs(A.nbr8, i, nb);
+        all = min(min(min(nb[0], nb[1]), min(nb[2], nb[3])), min(nb[4], nb[5])) >= 0 &&
+              max(max(max(nb[0], nb[1]), max(nb[2], nb[3])), max(nb[4], nb[5])) < NS;
+      }
       for (int col = lane * RPL; col < nrhs; col += 32 * RPL) {
         T out[RPL];
-        if (i < NS) {
+        if (all) {
+          T u0[RPL], uk[6][RPL], ak[6][RPL];
+          ldv<T, RPL>(u + (uint64_t)(unsigned)i * ld + col, u0);
+#pragma unroll
+          for (int q = 0; q < 6; ++q) {
+            const uint64_t o = (uint64_t)(unsigned)nb[q] * ld + col;
+            ldv<T, RPL>(u + o, uk[q]);
+            ldv<T, RPL>(a + o, ak[q]);
+          }
+#pragma unroll
+          for (int k = 0; k < RPL; ++k) {
+            T x[6], y[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) { x[q] = uk[q][k]; y[q] = ak[q][k]; }
+            out[k] = combine_row<true>(S, NS, A.nfd, nb, u0[k], x, y);
+          }
+        } else if (i < NS) {
           T u0[RPL], uk[6][RPL], ak[6][RPL];
           ldv<T, RPL>(u + (uint64_t)(unsigned)i * ld + col, u0);
 #pragma unroll
@@ -244,7 +269,7 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 3 : 4) combine_batched
             T x[6], y[6];
 #pragma unroll
             for (int q = 0; q < 6; ++q) { x[q] = uk[q][k]; y[q] = ak[q][k]; }
-            out[k] = combine_row(S, NS, A.nfd, nb, u0[k], x, y);
+            out[k] = combine_row<false>(S, NS, A.nfd, nb, u0[k], x, y);
           }
         } else {
           const int64_t al = i - NS;

@@ -709,8 +709,11 @@ done:
   return rc;
 }
 
-// the default number of x passes (node values of one pass near 64 registers)
-int cpm_cells_default_xh(int np1, bool fp64, int /*rpl*/) { return (np1 == 3 || fp64) ? 1 : 2; }
+// the default number of x passes (node values of one pass near 64 registers); the
+// FP64 gather has no passes and names what its columns per lane would have had
+int cpm_cells_default_xh(int np1, bool fp64, int rpl) {
+  return (np1 == 3) ? ((fp64 && rpl == 2) ? 3 : 1) : (fp64 ? (rpl == 2 ? 4 : 2) : 2);
+}
 
 static CellArgs cell_args(const cpm_ctx *c) {
   return CellArgs{c->d_cell_start, c->d_cell_rows, c->d_cell_key, reinterpret_cast<const int2 *>(c->d_cell_lines),

@@ -61,7 +61,8 @@ constexpr int unroll_of() { return (sizeof(T) == 8) ? 2 : 4; }
 // grid-stride element loop with UNR elements per thread in flight; the body
 // functor loads into its element state, then updates and accumulates.  Runs
 // of 16 products are summed in T, the runs in FP64 (for FP32 vectors this
-// keeps the FP64 pipe, 1/64 of the FP32 rate here, off the hot loop).
+// keeps the FP64 pipe, 1/64 of the FP32 rate here, off the hot loop).  A block
+// keeps its threads on fixed columns.
 template <typename T, int NQ, class Body>
 __device__ __forceinline__ void vloop(const Body &body, int64_t N, int nrhs, int64_t ld, double (&acc)[NQ]) {
   constexpr int UNR = unroll_of<T>();
@@ -75,18 +76,15 @@ __device__ __forceinline__ void vloop(const Body &body, int64_t N, int nrhs, int
 #pragma unroll
   for (int q = 0; q < NQ; ++q) run[q] = T(0);
   int k = 0;
-  for (int64_t i0 = (int64_t)blockIdx.x * rows_per + sub; i0 < N; i0 += UNR * stride) {
-    typename Body::Elt e[UNR];
+  int64_t i0 = (int64_t)blockIdx.x * rows_per + sub, o = i0 * ld + c;
+  const int64_t so = stride * ld;
+  typename Body::Elt e[UNR];
+  // whole groups: all loads of UNR elements start together
+  for (; i0 + (UNR - 1) * stride < N; i0 += UNR * stride, o += UNR * so) {
 #pragma unroll
-    for (int u = 0; u < UNR; ++u) {
-      const int64_t i = i0 + u * stride;
-      if (i < N) body.load(e[u], i, i * ld + c);
-    }
+    for (int u = 0; u < UNR; ++u) body.load(e[u], i0 + u * stride, o + u * so);
 #pragma unroll
-    for (int u = 0; u < UNR; ++u) {
-      const int64_t i = i0 + u * stride;
-      if (i < N) body.apply(e[u], i, i * ld + c, run);
-    }
+    for (int u = 0; u < UNR; ++u) body.apply(e[u], i0 + u * stride, o + u * so, run);
     k += UNR;
     if (k >= 16) {
 #pragma unroll
@@ -94,6 +92,12 @@ __device__ __forceinline__ void vloop(const Body &body, int64_t N, int nrhs, int
       k = 0;
     }
   }
+#pragma unroll
+  for (int u = 0; u < UNR - 1; ++u)
+    if (i0 + u * stride < N) body.load(e[u], i0 + u * stride, o + u * so);
+#pragma unroll
+  for (int u = 0; u < UNR - 1; ++u)
+    if (i0 + u * stride < N) body.apply(e[u], i0 + u * stride, o + u * so, run);
 #pragma unroll
   for (int q = 0; q < NQ; ++q) acc[q] += (double)run[q];
 }
