@@ -215,133 +215,118 @@ __device__ __forceinline__ CellHead cell_head(const CellArgs &A, int64_t cid, in
   return h;
 }
 
-// One warp per cell; each lane takes R adjacent columns (32 R per group).  For
-// a group the lane loads the cell's node values (NX x positions per pass, XH
-// passes) into registers and applies each row of the cell: the y-z weights
-// along each x position (P[cx] = sum_{cy,cz} w_y w_z u), then the x weights.
-// Partial sums of the passes wait in shared memory.  A block's warps take
-// neighbouring cells, which share most of their nodes in L1, and a warp reads
-// the head and the fractions of its next cell while it works on this one.
+// One warp per cell and group of 32 R columns, R adjacent ones per lane.  The lane
+// takes the cell's nodes plane by plane (z), 16 values times R columns in registers,
+// and applies w_x, w_y, w_z of up to CHUNK rows one after the other.  A weight that a
+// warp reads from shared memory takes the LSU a wavefront whatever its width, so
+// rows read the 9 weights of a plane and not 16 products of two and the third
+// (850 -> 800 us of the 64-column product on the sphere at h = 1/128, whose
+// multiply-adds take 230; 16 warps per SM then wait for L2 and for each other's
+// 64 node rows of 256 B in L1).  The lines of the next cell are read while this one
+// is worked on.
 //
 // The node values enter as differences to the cell's base-node value u_c and
 // each row adds u_c - u_i, which equals sum_n w_n (u_n - u_i) since
 // sum_n w_n = 1; rounding then stays relative to local differences.
-template <int DIM, int NP, int XH, int R>
-__global__ void __launch_bounds__(WARPS * 32, (NP / XH * R <= 2) ? 3 : 2)
+template <int DIM, int NP, int R>
+__global__ void __launch_bounds__(WARPS * 32, 2)
     gather_cells_kernel(CellArgs A, const float *__restrict__ tc, float cs, const float *__restrict__ u,
-                        float *__restrict__ a, int nrhs, unsigned ld_) {
-  typedef float T;
+                        float *__restrict__ a, int nrhs, unsigned ld) {
   constexpr int NZ = (DIM == 3) ? NP : 1;
-  constexpr int NL = NP * NZ;  // stencil lines along x
-  constexpr int NX = NP / XH;  // x positions per pass
-  static_assert(NX * XH == NP, "passes must split the stencil's x positions");
-  typedef typename VecT<T, R>::t V;
-  typedef typename Weight<R>::t WT;
-  __shared__ __align__(16) WT s_wyz[WARPS][CHUNK][(NL + 3) / 4 * 4];
-  __shared__ __align__(16) WT s_wx[WARPS][CHUNK][4];
+  __shared__ __align__(16) float s_w[WARPS][CHUNK][3][4];
   __shared__ int32_t s_row[WARPS][CHUNK];
   __shared__ __align__(16) int32_t s_idx[WARPS][16 * 4];
-  __shared__ V s_acc[(XH > 1) ? WARPS : 1][CHUNK][32];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int ngroups = (nrhs + 32 * R - 1) / (32 * R);
-  if (warp >= A.ncells) return;
-  CellHead h = cell_head<NP>(A, warp, lane);
-  for (int64_t cid = warp; cid < A.ncells; cid += nwarps) {
-    // node x of line cz * 4 + cy at s_idx[line * 4 + x]
-    if (lane < 16) {
+  const int64_t items = A.ncells * ngroups;
+  if (warp >= items) return;
+  int64_t cid = (ngroups == 1) ? warp : warp / ngroups;
+  CellHead h = cell_head<NP>(A, cid, lane);
+  const int ax = lane >> 3, j0 = lane & 7;
+  for (int64_t it = warp; it < items; it += nwarps) {
+    const int col = ((int)(it - cid * ngroups) * 32 + lane) * R;
+    const bool on = col < nrhs;
+    const float *ul = u + (on ? col : 0);  // lanes past the last column read the first ones (and store nothing)
+    const int32_t r0 = h.r0, r1 = h.r1;
+    if (lane < 16) {  // node x of line cz * 4 + cy at s_idx[line * 4 + x]
       int4 o;
       o.x = h.line.x;
       o.y = (1 < h.split) ? h.line.x + 1 : h.line.y + (1 - h.split);
       o.z = (2 < h.split) ? h.line.x + 2 : h.line.y + (2 - h.split);
       o.w = (3 < h.split) ? h.line.x + 3 : h.line.y + (3 - h.split);
-      *reinterpret_cast<int4 *>(&s_idx[wib][lane * 4]) = o;
+      *reinterpret_cast<int4 *>(&s_idx[w][lane * 4]) = o;
     }
-    const int32_t r0 = h.r0, r1 = h.r1;
-    if (cid + nwarps < A.ncells) h = cell_head<NP>(A, cid + nwarps, lane);
-    __syncwarp();
-    const int32_t base = s_idx[wib][0];
+    const int64_t itn = it + nwarps;
+    if (itn < items) {
+      cid = (ngroups == 1) ? itn : itn / ngroups;
+      h = cell_head<NP>(A, cid, lane);
+    }
     for (int32_t c0 = r0; c0 < r1; c0 += CHUNK) {
       const int k = min(CHUNK, r1 - c0);
-      if (lane < k) {
-        s_row[wib][lane] = __ldg(A.crows + c0 + lane);
-        const T *tq = tc + 3 * (int64_t)(c0 + lane);
-        T wx[4], wy[4], wz[4];
-        cpm_lagrange<NP, T>(__ldg(tq), wx);
-        cpm_lagrange<NP, T>(__ldg(tq + 1), wy);
-        if (DIM == 3) cpm_lagrange<NP, T>(__ldg(tq + 2), wz);
-        else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
-#pragma unroll
-        for (int q = 0; q < NP; ++q) s_wx[wib][lane][q] = Weight<R>::of(wx[q]);
-#pragma unroll
-        for (int q = 0; q < NL; ++q) s_wyz[wib][lane][q] = Weight<R>::of(wy[q % NP] * wz[q / NP]);
+      const int32_t q = c0 + min(j0, k - 1);  // (rows past the last repeat it)
+      if (ax < 3) {  // lane 8 axis + j forms the weights of one axis of row j
+        float wt[4] = {1.0f, 0.0f, 0.0f, 0.0f};
+        if (ax < DIM) cpm_lagrange<NP, float>(__ldg(tc + 3 * (int64_t)q + ax), wt);
+        *reinterpret_cast<float4 *>(s_w[w][j0][ax]) = make_float4(wt[0], wt[1], wt[2], (NP == 4) ? wt[3] : 0.0f);
+      } else {
+        s_row[w][j0] = __ldg(A.crows + q);
       }
       __syncwarp();
-      for (int grp = 0; grp < ngroups; ++grp) {
-        const int col = (grp * 32 + lane) * R;
-        const bool on = col < nrhs;
-        T uc[R];
+      float part[CHUNK][R], uc[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) uc[q] = T(0);
-        vld<T, R>(u + (uint64_t)(unsigned)base * ld_ + (on ? col : 0), uc);
+      for (int j = 0; j < CHUNK; ++j)
+#pragma unroll
+        for (int r = 0; r < R; ++r) part[j][r] = 0.0f;
+      vld<float, R>(ul + (uint64_t)(unsigned)s_idx[w][0] * ld, uc);
 #pragma unroll 1
-        for (int xp = 0; xp < XH; ++xp) {
-          T d[NL][NX][R];
+      for (int cz = 0; cz < NZ; ++cz) {
+        float d[NP][NP][R];
 #pragma unroll
-          for (int ln = 0; ln < NL; ++ln) {
+        for (int cy = 0; cy < NP; ++cy) {
+          const int4 n4 = *reinterpret_cast<const int4 *>(&s_idx[w][(cz * 4 + cy) * 4]);
+          const int32_t n[4] = {n4.x, n4.y, n4.z, n4.w};
 #pragma unroll
-            for (int q = 0; q < NX; ++q) {
-              const int32_t idx = s_idx[wib][((ln / NP) * 4 + ln % NP) * 4 + xp * NX + q];
-              // lanes past the last column read the first ones (and store nothing)
-              vld<T, R>(u + (uint64_t)(unsigned)idx * ld_ + (on ? col : 0), d[ln][q]);
-            }
-          }
-#pragma unroll
-          for (int ln = 0; ln < NL; ++ln)
-#pragma unroll
-            for (int q = 0; q < NX; ++q) sub_v<T, R>(d[ln][q], uc);
-#pragma unroll 1
-          for (int j = 0; j < k; ++j) {
-            T P[NX][R];
-#pragma unroll
-            for (int q = 0; q < NX; ++q)
-#pragma unroll
-              for (int r = 0; r < R; ++r) P[q][r] = T(0);
-#pragma unroll
-            for (int ln = 0; ln < NL; ++ln) {
-              const WT w = s_wyz[wib][j][ln];
-#pragma unroll
-              for (int q = 0; q < NX; ++q) axpy_w(P[q], w, d[ln][q]);
-            }
-            T part[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) part[r] = T(0);
-#pragma unroll
-            for (int q = 0; q < NX; ++q) axpy_w(part, s_wx[wib][j][xp * NX + q], P[q]);
-            if (XH > 1 && xp > 0) {
-              const V pv = s_acc[(XH > 1) ? wib : 0][j][lane];
-              const T *pp = reinterpret_cast<const T *>(&pv);
-#pragma unroll
-              for (int r = 0; r < R; ++r) part[r] += pp[r];
-            }
-            if (XH > 1 && xp < XH - 1) {
-              V pv;
-              T *pp = reinterpret_cast<T *>(&pv);
-#pragma unroll
-              for (int r = 0; r < R; ++r) pp[r] = part[r];
-              s_acc[(XH > 1) ? wib : 0][j][lane] = pv;
-            } else if (on) {
-              const unsigned row = (unsigned)s_row[wib][j];
-              T ui[R];
-              vld<T, R>(u + (uint64_t)row * ld_ + col, ui);
-#pragma unroll
-              for (int r = 0; r < R; ++r) part[r] = cs * (part[r] + (uc[r] - ui[r]));
-              vst<T, R>(a + (uint64_t)row * ld_ + col, part);
-            }
-          }
+          for (int cx = 0; cx < NP; ++cx) vld<float, R>(ul + (uint64_t)(unsigned)n[cx] * ld, d[cy][cx]);
         }
+#pragma unroll
+        for (int cy = 0; cy < NP; ++cy)
+#pragma unroll
+          for (int cx = 0; cx < NP; ++cx) sub_v<float, R>(d[cy][cx], uc);
+#pragma unroll
+        for (int j = 0; j < CHUNK; ++j)
+          if (j < k) {
+            const float4 x4 = *reinterpret_cast<const float4 *>(s_w[w][j][0]);
+            const float4 y4 = *reinterpret_cast<const float4 *>(s_w[w][j][1]);
+            const float wx[4] = {x4.x, x4.y, x4.z, x4.w}, wy[4] = {y4.x, y4.y, y4.z, y4.w};
+            float S[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) S[r] = 0.0f;
+#pragma unroll
+            for (int cy = 0; cy < NP; ++cy) {
+              float L[R];
+#pragma unroll
+              for (int r = 0; r < R; ++r) L[r] = 0.0f;
+#pragma unroll
+              for (int cx = 0; cx < NP; ++cx) axpy_w(L, Weight<R>::of(wx[cx]), d[cy][cx]);
+              axpy_w(S, Weight<R>::of(wy[cy]), L);
+            }
+            axpy_w(part[j], Weight<R>::of(s_w[w][j][2][cz]), S);
+          }
       }
+      float ui[CHUNK][R];
+#pragma unroll
+      for (int j = 0; j < CHUNK; ++j) vld<float, R>(ul + (uint64_t)(unsigned)s_row[w][j] * ld, ui[j]);
+      if (on)
+#pragma unroll
+        for (int j = 0; j < CHUNK; ++j)
+          if (j < k) {
+            float o[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] = cs * (part[j][r] + (uc[r] - ui[j][r]));
+            vst<float, R>(a + (uint64_t)(unsigned)s_row[w][j] * ld + col, o);
+          }
       __syncwarp();
     }
   }
@@ -709,8 +694,8 @@ done:
   return rc;
 }
 
-// the default number of x passes (node values of one pass near 64 registers); the
-// FP64 gather has no passes and names what its columns per lane would have had
+// the x passes that cpm_tune_info names; the gathers take z planes and have no use
+// for them, recorded shapes stay valid
 int cpm_cells_default_xh(int np1, bool fp64, int rpl) {
   return (np1 == 3) ? ((fp64 && rpl == 2) ? 3 : 1) : (fp64 ? (rpl == 2 ? 4 : 2) : 2);
 }
@@ -720,27 +705,15 @@ static CellArgs cell_args(const cpm_ctx *c) {
                   c->ncells};
 }
 
-template <int DIM, int NP, int R, int XH>
-static void launch_cells_xh(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
-                            cudaStream_t st, unsigned g) {
-  if constexpr (NP % XH == 0)
-    gather_cells_kernel<DIM, NP, XH, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, (unsigned)ld);
-}
-
 template <int DIM, int NP, int R>
 static void launch_cells_k(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
                            cudaStream_t st) {
-  int xh = c->tune.cells_xh[0][R - 1];
-  if (xh <= 0 || xh > 4 || NP % xh != 0) xh = cpm_cells_default_xh(NP, false, R);
-  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : 16;
-  unsigned g = (unsigned)std::min<int64_t>((c->ncells + WARPS - 1) / WARPS, (int64_t)c->nsm * per_sm);
-  if (g < 1) g = 1;
-  switch (xh) {
-    case 1: launch_cells_xh<DIM, NP, R, 1>(c, cs, u, a, nrhs, ld, st, g); break;
-    case 2: launch_cells_xh<DIM, NP, R, 2>(c, cs, u, a, nrhs, ld, st, g); break;
-    case 3: launch_cells_xh<DIM, NP, R, 3>(c, cs, u, a, nrhs, ld, st, g); break;
-    default: launch_cells_xh<DIM, NP, R, 4>(c, cs, u, a, nrhs, ld, st, g); break;
-  }
+  // by default 4 blocks per SM (two rounds) with two columns per lane, 16 with one:
+  // 1324 / 1353 us of the 64-column product, 1202 / 1061 us of 24 columns (4 / 16)
+  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : (R == 2 ? 4 : 16);
+  const int64_t items = c->ncells * ((nrhs + 32 * R - 1) / (32 * R));
+  const unsigned g = (unsigned)std::min<int64_t>((items + WARPS - 1) / WARPS, (int64_t)c->nsm * per_sm);
+  gather_cells_kernel<DIM, NP, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, (unsigned)ld);
 }
 
 template <int R>

@@ -113,7 +113,7 @@ struct PBody {
   __device__ void init(int c) const {
     c_ = c;
     restart = sc[c * NSC + S_RESTART] != 0.0;
-    nres = (unsigned)sc[c * NSC + S_NRESTART];
+    nres = (unsigned)(sc[c * NSC + S_SEED] + sc[c * NSC + S_NRESTART]);
     beta = T(sc[c * NSC + S_BETA]);
     omega = T(sc[c * NSC + S_OMEGA]);
   }
@@ -194,7 +194,7 @@ struct XRBody {
   __device__ bool on(int c) const { return sc[c * NSC + S_ACTIVE] != 0.0; }
   __device__ void init(int c) const {
     c_ = c;
-    nres = (unsigned)sc[c * NSC + S_NRESTART] + 1u;
+    nres = (unsigned)(sc[c * NSC + S_SEED] + sc[c * NSC + S_NRESTART]) + 1u;
     alpha = T(sc[c * NSC + S_ALPHA]);
     omega = T(sc[c * NSC + S_OMEGA]);
   }
@@ -235,7 +235,7 @@ struct InitBody {
   __device__ void load(Elt &e, int64_t, int64_t o) const { e.f = f[o]; e.r = x_zero ? T(0) : r[o]; }
   __device__ void apply(Elt &e, int64_t i, int64_t o, T (&run)[4]) const {
     const T rv = e.f - e.r;
-    const T sh = shadow_of(cv, i, c_, rv, 0u);
+    const T sh = shadow_of(cv, i, c_, rv, cv.seed);
     r[o] = rv; rh[o] = sh; p[o] = T(0); v[o] = T(0);
     run[0] += rv * rv;
     run[1] += e.f * e.f;
@@ -355,9 +355,10 @@ struct GraphKey {
   double m = 0, n = 0, rs = 0, cs = 0, tol = 0, stall = 0;
   float mix = 0;
   int shadow = 0;
-  unsigned seed = 0;
   const void *x = nullptr, *vecs = nullptr;
+  const void *a_scr = nullptr, *b_scr = nullptr;  // the products' intermediates (cpm_reserve may move them)
   int nrhs = 0, steps = 0, elem = 0, xelem = 0, G = 0;
+  int single_mode = 0, cells_blocks = 0, combine_warps = 0;  // launch shapes in force
   int64_t ld = 0;
   bool operator==(const GraphKey &o) const { return std::memcmp(this, &o, sizeof(GraphKey)) == 0; }
 };
@@ -374,9 +375,15 @@ struct SolveWork {
   unsigned *ticket = nullptr;
   double *h_pin = nullptr;   // host mirror: [NSC * ld] scalars, then [NQMAX * ld] dots
   int G = 0;                 // blocks of the vector kernels (fixed: deterministic reductions)
-  cudaGraphExec_t gexec = nullptr;
-  GraphKey gkey;
-  int64_t glaunches = 0;     // kernels per replay
+  // captured iteration groups, the least recently used one replaced: forward and
+  // adjoint, FP64 and FP32 solves of a program that alternates them
+  struct Graph {
+    cudaGraphExec_t exec = nullptr;
+    GraphKey key;
+    int64_t launches = 0;    // kernels per replay
+    uint64_t used = 0;
+  } graphs[4];
+  uint64_t guses = 0;
   bool graphs_ok = true;
 };
 
@@ -388,7 +395,8 @@ static void free_work(SolveWork *w) {
   cudaFree(w->r64); cudaFree(w->xc);
   cudaFree(w->part); cudaFree(w->sc); cudaFree(w->out); cudaFree(w->cols); cudaFree(w->ticket);
   if (w->h_pin) cudaFreeHost(w->h_pin);
-  if (w->gexec) cudaGraphExecDestroy(w->gexec);
+  for (auto &g : w->graphs)
+    if (g.exec) cudaGraphExecDestroy(g.exec);
   delete w;
 }
 
@@ -497,35 +505,45 @@ cpm_status iterations(cpm_ctx *c, const Op<T> &op, TX *x, const Vecs<T> &V, Solv
     GraphKey k;
     std::memset(&k, 0, sizeof(k));
     k.fn = (const void *)op.fn; k.m = op.m; k.n = op.n; k.rs = op.rowscale; k.cs = op.colscale;
-    k.tol = cv.tol; k.stall = cv.stall; k.mix = cv.mix; k.shadow = cv.shadow; k.seed = cv.seed;
+    k.tol = cv.tol; k.stall = cv.stall; k.mix = cv.mix; k.shadow = cv.shadow;
     k.x = x; k.vecs = V.r; k.nrhs = nrhs; k.steps = steps;
     k.elem = (int)sizeof(T); k.xelem = (int)sizeof(TX); k.ld = ld; k.G = w->G;
-    if (!(w->gexec && w->gkey == k)) {
-      if (w->gexec) { cudaGraphExecDestroy(w->gexec); w->gexec = nullptr; }
+    k.a_scr = c->a_scratch.p; k.b_scr = c->b_scratch.p;
+    k.single_mode = c->tune.single_mode; k.cells_blocks = c->tune.cells_blocks_per_sm;
+    k.combine_warps = c->tune.combine_warps_per_sm;
+    SolveWork::Graph *g = nullptr;
+    for (auto &e : w->graphs)
+      if (e.exec && e.key == k) g = &e;
+    if (!g) {
+      g = &w->graphs[0];
+      for (auto &e : w->graphs)
+        if (e.used < g->used) g = &e;
+      if (g->exec) { cudaGraphExecDestroy(g->exec); g->exec = nullptr; }
       const int64_t before = c->prof.launches;
-      cudaGraph_t g = nullptr;
+      cudaGraph_t gr = nullptr;
       cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
       cpm_status rc = CPM_OK;
       if (e == cudaSuccess) {
         for (int s = 0; s < steps && rc == CPM_OK; ++s) rc = iteration<T, TX>(c, op, x, V, w, nrhs, ld, cv, st);
-        e = cudaStreamEndCapture(st, &g);
+        e = cudaStreamEndCapture(st, &gr);
       }
-      if (rc == CPM_OK && e == cudaSuccess && g) e = cudaGraphInstantiate(&w->gexec, g, 0);
-      if (g) cudaGraphDestroy(g);
-      w->glaunches = c->prof.launches - before;
+      if (rc == CPM_OK && e == cudaSuccess && gr) e = cudaGraphInstantiate(&g->exec, gr, 0);
+      if (gr) cudaGraphDestroy(gr);
+      g->launches = c->prof.launches - before;
       c->prof.launches = before;
       if (rc != CPM_OK || e != cudaSuccess) {
         // capture not available here: plain launches from now on
         (void)cudaGetLastError();
-        if (w->gexec) { cudaGraphExecDestroy(w->gexec); w->gexec = nullptr; }
+        if (g->exec) { cudaGraphExecDestroy(g->exec); g->exec = nullptr; }
         w->graphs_ok = false;
         if (rc != CPM_OK) return rc;
         return iterations<T, TX>(c, op, x, V, w, nrhs, ld, cv, steps, false, st);
       }
-      w->gkey = k;
+      std::memcpy(&g->key, &k, sizeof(k));  // (padding too: keys are compared as bytes)
     }
-    CPM_CUDA_TRY(cudaGraphLaunch(w->gexec, st));
-    cpm_count_launches(c, (int)w->glaunches);
+    g->used = ++w->guses;
+    CPM_CUDA_TRY(cudaGraphLaunch(g->exec, st));
+    cpm_count_launches(c, (int)g->launches);
     return CPM_OK;
   }
   for (int s = 0; s < steps; ++s) {

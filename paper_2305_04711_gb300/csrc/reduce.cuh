@@ -11,7 +11,7 @@ constexpr int NQMAX = 4;   // dot products reduced by one kernel at most
 // per right-hand side scalar slots
 enum {
   S_RHO_OLD = 0, S_ALPHA, S_OMEGA, S_RHO, S_BETA, S_ACTIVE, S_RESTART, S_NRESTART, S_FN2, S_RN2, S_BROKE,
-  S_BEST, S_STALL, S_STOPPED, S_RN2_0, S_ITERS, S_RH2, NSC
+  S_BEST, S_STALL, S_STOPPED, S_RN2_0, S_ITERS, S_RH2, S_SEED, NSC
 };
 
 enum { ST_OUT = 0, ST_INIT, ST_ALPHA, ST_OMEGA, ST_XR };
@@ -29,7 +29,7 @@ struct Conv {
   double stall;   // iterations without the residual halving before giving up
   float mix;      // shadow = r o (1 + mix u) (shadow 0; mix 0: the classical rhat = r)
   int shadow;     // 0: rhat from r as above; 1: rhat = u, independent of r
-  unsigned seed;  // of the hash u
+  unsigned seed;  // of the hash u (kept as S_SEED from the initial residual on: captured iterations serve any)
 };
 
 namespace {
@@ -47,14 +47,15 @@ __device__ __forceinline__ float hash_unit(int64_t i, int c, unsigned seed) {
 // right-hand side on the BC rows only) A r lives elsewhere and (rhat, A r) = 0:
 // the first step breaks down.  A random rhat (shadow 1) meets every row; its
 // (rhat, r) ~ |rhat| |r| / sqrt(N) is still far above the rounding of the dot
-// products.  `restarts` selects a fresh hash after a near-breakdown.
-__device__ __forceinline__ float shadow_of(const Conv &cv, int64_t i, int c, float r, unsigned restarts) {
-  if (cv.shadow == 1) return hash_unit(i, c, cv.seed + restarts);
+// products.  `seed` is the hash's seed plus the restarts so far, which select a fresh
+// hash after a near-breakdown.
+__device__ __forceinline__ float shadow_of(const Conv &cv, int64_t i, int c, float r, unsigned seed) {
+  if (cv.shadow == 1) return hash_unit(i, c, seed);
   if (cv.mix == 0.0f) return r;
   return r * (1.0f + cv.mix * hash_unit(i, c, 0u));
 }
-__device__ __forceinline__ double shadow_of(const Conv &cv, int64_t i, int c, double r, unsigned restarts) {
-  if (cv.shadow == 1) return (double)hash_unit(i, c, cv.seed + restarts);
+__device__ __forceinline__ double shadow_of(const Conv &cv, int64_t i, int c, double r, unsigned seed) {
+  if (cv.shadow == 1) return (double)hash_unit(i, c, seed);
   if (cv.mix == 0.0f) return r;
   return r * (1.0 + (double)cv.mix * (double)hash_unit(i, c, 0u));
 }
@@ -137,6 +138,7 @@ __device__ void stage_finish(int stage, const Red &R, const Conv &cv, int c, con
     s[S_RHO] = d[2]; s[S_RHO_OLD] = 1.0; s[S_ALPHA] = 1.0; s[S_OMEGA] = 1.0; s[S_BETA] = 0.0;
     s[S_RESTART] = 0.0; s[S_NRESTART] = 0.0; s[S_BROKE] = 0.0; s[S_STALL] = 0.0; s[S_STOPPED] = 0.0;
     s[S_ITERS] = 0.0;
+    s[S_SEED] = (double)cv.seed;
     const bool fin = isfinite(d[0]);
     s[S_ACTIVE] = (!fin || sqrt(d[0]) <= cv.tol * sqrt(fn2)) ? 0.0 : 1.0;
     if (!fin) s[S_STOPPED] = 1.0;
