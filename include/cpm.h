@@ -304,8 +304,9 @@ cpm_status cpm_surface_divergence(cpm_ctx *ctx, const double *X_dev, double *b_d
  * added to x in FP64; whenever a right-hand side's FP32 residual has fallen by
  * inner_tol, the FP64 residual r = f - A x restarts its inner solve in a fresh
  * Krylov space (random shadow residual), and the right-hand side stops once r
- * meets tol.  One whose FP64 residual stops falling is finished by FP64
- * BiCGSTAB from its current iterate, so the result always meets tol in FP64.
+ * meets tol.  One whose FP64 residual stops falling, and the last sixteenth of a
+ * batch, is finished by FP64 BiCGSTAB from its current iterate (at most half of
+ * the columns: those alone), so the result always meets tol in FP64.
  * All right-hand sides of a batch iterate together with their own scalars; every dot product is reduced on the device in a fixed
  * order (results do not depend on scheduling), and groups of check_every
  * iterations are replayed from a captured CUDA graph on the context's internal
@@ -353,11 +354,12 @@ cpm_status cpm_profile(cpm_ctx *ctx, int enable, double *apply_ms, int64_t *appl
 
 /* Launch shapes chosen by cpm_autotune. */
 typedef struct {
-  int cells_xh;              /* x passes of the batched cell gather (0: the batch width does not use it) */
+  int cells_xh;              /* x passes an earlier batched cell gather took: checked and reported, without
+                              * effect on the present one (0: the batch width has none) */
   int cells_blocks_per_sm;   /* grid cap of the cell gather, blocks of 8 warps per SM (0: default 16) */
   int combine_warps_per_sm;  /* grid cap of the warp-per-row combine (0: default 64) */
   int vec_blocks_per_sm;     /* blocks of 512 threads per SM of the Krylov vector kernels (1, 2 or 4) */
-  int single_mode;           /* single right-hand side product: 0 = per-cell gather then combine (default),
+  int single_mode;           /* single right-hand side product: 0 = gather by tiles of cells then combine (default),
                               * 1 = per-row gather then combine, 2 = fused persistent kernel (its bounded
                               * waits set a device flag if they give up, which the next solve reports
                               * as CPM_ERR_TIMEOUT) */

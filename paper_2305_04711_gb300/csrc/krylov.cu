@@ -347,6 +347,14 @@ __global__ void add_kernel(int64_t N, int nrhs, int64_t ld, const double *s, con
   }
 }
 
+// columns cols[0..k) of src ([N][ld]) to dst ([N][k]), or back
+__global__ void take_columns_kernel(int64_t N, int k, int64_t ld, const double *cols, const double *src, double *dst) {
+  CPM_ROWS_COLS_LOOP(N, k, i, c) dst[i * k + c] = src[i * ld + (int)cols[c]];
+}
+__global__ void put_columns_kernel(int64_t N, int k, int64_t ld, const double *cols, const double *src, double *dst) {
+  CPM_ROWS_COLS_LOOP(N, k, i, c) dst[i * ld + (int)cols[c]] = src[i * k + c];
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -716,6 +724,12 @@ cpm_status ir_refine(cpm_ctx *c, ApplyFn<double> ap64, const Op<float> &op32, do
       if (rc) return rc;
     }
     bool any = false;
+    int left = 0;
+    for (int q = 0; q < nrhs; ++q) left += !done_col(rn2[q], fn2[q], tol, floors[q]);
+    // a sixteenth of the batch or less: an FP64 solve of these columns alone is
+    // cheaper than another FP32 step of all (sphere h = 1/128: an FP64 iteration of
+    // one column 0.49 ms, an FP32 iteration of 64 3.9 ms)
+    if (nrep > 0 && left * 16 <= nrhs) break;
     for (int q = 0; q < nrhs; ++q) {
       flag[q] = 0.0;
       if (done_col(rn2[q], fn2[q], tol, floors[q])) continue;
@@ -840,6 +854,14 @@ cpm_status fp64_passes(cpm_ctx *c, ApplyFn<double> ap64, bool left, double dS, d
   return CPM_OK;
 }
 
+// blocks of the vector kernels: no more than have a row to work on, since the last
+// one sums all their partials
+int vector_blocks(const cpm_ctx *c, int64_t N, int nrhs) {
+  const int bps = (c->tune.vec_blocks_per_sm >= 1 && c->tune.vec_blocks_per_sm <= 4) ? c->tune.vec_blocks_per_sm : 2;
+  const int64_t rows_per = KT / nrhs > 0 ? KT / nrhs : 1;
+  return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->nsm * bps, (N + rows_per - 1) / rows_per));
+}
+
 cpm_status solve_impl(cpm_ctx *c, bool adjoint, double m, double n, const double *f, double *x, int nrhs,
                       int64_t ld, const cpm_solve_opts *o, cpm_solve_stats *stats, cudaStream_t st) {
   cpm_solve_opts opts{1e-10, 10000, CPM_SOLVE_FP64, 1e-1, 200, 16, CPM_NORM_PLAIN, 1000};
@@ -872,12 +894,9 @@ cpm_status solve_impl(cpm_ctx *c, bool adjoint, double m, double n, const double
   // always iterates right-preconditioned, A^T W mu = g with lambda = W mu: this
   // is the transpose of the row-scaled forward system, whereas scaling the rows
   // of A^T leaves the BC rows with O(1/h^2) couplings and BiCGSTAB breaks down.
-  const bool left = scaled && !adjoint;
+  const bool left_scaled = scaled && !adjoint;
   CPM_CUDA_TRY(cudaMemsetAsync(w->ticket, 0, sizeof(unsigned), st));
-  // no more blocks than have a row to work on: the last one sums all their partials
-  const int bps = (c->tune.vec_blocks_per_sm >= 1 && c->tune.vec_blocks_per_sm <= 4) ? c->tune.vec_blocks_per_sm : 2;
-  const int64_t rows_per = KT / nrhs > 0 ? KT / nrhs : 1;
-  w->G = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)c->nsm * bps, (N + rows_per - 1) / rows_per));
+  w->G = vector_blocks(c, N, nrhs);
   // the initial residual: a right-hand side (or guess) that is not finite is
   // rejected before any iteration
   rc = residual64(c, ap64, m, n, f, x, w, nrhs, ld, wrow, rn2, fn2, st);
@@ -892,7 +911,7 @@ cpm_status solve_impl(cpm_ctx *c, bool adjoint, double m, double n, const double
       return CPM_ERR_ARG;
     }
   if (opts.mode == CPM_SOLVE_FP64) {
-    rc = fp64_passes(c, ap64, left, dS, m, n, f, x, w, nrhs, ld, wrow, opts.tol, opts.maxit, opts.check_every, &iters,
+    rc = fp64_passes(c, ap64, left_scaled, dS, m, n, f, x, w, nrhs, ld, wrow, opts.tol, opts.maxit, opts.check_every, &iters,
                      &restarts, &broke, rn2, fn2, floors, st);
     if (rc) return rc;
     iters64 = iters;
@@ -906,16 +925,44 @@ cpm_status solve_impl(cpm_ctx *c, bool adjoint, double m, double n, const double
                      opts.maxit, opts.max_refine, opts.check_every, trace, &iters, &refinements, &restarts, rn2, fn2,
                      floors, st);
     if (rc) return rc;
-    bool all = true;
-    for (int q = 0; q < nrhs; ++q) all = all && done_col(rn2[q], fn2[q], opts.tol, floors[q]);
-    if (!all && iters < opts.maxit) {
-      // FP64 finish from the current iterate for the columns the FP32 phase
-      // left above tol
-      if (trace) std::fprintf(stderr, "[cpm] FP64 finish from relres %.3e\n", worst_relres(rn2, fn2));
+    std::vector<double> left;
+    for (int q = 0; q < nrhs; ++q)
+      if (!done_col(rn2[q], fn2[q], opts.tol, floors[q])) left.push_back((double)q);
+    const int k = (int)left.size();
+    if (k > 0 && iters < opts.maxit) {
+      // FP64 finish from the current iterate for the columns the FP32 phase left
+      // above tol: those alone, side by side in the FP32 vectors' memory, where they
+      // are at most half of the batch
+      if (trace) std::fprintf(stderr, "[cpm] FP64 finish of %d columns from relres %.3e\n", k, worst_relres(rn2, fn2));
+      const bool some = 2 * k <= nrhs && nrhs > 1;
+      const double *fk = f;
+      double *xk = x;
+      int64_t ldk = ld;
+      const unsigned g = cpm_grid(N * k, 256);
+      if (some) {
+        double *fc = reinterpret_cast<double *>(w->v32[0]), *xc = reinterpret_cast<double *>(w->v32[1]);
+        CPM_CUDA_TRY(cudaMemcpyAsync(w->cols, left.data(), sizeof(double) * k, cudaMemcpyHostToDevice, st));
+        take_columns_kernel<<<g, 256, 0, st>>>(N, k, ld, w->cols, f, fc);
+        take_columns_kernel<<<g, 256, 0, st>>>(N, k, ld, w->cols, x, xc);
+        cpm_count_launches(c, 2);
+        fk = fc; xk = xc; ldk = k;
+        w->G = vector_blocks(c, N, k);
+      }
       int it64 = 0;
-      rc = fp64_passes(c, ap64, left, dS, m, n, f, x, w, nrhs, ld, wrow, opts.tol, opts.maxit - iters,
-                       opts.check_every, &it64, &restarts, &broke, rn2, fn2, floors, st);
+      std::vector<double> rk, nk, flk(some ? k : nrhs, 0.0);
+      rc = fp64_passes(c, ap64, left_scaled, dS, m, n, fk, xk, w, some ? k : nrhs, ldk, wrow, opts.tol,
+                       opts.maxit - iters, opts.check_every, &it64, &restarts, &broke, rk, nk, flk, st);
       if (rc) return rc;
+      if (some) {
+        put_columns_kernel<<<g, 256, 0, st>>>(N, k, ld, w->cols, xk, x);
+        cpm_count_launches(c, 1);
+        for (int e = 0; e < k; ++e) {
+          const int q = (int)left[e];
+          rn2[q] = rk[e]; fn2[q] = nk[e]; floors[q] = flk[e];
+        }
+      } else {
+        rn2 = rk; fn2 = nk; floors = flk;
+      }
       iters += it64;
       iters64 += it64;
     }
