@@ -151,7 +151,7 @@ struct TArgs {
 // product: the kernels then apply A^T C)
 template <typename T>
 __global__ void __launch_bounds__(256) tb_kernel(TArgs<T> A, T s, const T *__restrict__ lam, T *__restrict__ bv,
-                                                 int nrhs, int64_t ld) {
+                                                 int nrhs, int64_t ld, int64_t ldb) {
   const int nfd = 2 * A.v.dim;
   CPM_ROWS_COLS_LOOP(A.v.NS, nrhs, c, r) {
     const uint32_t rs = __ldg(A.rself + c);
@@ -167,11 +167,11 @@ __global__ void __launch_bounds__(256) tb_kernel(TArgs<T> A, T s, const T *__res
       // row i's slot in the opposite direction points back at c unless flipped
       if (__ldg(A.nbr8 + (int64_t)i * 8 + (d ^ 1)) == (int32_t)c) acc += __ldg(lam + (int64_t)i * ld + r);
     }
-    bv[c * ld + r] = s * acc;
+    bv[c * ldb + r] = s * acc;
   }
 }
 
-// ---- one right-hand side -------------------------------------------------------
+// ---- column by column -------------------------------------------------------
 // Per stencil cell the block of its E^T b contributions,
 //   blk[cz*16 + cy*4 + cx] = sum over the cell's rows of w_x[cx] w_y[cy] w_z[cz] b_row,
 // one warp per cell, two nodes per lane.  In FP64 the block is summed in integers
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(TCW * 32)
 template <typename T>
 __global__ void __launch_bounds__(256) t_rest_kernel(TArgs<T> A, const int32_t *__restrict__ cols, int64_t ncols, T s,
                                                      T rowscale, T cs, const T *__restrict__ lam,
-                                                     const T *__restrict__ bv, T *__restrict__ y) {
+                                                     const T *__restrict__ bv, T *__restrict__ y, int64_t ld) {
   const int sub = threadIdx.x & 7;
   const unsigned m = 0xFFu << (threadIdx.x & 24);
   const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
@@ -342,12 +342,12 @@ __global__ void __launch_bounds__(256) t_rest_kernel(TArgs<T> A, const int32_t *
       const int64_t src = __ldg(A.T_src + e);
       const int kind = __ldg(A.T_kind + e);
       const T w = (kind == 0) ? s * cs : __ldg(A.T_val + e);
-      acc += w * __ldg((kind == 1 ? bv : lam) + src);
+      acc += w * (kind == 1 ? __ldg(bv + src) : __ldg(lam + src * ld));
     }
     acc += __shfl_xor_sync(m, acc, 1);
     acc += __shfl_xor_sync(m, acc, 2);
     acc += __shfl_xor_sync(m, acc, 4);
-    if (sub == 0) y[j] = (j < A.v.NS) ? y[j] + rowscale * acc : acc;
+    if (sub == 0) y[j * ld] = (j < A.v.NS) ? y[j * ld] + rowscale * acc : acc;
   }
 }
 
@@ -360,7 +360,7 @@ constexpr int TYT = 256;
 template <typename T, int DIM, int NP>
 __global__ void __launch_bounds__(TYT, 5)
     ty_brick_kernel(TArgs<T> A, const void *__restrict__ blk_, const int32_t *__restrict__ bexp, T dg, T rowscale,
-                    T cs, const T *__restrict__ lam, T *__restrict__ y) {
+                    T cs, const T *__restrict__ lam, T *__restrict__ y, int64_t ld) {
   constexpr int H = 7 + NP, HZ = (DIM == 3) ? H : 1;  // NP - 1 before, 8 of the brick
   constexpr int NZ = (DIM == 3) ? NP : 1;
   constexpr int SLOTS = (DIM == 3) ? 64 : 16;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(TYT, 5)
       constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
       if (top != E_NONE) sum = scaled_sum(fx_scale(back, top), acc, plain ? sum : 0.0);
     }
-    y[j] = rowscale * (sum + (dg * cs) * __ldg(lam + j));
+    y[j * ld] = rowscale * (sum + (dg * cs) * __ldg(lam + j * ld));
   }
 }
 
@@ -590,36 +590,51 @@ cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowsc
   const T s = T(n * inv_h2), dg = T(m + n * (-2.0 * c->dim * inv_h2));
   const int64_t N = c->NS + c->NC;
   cpm_prof_begin(c, st);
-  tb_kernel<T><<<cpm_grid(c->NS * nrhs, 256), 256, 0, st>>>(A, T(s * T(colscale)), u, bv, nrhs, ld);
-  int launched = 2;
-  if (nrhs == 1 && ld == 1 && c->d_tblk && c->ncells > 0) {
-    // one right-hand side: per-cell blocks of E^T b (reserved at set-up), then the nodes by bricks
+  int launched = 0;
+  // One column, or a few of a 3D band, one by one: per-cell blocks of E^T b (one
+  // column's are reserved at set-up), then the nodes by bricks.  All columns at once
+  // revisit every row of a node's 64 cells but share the walk: sphere h = 1/100
+  // (1.04M rows), one by one / at once, FP64: 3 columns 0.97 / 5.9 ms, 16 columns 5.6 /
+  // 10.1; FP32: 3 columns 0.54 / 1.48 ms, 16 columns 3.1 / 3.6; at h = 1/64 with 64
+  // columns 11.5 / 10.6 and 7.7 / 4.5 ms, at h = 1/32 4.5 / 2.7 and 3.0 / 1.2 ms, and a
+  // small band pays four launches a column.
+  const bool by_column = c->d_tblk && c->ncells > 0 &&
+                         (nrhs == 1 || (c->dim == 3 && (sizeof(T) == 8 ? nrhs <= 8 && c->NS >= 25000
+                                                                       : nrhs <= 4 && c->NS >= 100000)));
+  if (by_column) {
     TCellArgs C{c->d_cell_start, c->d_cell_rows, c->ncells, c->d_tc64, c->d_tc32};
     int32_t *bexp = reinterpret_cast<int32_t *>(c->d_tblk + 64 * c->ncells);
     const unsigned gc = (unsigned)std::min<int64_t>((c->ncells + TCW - 1) / TCW, (int64_t)c->nsm * 64);
-#define CPM_TCELL(D, NP)                                                                                           \
-  do {                                                                                                             \
-    if constexpr (sizeof(T) == 8)                                                                                  \
-      tcell_fx_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<long long *>(c->d_tblk), bexp);      \
-    else                                                                                                           \
-      tcell_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<float *>(c->d_tblk));                   \
-    ty_brick_kernel<T, D, NP><<<(unsigned)c->nb, TYT, 0, st>>>(A, c->d_tblk, bexp, dg, T(rowscale), T(colscale), u, \
-                                                               v);                                                 \
+    for (int r = 0; r < nrhs; ++r) {
+      const T *ur = u + r;
+      T *vr = v + r;
+      tb_kernel<T><<<cpm_grid(c->NS, 256), 256, 0, st>>>(A, T(s * T(colscale)), ur, bv, 1, ld, 1);
+#define CPM_TCELL(D, NP)                                                                                             \
+  do {                                                                                                               \
+    if constexpr (sizeof(T) == 8)                                                                                    \
+      tcell_fx_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<long long *>(c->d_tblk), bexp);        \
+    else                                                                                                             \
+      tcell_kernel<D, NP><<<gc, TCW * 32, 0, st>>>(C, bv, reinterpret_cast<float *>(c->d_tblk));                     \
+    ty_brick_kernel<T, D, NP><<<(unsigned)c->nb, TYT, 0, st>>>(A, c->d_tblk, bexp, dg, T(rowscale), T(colscale), ur, \
+                                                               vr, ld);                                              \
   } while (0)
-    if (c->dim == 3) {
-      if (c->p == 2) CPM_TCELL(3, 3); else CPM_TCELL(3, 4);
-    } else {
-      if (c->p == 2) CPM_TCELL(2, 3); else CPM_TCELL(2, 4);
-    }
+      if (c->dim == 3) {
+        if (c->p == 2) CPM_TCELL(3, 3); else CPM_TCELL(3, 4);
+      } else {
+        if (c->p == 2) CPM_TCELL(2, 3); else CPM_TCELL(2, 4);
+      }
 #undef CPM_TCELL
-    ++launched;
-    if (c->nTcols > 0) {
-      t_rest_kernel<T><<<cpm_grid(8 * c->nTcols, 256), 256, 0, st>>>(A, c->d_T_cols, c->nTcols, s, T(rowscale),
-                                                                     T(colscale), u, bv, v);
-      ++launched;
+      launched += 3;
+      if (c->nTcols > 0) {
+        t_rest_kernel<T><<<cpm_grid(8 * c->nTcols, 256), 256, 0, st>>>(A, c->d_T_cols, c->nTcols, s, T(rowscale),
+                                                                       T(colscale), ur, bv, vr, ld);
+        ++launched;
+      }
     }
   } else {
+    tb_kernel<T><<<cpm_grid(c->NS * nrhs, 256), 256, 0, st>>>(A, T(s * T(colscale)), u, bv, nrhs, ld, ld);
     ty_kernel<T><<<cpm_grid(N * nrhs, 256), 256, 0, st>>>(A, dg, s, T(rowscale), T(colscale), u, bv, v, nrhs, ld);
+    launched = 2;
   }
   cpm_prof_end(c, st, c->NS * (int64_t)nrhs);
   cpm_count_launches(c, launched);

@@ -41,6 +41,24 @@ def test_transpose_matches_oracle(oracle_mod, name, p):
         assert np.max(np.abs(ys - yr * scale)) <= 1e-14 * top * scale
 
 
+def test_columns_one_by_one_and_at_once_agree(oracle_mod):
+    """Both sides of the rules on the number of columns, strided columns included."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.config2(1 / 32, ci.BC_DIR2)
+    band = Band(w.shape, w.h).set_boundary(w.curves)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(2)
+    U = torch.randn((band.N, 9), generator=gen, dtype=torch.float64, device="cuda")
+    one = torch.stack([band.apply(0.0, 1.0, U[:, r].contiguous(), transpose=True) for r in range(9)], 1)
+    top = float(one.abs().max())
+    for nrhs in (2, 4, 5, 8, 9):
+        V = band.apply(0.0, 1.0, U[:, :nrhs].contiguous(), transpose=True)
+        assert float((V - one[:, :nrhs]).abs().max()) <= 1e-14 * top
+        V32 = band.apply(0.0, 1.0, U[:, :nrhs].float().contiguous(), transpose=True)
+        assert float((V32.double() - one[:, :nrhs]).abs().max()) <= 2e-6 * top
+
+
 def test_an_infinity_stays_in_its_columns(oracle_mod):
     torch = need_gpu()
     band, ref = _pair(oracle_mod, "sphere_closed", 3)
