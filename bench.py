@@ -384,7 +384,7 @@ def apply_bandwidth(h, hbm, peak_src, log):
         out[key] = {"ms": tms, "GB/s_algorithmic": gbs, "hbm_peak_GB/s": hbm, "frac": gbs / hbm,
                     "peak_source": peak_src, "bytes_per_row": bytes_row,
                     "launches_per_product": p["launches"] / max(p["applies"], 1),
-                    "single_mode": {0: "per-cell gather + combine", 1: "per-row gather + combine",
+                    "single_mode": {0: "gather by tiles of cells + combine", 1: "per-row gather + combine",
                                     2: "fused"}[tune["single_mode"]]}
         if key == "fp64":
             out[key]["TFLOP/s"] = FLOPS_ROW_FP64 * band.NS / (tms * 1e-3) / 1e12

@@ -1,17 +1,15 @@
 // tune.cu -- the launch-shape autotuner.
 //
-// The batched product's cell gather keeps a cell's node values in registers
-// for x passes of the stencil (more passes: fewer registers and more warps per
-// SM, but more weight loads and partial sums through shared memory); its grid,
-// the warp-per-row combine's grid and the Krylov vector kernels' blocks per SM
-// trade occupancy against tail effects.  Which is fastest depends on the band
-// (cells per brick, rows per cell), the batch width and the precision, so the
-// tuner times each candidate on the context's own band with the caller's batch
-// layout, by coordinate descent (passes, then the gather grid, then the
-// combine grid, then the vector kernels), and keeps the fastest in the
-// context.  Every candidate computes the same product; only the vector
-// kernels' reduction grouping changes with their block count (each choice is
-// deterministic).
+// The grids of the batched cell gather and of the warp-per-row combine and the
+// Krylov vector kernels' blocks per SM trade occupancy against tail effects.
+// Which is fastest depends on the band (cells per brick, rows per cell), the batch
+// width and the precision, so the tuner times each candidate on the context's own
+// band with the caller's batch layout, by coordinate descent (the gather grid, then
+// the combine grid, then the vector kernels), and keeps the fastest in the context.
+// The x passes that an earlier cell gather took are still accepted and reported, so
+// that recorded shapes stay valid; they choose nothing now.  Every candidate computes
+// the same product; only the vector kernels' reduction grouping changes with their
+// block count (each choice is deterministic).
 #include <algorithm>
 #include <vector>
 
