@@ -1,10 +1,10 @@
 // tile.cu -- E u for one or a few right-hand sides: warp tiles of stencil cells.
 //
-// A warp takes CT consecutive cells (cells.cu) and stages the differences of
-// their node values to each cell's base-node value in shared memory, then its
+// A warp takes CT consecutive cells (cells.cu) and stages their node values in
+// shared memory (FP64: as differences to each cell's base-node value u_c), then its
 // lanes take the tile's rows (~5 per cell, in cell order), one row each: the
 // weights of the row, the separable sum over the cell's nodes from shared
-// memory, and a_i = sum_j w_j (u_j - u_c) + (u_c - u_i).  Rows, not cells, are
+// memory, and a_i = sum_j w_j (u_j - u_i), in FP64 from sum_j w_j (u_j - u_c) + (u_c - u_i).  Rows, not cells, are
 // spread over the lanes because cells hold between 1 and a dozen rows: one
 // thread per cell left a warp waiting for its fullest cell, and 64 FP64 node
 // values per thread left 2 blocks of 128 threads per SM.  The staging loads
@@ -37,8 +37,10 @@ struct TileArgs {
 // FP64, sphere h = 1/128 (1.70M rows, 309k cells): 140 us (one thread per cell in
 // FP64 arithmetic: 820 us), with the multiply-add pipe busy 55 % and the integer
 // pipe 46 %; what is left is the latency of the staging loads at 24 warps per SM,
-// which is why they are unrolled over 8 cells.  FP32, bumpy sphere h = 1/320
-// (10.7M rows): 250 us (272 us), held by L1 wavefronts (74 %).
+// which is why they are unrolled over 8 cells.  FP32 keeps the node values as they are
+// and takes the differences to u_i per row (one rounding less, and no base value to
+// pass on: the product on the bumpy sphere at h = 1/640, 43M rows, 1335 -> 1192 us); it
+// is held by L1 wavefronts (74 %).
 template <typename T, bool DIFF, int DIM, int NP, int CT>
 __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
     gather_tile_kernel(TileArgs A, const T *__restrict__ tc, T cs, const T *__restrict__ u, T *__restrict__ a,
@@ -60,7 +62,7 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
   const int32_t q0 = __ldg(A.cstart + c0), q1 = __ldg(A.cstart + c0 + nc);
   for (int r = 0; r < nrhs; ++r) {
     const T *ur = u + r;
-    // ---- stage the tile's node values as differences to each cell's base node
+    // ---- stage the tile's node values
 #pragma unroll(FX ? 8 : 4)
     for (int cb = 0; cb < nc; cb += CPI) {
       const int sub = (CPI > 1) ? lane / SLOTS : 0;
@@ -128,9 +130,8 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
           const int slot = (CPI > 1) ? (lane & (SLOTS - 1)) : lane + 32 * k;
-          if (live && slot < SLOTS) s_d[w][c][slot] = d[k];
+          if (live && slot < SLOTS) s_d[w][c][slot] = v[k];  // (differences to u_i are taken per row)
         }
-        if (live && (lane & (SLOTS - 1 < 31 ? SLOTS - 1 : 31)) == 0) s_uc[w][c] = uc;
       }
     }
     __syncwarp();
@@ -139,10 +140,10 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
       const int64_t row = __ldg(A.crows + q);
       const int c = (int)(__ldg(A.row_cell + q) - c0);
       const T *tq = tc + 3 * (int64_t)q;
-      const T uc = s_uc[w][c];
       const T ui = DIFF ? __ldg(ur + row * ld) : T(0);
       T acc;
       if constexpr (FX) {
+        const T uc = s_uc[w][c];
         int32_t wxh[4], wxl[4], wyh[4], wyl[4], wzh[4], wzl[4];
         fixed_weights<NP>(__ldg(tq), wxh, wxl);
         fixed_weights<NP>(__ldg(tq + 1), wyh, wyl);
@@ -190,20 +191,20 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
         else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
         const float4 *dn = reinterpret_cast<const float4 *>(&s_d[w][c][0]);
         float2 p01 = make_float2(0.0f, 0.0f), p23 = p01;
+        const float2 mu = make_float2(-ui, -ui);
 #pragma unroll
         for (int cz = 0; cz < NZ; ++cz)
 #pragma unroll
           for (int cy = 0; cy < NP; ++cy) {
             const float g = wy[cy] * wz[cz];
             const float4 p = dn[cz * 4 + cy];
-            p01 = __ffma2_rn(make_float2(g, g), make_float2(p.x, p.y), p01);
-            p23 = __ffma2_rn(make_float2(g, g), make_float2(p.z, p.w), p23);
+            p01 = __ffma2_rn(make_float2(g, g), __fadd2_rn(make_float2(p.x, p.y), mu), p01);
+            p23 = __ffma2_rn(make_float2(g, g), __fadd2_rn(make_float2(p.z, p.w), mu), p23);
           }
         acc = wx[0] * p01.x;
         acc += wx[1] * p01.y;
         acc += wx[2] * p23.x;
         if (NP == 4) acc += wx[3] * p23.y;
-        acc += DIFF ? uc - ui : uc;
       }
       if (cs != T(1)) acc *= cs;
       a[row * ld + r] = acc;
