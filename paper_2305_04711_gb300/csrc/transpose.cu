@@ -210,9 +210,11 @@ __global__ void __launch_bounds__(TCW * 32)
     for (int32_t q = r0 + lane; q < r1; q += 32) top = max(top, fx_key(__ldg(bv + __ldg(A.crows + q))));
     top = __reduce_max_sync(0xffffffffu, top);
     const int em = (int)(top >> 20);
-    // an axis multiplies by 6 / 16, so a row adds less than 2^56.8 to a sum; more
-    // than 64 rows take fewer bits each
-    const int K = 8 - max(0, 32 - __clz((r1 - r0 - 1) >> 6));
+    // |b| < 2^61 and an axis multiplies by at most 6 / 16 (|w| <= 1), so a row adds less
+    // than 2^58.2 (2D) or 2^56.8 (3D) to a sum: 16 or 64 rows of one sign stay below
+    // 2^62.9 in 64 bits, and every doubling of the rows takes a bit from the operands
+    constexpr int FULL = (DIM == 3) ? 6 : 4;
+    const int K = 8 - max(0, 32 - __clz((r1 - r0 - 1) >> FULL));
     // (the exponent limits leave room for the scale factors of the node gather)
     const bool ok = top == 0u || (em >= 300 && em < 2040 && K >= 0);
     long long a0 = 0, a1 = 0;

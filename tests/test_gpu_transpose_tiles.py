@@ -91,3 +91,23 @@ def test_cells_with_many_rows():
     b = float(torch.dot(u, band.apply(0.0, 1.0, v, transpose=True)))
     # rounding of the two products, each entry of size <= 8/h^2 * 3 per unit of u
     assert abs(a - b) <= 1e-13 * band.N * 24 / 0.05 ** 2
+
+
+@pytest.mark.parametrize("p", [3, 2])
+@pytest.mark.parametrize("shape, h, r_band", [("circle", 0.0451, 0.7), ("circle", 0.05, 1.0), ("circle", 0.05, 3.0),
+                                              ("sphere", 0.25, 3.0)])
+def test_wide_bands_with_values_of_one_sign(oracle_mod, shape, h, r_band, p):
+    """40 to 200 rows share a cell and all add up: the sums come as close to their integer limits as a
+    field can bring them.  The reference adds the assembled entries up in extended precision."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    sh = ci.circle2d() if shape == "circle" else ci.sphere()
+    band = Band(sh, h, r_band=r_band, p=p).set_boundary([])
+    ref = oracle_mod.Oracle(sh, h, rband=r_band, p=p).set_curves([])
+    A = sp.csc_matrix(ref.A(0.0, 1.0))
+    gen = np.random.default_rng(3)
+    for lam in (np.ones(ref.N), np.full(ref.N, -1.99), gen.uniform(1.0, 2.0, ref.N)):
+        terms = A.data.astype(np.longdouble) * lam[A.indices]
+        yr = np.array([terms[a:b].sum() for a, b in zip(A.indptr[:-1], A.indptr[1:])])
+        y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda"), transpose=True).cpu().numpy()
+        assert np.max(np.abs(y - yr)) <= 1e-14 * np.max(np.abs(yr))
