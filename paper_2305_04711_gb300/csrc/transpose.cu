@@ -189,7 +189,7 @@ struct TCellArgs {
   const int32_t *cstart, *crows;
   int64_t ncells;
   const double *tc64;
-  const float *tc32;
+  const float *w1d32;
 };
 
 template <int DIM, int NP>
@@ -303,13 +303,15 @@ __global__ void __launch_bounds__(TCW * 32)
     float a0 = 0.0f, a1 = 0.0f;
     for (int32_t c0 = r0; c0 < r1; c0 += TCR) {
       const int k = min(TCR, r1 - c0);
+      // (weights formed in FP64 and rounded once, as the batches take them: formed from
+      // a fraction rounded to FP32, those near zero lose their relative accuracy)
+      const int64_t row = (j0 < k) ? __ldg(A.crows + c0 + j0) : 0;
       if (ax < 3) {
-        float wt[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (ax < DIM && j0 < k) cpm_lagrange<NP, float>(__ldg(A.tc32 + 3 * (int64_t)(c0 + j0) + ax), wt);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) s_w[w][j0][ax][q] = (q < NP) ? wt[q] : 0.0f;
+        float4 wt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (j0 < k) wt = __ldg(reinterpret_cast<const float4 *>(A.w1d32 + row * 12 + 4 * ax));
+        *reinterpret_cast<float4 *>(s_w[w][j0][ax]) = wt;
       } else if (j0 < k) {
-        s_b[w][j0] = __ldg(bv + __ldg(A.crows + c0 + j0));
+        s_b[w][j0] = __ldg(bv + row);
       }
       __syncwarp();
       for (int j = 0; j < k; ++j) {
@@ -405,7 +407,9 @@ __global__ void __launch_bounds__(TYT, 5)
           }
           if (yes) have |= 1ull << (cz * 16 + cy * 4 + cx);
         }
-    T sum = T(0);
+    // (FP32 starts from the diagonal, which the blocks mostly cancel: partial sums, and
+    // with them the rounding, shrink on the way)
+    T sum = FX ? T(0) : (dg * cs) * __ldg(lam + (int64_t)j * ld);
     long long acc = 0;
     while (have) {
       int slot[4], e[4];
@@ -447,8 +451,9 @@ __global__ void __launch_bounds__(TYT, 5)
     if constexpr (FX) {
       constexpr double back = (DIM == 3) ? 4096.0 / 216.0 : 256.0 / 36.0;  // every axis multiplied by 6 / 16
       if (top != E_NONE) sum = scaled_sum(fx_scale(back, top), acc, plain ? sum : 0.0);
+      sum += (dg * cs) * __ldg(lam + j * ld);
     }
-    y[j * ld] = rowscale * (sum + (dg * cs) * __ldg(lam + j * ld));
+    y[j * ld] = rowscale * sum;
   }
 }
 
@@ -604,7 +609,7 @@ cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowsc
                          (nrhs == 1 || (c->dim == 3 && (sizeof(T) == 8 ? nrhs <= 8 && c->NS >= 25000
                                                                        : nrhs <= 4 && c->NS >= 100000)));
   if (by_column) {
-    TCellArgs C{c->d_cell_start, c->d_cell_rows, c->ncells, c->d_tc64, c->d_tc32};
+    TCellArgs C{c->d_cell_start, c->d_cell_rows, c->ncells, c->d_tc64, c->d_w1d32};
     int32_t *bexp = reinterpret_cast<int32_t *>(c->d_tblk + 64 * c->ncells);
     const unsigned gc = (unsigned)std::min<int64_t>((c->ncells + TCW - 1) / TCW, (int64_t)c->nsm * 64);
     for (int r = 0; r < nrhs; ++r) {

@@ -111,3 +111,22 @@ def test_wide_bands_with_values_of_one_sign(oracle_mod, shape, h, r_band, p):
         yr = np.array([terms[a:b].sum() for a, b in zip(A.indptr[:-1], A.indptr[1:])])
         y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda"), transpose=True).cpu().numpy()
         assert np.max(np.abs(y - yr)) <= 1e-14 * np.max(np.abs(yr))
+
+
+@pytest.mark.parametrize("name", ["circle_dir1", "sphere_closed"])
+@pytest.mark.parametrize("p", [3, 2])
+def test_fp32_weights_keep_their_relative_accuracy(oracle_mod, name, p):
+    """Single rows of A in FP32, entry by entry: a term rounds three weights, b twice, three products, at
+    most six additions in its cell and six at its node, the diagonal and its scale: 24 roundings of 2^-24 of the
+    terms' sizes (and 1e-14 of the largest for the FP64 weights themselves).  A weight near zero formed from a fraction rounded to FP32 is off by far more than its own 2^-24."""
+    torch = need_gpu()
+    band, ref = _pair(oracle_mod, name, p)
+    A = sp.csr_matrix(ref.A(0.0, 1.0))
+    size = abs(ref.Loff)[:, :ref.NS] @ abs(ref.E) + sp.eye(ref.NS, ref.N, format="csr") * abs(ref.diagL())
+    far = np.flatnonzero(ref.near_c < 0)
+    for i in far[:: len(far) // 24]:
+        lam = np.zeros(ref.N)
+        lam[i] = 1.0
+        y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda").float(), transpose=True).cpu().numpy()
+        err = np.abs(y - A[i].toarray()[0])
+        assert np.all(err <= 24 * 2.0 ** -24 * size[i].toarray()[0] + 1e-14 * size[i].max())
