@@ -190,17 +190,23 @@ __global__ void __launch_bounds__(TW * 32, (sizeof(T) == 8) ? 6 : 8)
         if (DIM == 3) cpm_lagrange<NP, T>(__ldg(tq + 2), wz);
         else { wz[0] = T(1); wz[1] = wz[2] = wz[3] = T(0); }
         const float4 *dn = reinterpret_cast<const float4 *>(&s_d[w][c][0]);
+        // (axis by axis: with products w_y w_z as weights every term took one rounding more)
         float2 p01 = make_float2(0.0f, 0.0f), p23 = p01;
         const float2 mu = make_float2(-ui, -ui);
 #pragma unroll
-        for (int cz = 0; cz < NZ; ++cz)
+        for (int cz = 0; cz < NZ; ++cz) {
+          float2 q01 = make_float2(0.0f, 0.0f), q23 = q01;
 #pragma unroll
           for (int cy = 0; cy < NP; ++cy) {
-            const float g = wy[cy] * wz[cz];
+            const float2 g = make_float2(wy[cy], wy[cy]);
             const float4 p = dn[cz * 4 + cy];
-            p01 = __ffma2_rn(make_float2(g, g), __fadd2_rn(make_float2(p.x, p.y), mu), p01);
-            p23 = __ffma2_rn(make_float2(g, g), __fadd2_rn(make_float2(p.z, p.w), mu), p23);
+            q01 = __ffma2_rn(g, __fadd2_rn(make_float2(p.x, p.y), mu), q01);
+            q23 = __ffma2_rn(g, __fadd2_rn(make_float2(p.z, p.w), mu), q23);
           }
+          const float2 g = make_float2(wz[cz], wz[cz]);
+          p01 = (DIM == 3) ? __ffma2_rn(g, q01, p01) : q01;
+          p23 = (DIM == 3) ? __ffma2_rn(g, q23, p23) : q23;
+        }
         acc = wx[0] * p01.x;
         acc += wx[1] * p01.y;
         acc += wx[2] * p23.x;
