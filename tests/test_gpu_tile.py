@@ -113,3 +113,22 @@ def test_fp32_gather_takes_no_products_of_weights():
         band.set_tune(1, torch.float32, single_mode=mode)
         err.append(float((band.apply(0.0, 1.0, u).double() - v).norm() / v.norm()))
     assert err[0] <= 0.97 * err[1], err
+
+
+def test_fp32_of_smooth_columns_rounds_alike_in_every_width():
+    """A smooth field's rounding is relative to local differences in every width: to u_i for a column alone (0.106
+    of the result's own size in a model of random cells with linear fields), to a value from the middle of the
+    stencil in batches (0.126; 0.35 to the stencil's first node).  The bar is a quarter above equality."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    band = Band(ci.sphere(), 1 / 12).set_boundary([])
+    _, cp = band.export_band()
+    gen = np.random.default_rng(6)
+    U = torch.sin(cp @ torch.tensor(gen.normal(size=(3, 130)), device="cuda")
+                  + torch.tensor(gen.uniform(0, 6, 130), device="cuda")).float()
+    V = band.apply(0.0, 1.0, U[:, :8].double().contiguous())
+    alone = torch.stack([band.apply(0.0, 1.0, U[:, r].contiguous()) for r in range(8)], 1)
+    e1 = float((alone.double() - V).norm())
+    for nrhs in (8, 16, 33, 64, 65, 66, 130):
+        en = float((band.apply(0.0, 1.0, U[:, :nrhs].contiguous())[:, :8].double() - V).norm())
+        assert en <= 1.25 * e1, (nrhs, en, e1)
