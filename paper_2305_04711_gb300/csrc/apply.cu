@@ -161,6 +161,51 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 8) ? 6 : 8)
   CPM_ROWS_COLS_LOOP(A.N, nrhs, i, r) v[i * ld + r] = combine_element<T>(A, S, bc_val, u, a, i, r, ld);
 }
 
+// ---- gather of small 2D batches -------------------------------------------------
+// a_i = cs (E u - u)_i with one thread per row and column, flipped entries included (the
+// rows near curves read their explicit stencils): one launch where tiles or cells of
+// rows and the flipped entries take two.
+template <int NP>
+__global__ void __launch_bounds__(256) gather_rows2d_kernel(ApplyArgs<float> A, float cs, const float *__restrict__ u,
+                                                            float *__restrict__ a, int nrhs, int64_t ld) {
+  const int64_t NS = A.v.NS;
+  CPM_ROWS_COLS_LOOP(NS, nrhs, i, r) {
+    const uint32_t rb = __ldg(A.rbase + i);
+    const float ui = __ldg(u + i * ld + r);
+    float acc = 0.0f;
+    if (rb & CPM_SPECIAL_BIT) {
+      const int64_t s = __ldg(A.spec_of + i);
+      for (int e = 0; e < 16; ++e) {  // (the 4 x 4 entries of a 2D stencil; absent ones are -1)
+        const int32_t c = __ldg(A.ecol + s * 64 + e);
+        if (c < 0) continue;
+        const float val = __ldg(u + (int64_t)c * ld + r) * ((c < NS) ? cs : 1.0f);
+        acc += __ldg(A.ew + s * 64 + e) * (val - cs * ui);
+      }
+    } else {
+      const int32_t b = (int32_t)(rb >> 9);
+      const int l = (int)(rb & 511u), lx = l & 7, ly = (l >> 3) & 7;
+      const int split = (lx + NP - 1 < 8) ? NP : 8 - lx;
+      float wx[4], wy[4];
+      cpm_lagrange<NP, float>(__ldg(A.t + 3 * i), wx);
+      cpm_lagrange<NP, float>(__ldg(A.t + 3 * i + 1), wy);
+#pragma unroll
+      for (int cy = 0; cy < NP; ++cy) {
+        int32_t s0, s1;
+        if (!cpm_line_start<NP>(A.v, b, lx, ly, 0, cy, 0, s0, s1)) continue;  // (set-up excludes it)
+        float line = 0.0f;
+#pragma unroll
+        for (int cx = 0; cx < NP; ++cx) {
+          const int32_t j = (cx < split) ? s0 + cx : s1 + (cx - split);
+          line += wx[cx] * (__ldg(u + (int64_t)j * ld + r) - ui);
+        }
+        acc += wy[cy] * line;
+      }
+      acc *= cs;
+    }
+    a[i * ld + r] = acc;
+  }
+}
+
 // one column with the iteration's dot products of v: (w, v), or (v, u) and (v, v)
 // (STAGE); reading v back for them was a launch and a pass over two vectors
 template <typename T, int STAGE>
@@ -468,6 +513,23 @@ static int launch_product(cpm_ctx *c, T m, T n, T rowscale, T cs, const T *u, T 
   // columns per lane need an even column count and 2-element alignment
   const bool aligned2 = (ld % 2 == 0) && ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v) |
                                            reinterpret_cast<uintptr_t>(a)) % (2 * sizeof(T)) == 0);
+  if constexpr (sizeof(T) == 4) {
+    // Small 2D batches are bound by their launches: below a quarter (16 columns on: half)
+    // of a million elements a thread per row and column takes two of them where tiles or
+    // cells take three (circle, cubic, us a product, rows / tiles or cells: h = 0.01,
+    // 2 columns 10.3 / 12.3, 15 columns 12.3 / 20.6, 33 15.3 / 26.7, 65 18.5 / 31.3; h = 0.001,
+    // 5 columns 18.6 / 19.6, 8 columns, above the line, 23.6 / 18.5).  Widths that fill the
+    // warps of the cell gather evenly stay there (16 columns 16.5 / 14.4).
+    const bool even_batch = nrhs >= 16 && (nrhs <= 32 || (nrhs <= 64 && nrhs % 2 == 0 && aligned2));
+    if (c->dim == 2 && nrhs > 1 && !even_batch && c->NS * nrhs <= (nrhs < 16 ? 262144 : 524288)) {
+      const ApplyArgs<T> A = cpm_apply_args<T>(c);
+      const unsigned g = cpm_grid(c->NS * nrhs, 256);
+      if (c->p == 2) gather_rows2d_kernel<3><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
+      else gather_rows2d_kernel<4><<<g, 256, 0, st>>>(A, cs, u, a, nrhs, ld);
+      launch_combine<T>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st, dot);
+      return 2;
+    }
+  }
   if (nrhs > 32 && nrhs % 2 == 0 && aligned2)
     return launch_batched<T, 2>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);
   if (nrhs >= 16) return launch_batched<T, 1>(c, m, n, rowscale, cs, u, a, v, nrhs, ld, st);

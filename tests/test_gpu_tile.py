@@ -132,3 +132,27 @@ def test_fp32_of_smooth_columns_rounds_alike_in_every_width():
     for nrhs in (8, 16, 33, 64, 65, 66, 130):
         en = float((band.apply(0.0, 1.0, U[:, :nrhs].contiguous())[:, :8].double() - V).norm())
         assert en <= 1.25 * e1, (nrhs, en, e1)
+
+
+@pytest.mark.parametrize("p", [3, 2])
+def test_small_2d_batches_agree_with_columns_alone(p):
+    """Both sides of the rule that takes small FP32 batches of a 2D band row by row, near curves too.  Two FP32
+    products of the same column, each within 2e-6 of the largest entry."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.config1(0.001, ci.BC_DIR2)
+    band = Band(w.shape, w.h, p=p).set_boundary(w.curves)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(9)
+    U = torch.randn((band.N, 35), generator=gen, device="cuda")
+    alone = torch.stack([band.apply(0.3, 1.0, U[:, r].contiguous()) for r in range(35)], 1)
+    top = float(alone.abs().max())
+    for nrhs in (2, 5, 6, 7, 8, 15, 16, 33, 35):
+        V = band.apply(0.3, 1.0, U[:, :nrhs].contiguous())
+        assert float((V - alone[:, :nrhs]).abs().max()) <= 4e-6 * top, nrhs
+    small = Band(w.shape, 0.01, p=p).set_boundary(w.curves)
+    for nrhs in (33, 65, 129):
+        U = torch.randn((small.N, nrhs), generator=gen, device="cuda")
+        V = small.apply(0.3, 1.0, U)
+        one = torch.stack([small.apply(0.3, 1.0, U[:, r].contiguous()) for r in range(nrhs)], 1)
+        assert float((V - one).abs().max()) <= 4e-6 * float(one.abs().max()), nrhs
