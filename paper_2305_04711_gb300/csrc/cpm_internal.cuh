@@ -190,7 +190,7 @@ struct cpm_ctx {
   int32_t *d_cellid = nullptr;      // [nb*512] cell index of a packed base location, -1 if none
   double *d_tblk = nullptr;         // [ncells][64] per-cell blocks of E^T b (one right-hand side; integers, or FP32 in the
                                     // front half), then their [ncells] exponents
-  double *d_w1d64 = nullptr;        // [NS][12] per-axis Lagrange factors (transposed gather)
+  double *d_w1d64 = nullptr;        // [NS][12] per-axis Lagrange factors in cell order (transposed gather)
   float *d_w1d32 = nullptr;         // [NS][12]
   int32_t *d_T_ptr = nullptr;       // [N+1] CSR over columns
   int64_t nTcols = 0;

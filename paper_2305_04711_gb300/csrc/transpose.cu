@@ -35,13 +35,13 @@ __device__ __forceinline__ int64_t loc_of(const BandView &v, int32_t b, int lx, 
   return ((int64_t)b << 9) | (int64_t)((lz & 7) * 64 + (ly & 7) * 8 + (lx & 7));
 }
 
-// per PDE row its 1-D Lagrange factors along each axis ([NS][12]: x, y, z,
-// 4 slots each, zeros past the np1 stencil nodes)
-__global__ void w1d_kernel(int64_t NS, int dim, int np1, const double *t64, double *w64, float *w32) {
+// the 1-D Lagrange factors of the PDE rows along each axis, in cell order ([NS][12]: x,
+// y, z, 4 slots each, zeros past the np1 stencil nodes)
+__global__ void w1d_kernel(int64_t NS, int dim, int np1, const double *tc64, double *w64, float *w32) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < NS; i += (int64_t)gridDim.x * blockDim.x) {
     for (int a = 0; a < 3; ++a) {
       double w[4] = {1.0, 0.0, 0.0, 0.0};
-      if (a < dim) cpm_lagrange_rt<double>(np1, t64[3 * i + a], w);
+      if (a < dim) cpm_lagrange_rt<double>(np1, tc64[3 * i + a], w);
       for (int k = 0; k < 4; ++k) {
         w64[i * 12 + 4 * a + k] = w[k];
         w32[i * 12 + 4 * a + k] = (float)w[k];
@@ -135,7 +135,7 @@ template <typename T>
 struct TArgs {
   BandView v;
   const uint32_t *rself;
-  const T *w1d;  // [NS][12] per-axis Lagrange factors
+  const T *w1d;  // [NS][12] per-axis Lagrange factors, in cell order
   const int32_t *nbr8;
   const int32_t *cellid;
   const int32_t *cell_start;
@@ -305,13 +305,12 @@ __global__ void __launch_bounds__(TCW * 32)
       const int k = min(TCR, r1 - c0);
       // (weights formed in FP64 and rounded once, as the batches take them: formed from
       // a fraction rounded to FP32, those near zero lose their relative accuracy)
-      const int64_t row = (j0 < k) ? __ldg(A.crows + c0 + j0) : 0;
       if (ax < 3) {
         float4 wt = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (j0 < k) wt = __ldg(reinterpret_cast<const float4 *>(A.w1d32 + row * 12 + 4 * ax));
+        if (j0 < k) wt = __ldg(reinterpret_cast<const float4 *>(A.w1d32 + (int64_t)(c0 + j0) * 12 + 4 * ax));
         *reinterpret_cast<float4 *>(s_w[w][j0][ax]) = wt;
       } else if (j0 < k) {
-        s_b[w][j0] = __ldg(bv + row);
+        s_b[w][j0] = __ldg(bv + __ldg(A.crows + c0 + j0));
       }
       __syncwarp();
       for (int j = 0; j < k; ++j) {
@@ -482,7 +481,7 @@ __global__ void __launch_bounds__(256) ty_kernel(TArgs<T> A, T dg, T s, T rowsca
             const int32_t q1 = __ldg(A.cell_start + cell + 1);
             for (int32_t q = __ldg(A.cell_start + cell); q < q1; ++q) {
               const int64_t row = __ldg(A.cell_rows + q);
-              const T *wr = A.w1d + row * 12;
+              const T *wr = A.w1d + (int64_t)q * 12;
               const T w = __ldg(wr + cx) * __ldg(wr + 4 + cy) * __ldg(wr + 8 + cz);
               acc += w * __ldg(bv + row * ld + r);
             }
@@ -530,7 +529,7 @@ cpm_status cpm_build_transpose(cpm_ctx *c) {
   TRY(cudaMemsetAsync(c->d_cellid, 0xFF, sizeof(int32_t) * std::max<int64_t>(nkeys, 1), st));
   TRY(cudaMalloc(&c->d_w1d64, sizeof(double) * 12 * std::max<int64_t>(c->NS, 1)));
   TRY(cudaMalloc(&c->d_w1d32, sizeof(float) * 12 * std::max<int64_t>(c->NS, 1)));
-  w1d_kernel<<<cpm_grid(c->NS, 256), 256, 0, st>>>(c->NS, c->dim, c->p + 1, c->d_t64, c->d_w1d64, c->d_w1d32);
+  w1d_kernel<<<cpm_grid(c->NS, 256), 256, 0, st>>>(c->NS, c->dim, c->p + 1, c->d_tc64, c->d_w1d64, c->d_w1d32);
   if (c->ncells > 0)
     cellid_kernel<<<cpm_grid(c->ncells, 256), 256, 0, st>>>(c->d_cell_key, c->ncells, c->d_cellid);
   TRY(cudaMalloc(&count, sizeof(int32_t) * (N + 1)));
