@@ -622,14 +622,23 @@ cpm_status cpm_apply_transpose_rc_T(cpm_ctx *c, double m, double n, double rowsc
   int launched = 0;
   // One column, or a few of a 3D band, one by one: per-cell blocks of E^T b (one
   // column's are reserved at set-up), then the nodes by bricks.  All columns at once
-  // revisit every row of a node's 64 cells but share the walk: sphere h = 1/100
-  // (1.04M rows), one by one / at once, FP64: 3 columns 0.97 / 5.9 ms, 16 columns 5.6 /
-  // 10.1; FP32: 3 columns 0.54 / 1.48 ms, 16 columns 3.1 / 3.6; at h = 1/64 with 64
-  // columns 11.5 / 10.6 and 7.7 / 4.5 ms, at h = 1/32 4.5 / 2.7 and 3.0 / 1.2 ms, and a
-  // small band pays four launches a column.
-  const bool by_column = c->d_tblk && c->ncells > 0 &&
-                         (nrhs == 1 || (c->dim == 3 && (sizeof(T) == 8 ? nrhs <= 8 && c->NS >= 25000
-                                                                       : nrhs <= 4 && c->NS >= 100000)));
+  // revisit every row of a node's 64 (27) cells but share the walk, and a small band pays
+  // four launches a column, so the rows must make up for them.  Measured, one by one / at
+  // once in us:
+  //   FP64 cubic      27k rows: 6 columns 308 / 399, 8 columns 411 / 353; 42k: 8 431 / 477
+  //   FP64 quadratic  21k rows: 2 columns 78 / 103, 4 156 / 119; 42k: 4 156 / 167, 5 200 / 190;
+  //                   84k: 7 341 / 399, 8 394 / 365; 167k: 8 513 / 657
+  //   FP32 cubic      60k rows: 3 columns 118 / 142, 4 160 / 154; 106k: 4 186 / 209
+  //   FP32 quadratic  84k rows: 2 columns 66 / 68, 3 99 / 78; 167k: 2 86 / 104, 4 173 / 143;
+  //                   339k: 4 247 / 256
+  // (8 columns walk aligned 64-byte segments, hence their own line).  More columns than
+  // these gain only on bands of a million rows and lose below: FP64 16 columns 5.6 / 10.1 ms
+  // at 1.04M rows, 64 columns 11.5 / 10.6 ms at 424k.
+  int64_t rows_a_column;  // fewer rows than this for each column: all at once
+  if (sizeof(T) == 8) rows_a_column = (c->p == 2) ? (nrhs < 8 ? 8500 : 13500) : (nrhs < 8 ? 3800 : 4500);
+  else rows_a_column = (c->p == 2) ? 60000 : 25000;
+  const bool few = c->dim == 3 && nrhs <= (sizeof(T) == 8 ? 8 : 4) && c->NS >= nrhs * rows_a_column;
+  const bool by_column = c->d_tblk && c->ncells > 0 && (nrhs == 1 || few);
   if (by_column) {
     TCellArgs C{c->d_cell_start, c->d_cell_rows, c->ncells, c->d_tc64, c->d_w1d32};
     int32_t *bexp = reinterpret_cast<int32_t *>(c->d_tblk + 64 * c->ncells);

@@ -130,3 +130,22 @@ def test_fp32_weights_keep_their_relative_accuracy(oracle_mod, name, p):
         y = band.apply(0.0, 1.0, torch.tensor(lam, device="cuda").float(), transpose=True).cpu().numpy()
         err = np.abs(y - A[i].toarray()[0])
         assert np.all(err <= 24 * 2.0 ** -24 * size[i].toarray()[0] + 1e-14 * size[i].max())
+
+
+@pytest.mark.parametrize("p, inv_h", [(3, 12), (3, 18), (2, 16), (2, 28), (2, 40)])
+def test_few_columns_on_both_sides_of_their_rule(p, inv_h):
+    """Bands around the row counts from which 2 to 9 columns go one by one (12k to 130k rows), near curves too."""
+    torch = need_gpu()
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.config2(1 / inv_h, ci.BC_DIR2)
+    band = Band(w.shape, w.h, p=p).set_boundary(w.curves)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    U = torch.randn((band.N, 9), generator=gen, dtype=torch.float64, device="cuda")
+    one = torch.stack([band.apply(0.3, 1.0, U[:, r].contiguous(), transpose=True) for r in range(9)], 1)
+    top = float(one.abs().max())
+    for nrhs in range(2, 10):
+        V = band.apply(0.3, 1.0, U[:, :nrhs].contiguous(), transpose=True)
+        assert float((V - one[:, :nrhs]).abs().max()) <= 1e-14 * top, nrhs
+        V32 = band.apply(0.3, 1.0, U[:, :nrhs].float().contiguous(), transpose=True)
+        assert float((V32.double() - one[:, :nrhs]).abs().max()) <= 2e-6 * top, nrhs
