@@ -356,7 +356,8 @@ cpm_status cpm_profile(cpm_ctx *ctx, int enable, double *apply_ms, int64_t *appl
 typedef struct {
   int cells_xh;              /* x passes an earlier batched cell gather took: checked and reported, without
                               * effect on the present one (0: the batch width has none) */
-  int cells_blocks_per_sm;   /* grid cap of the cell gather, blocks of 8 warps per SM (0: default 16) */
+  int cells_blocks_per_sm;   /* grid cap of the FP32 cell gather, blocks of 8 warps per SM (0: default 4 with
+                              * two columns per lane, i.e. even widths above 32, else 16) */
   int combine_warps_per_sm;  /* grid cap of the warp-per-row combine (0: default 64) */
   int vec_blocks_per_sm;     /* blocks of 512 threads per SM of the Krylov vector kernels (1, 2 or 4) */
   int single_mode;           /* single right-hand side product: 0 = gather by tiles of cells then combine (default),
@@ -370,8 +371,8 @@ typedef struct {
 
 /* Autotuner of the launch shapes.  Times, on this context's band and with
  * nrhs right-hand sides of leading dimension ld in precision prec, the
- * candidate shapes of the batched product (x passes of the cell gather, its
- * grid, the combine's grid) and of the Krylov vector kernels (blocks per SM),
+ * candidate shapes of the batched product (the FP32 cell gather's grid, the
+ * combine's grid) and of the Krylov vector kernels (blocks per SM),
  * by coordinate descent, and keeps the fastest in the context for every later
  * product and solve (a later call for another width or precision refines
  * them).  Uses the reserved solve workspace as scratch: ld and prec must be

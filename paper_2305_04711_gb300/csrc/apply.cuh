@@ -63,9 +63,11 @@ int cpm_launch_correct_few(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, i
 template <typename T>
 void cpm_launch_gather1(const cpm_ctx *c, const ApplyArgs<T> &A, T cs, const T *u, T *a, cudaStream_t st);
 
-// the cell gather's default x passes for a stencil of np1 nodes per axis, the
-// precision and the columns per lane (1 or 2); the autotuner starts from it
+// the x passes reported for a stencil of np1 nodes per axis, the precision and the
+// columns per lane (1 or 2) where none are set
 int cpm_cells_default_xh(int np1, bool fp64, int rpl);
+// the FP32 cell gather's default grid cap (blocks of 8 warps per SM)
+int cpm_cells_default_blocks(int rpl);
 
 // the single right-hand side product in one persistent kernel (fused1.cu);
 // returns the launches (0: not built for this band)

@@ -712,6 +712,10 @@ int cpm_cells_default_xh(int np1, bool fp64, int rpl) {
   return (np1 == 3) ? ((fp64 && rpl == 2) ? 3 : 1) : (fp64 ? (rpl == 2 ? 4 : 2) : 2);
 }
 
+// 4 blocks per SM (two rounds) with two columns per lane, 16 with one: 1324 / 1353 us
+// of the 64-column product on the sphere at h = 1/128, 1202 / 1061 us of 24 columns (4 / 16)
+int cpm_cells_default_blocks(int rpl) { return rpl == 2 ? 4 : 16; }
+
 static CellArgs cell_args(const cpm_ctx *c) {
   return CellArgs{c->d_cell_start, c->d_cell_rows, c->d_cell_key, reinterpret_cast<const int2 *>(c->d_cell_lines),
                   c->ncells};
@@ -720,9 +724,7 @@ static CellArgs cell_args(const cpm_ctx *c) {
 template <int DIM, int NP, int R>
 static void launch_cells_k(const cpm_ctx *c, float cs, const float *u, float *a, int nrhs, int64_t ld,
                            cudaStream_t st) {
-  // by default 4 blocks per SM (two rounds) with two columns per lane, 16 with one:
-  // 1324 / 1353 us of the 64-column product, 1202 / 1061 us of 24 columns (4 / 16)
-  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : (R == 2 ? 4 : 16);
+  const int per_sm = c->tune.cells_blocks_per_sm > 0 ? c->tune.cells_blocks_per_sm : cpm_cells_default_blocks(R);
   const int64_t items = c->ncells * ((nrhs + 32 * R - 1) / (32 * R));
   const unsigned g = (unsigned)std::min<int64_t>((items + WARPS - 1) / WARPS, (int64_t)c->nsm * per_sm);
   gather_cells_kernel<DIM, NP, R><<<g, WARPS * 32, 0, st>>>(cell_args(c), c->d_tc32, cs, u, a, nrhs, (unsigned)ld);

@@ -1,15 +1,17 @@
 // tune.cu -- the launch-shape autotuner.
 //
-// The grids of the batched cell gather and of the warp-per-row combine and the
+// The grids of the FP32 cell gather and of the warp-per-row combine and the
 // Krylov vector kernels' blocks per SM trade occupancy against tail effects.
 // Which is fastest depends on the band (cells per brick, rows per cell), the batch
 // width and the precision, so the tuner times each candidate on the context's own
 // band with the caller's batch layout, by coordinate descent (the gather grid, then
 // the combine grid, then the vector kernels), and keeps the fastest in the context.
-// The x passes that an earlier cell gather took are still accepted and reported, so
-// that recorded shapes stay valid; they choose nothing now.  Every candidate computes
-// the same product; only the vector kernels' reduction grouping changes with their
-// block count (each choice is deterministic).
+// It starts from the shapes in force, a default where none is set, so that a candidate
+// replaces them only by a shorter time of its own.  The x passes that an earlier cell
+// gather took are still accepted and reported, so that recorded shapes stay valid; they
+// choose nothing and are not timed.  Every candidate computes the same product; only
+// the vector kernels' reduction grouping changes with their block count (each choice is
+// deterministic).
 #include <algorithm>
 #include <vector>
 
@@ -20,9 +22,9 @@
 namespace {
 
 // the columns per lane of the cell gather for a batch (0: the batch does not
-// use it): two above 32 columns, one from 16 to 32
+// use it), as the product chooses them for aligned vectors
 int cells_rpl(int nrhs, int64_t ld) {
-  return (nrhs > 32 && nrhs <= 64 && nrhs % 2 == 0 && ld % 2 == 0) ? 2 : (nrhs >= 16 && nrhs <= 32) ? 1 : 0;
+  return (nrhs > 32 && nrhs % 2 == 0 && ld % 2 == 0) ? 2 : (nrhs >= 16) ? 1 : 0;
 }
 
 template <typename T>
@@ -61,42 +63,29 @@ cpm_status tune_products(cpm_ctx *c, int nrhs, int64_t ld, T *u, T *v, cudaStrea
   CPM_CUDA_TRY(cudaGetLastError());
   Tune &t = c->tune;
   const int pi = (sizeof(T) == 8) ? 1 : 0;
-  // the cell gather serves batches of 16 to 64 columns (2 per lane above 32)
   const int rpl = cells_rpl(nrhs, ld);
+  if (rpl > 0) {
+    // the defaults made explicit, so that the report names the kept choice (the FP64
+    // gather's grid is fixed: it leaves the FP32 one's alone)
+    if (sizeof(T) == 4 && t.cells_blocks_per_sm <= 0) t.cells_blocks_per_sm = cpm_cells_default_blocks(rpl);
+    if (t.combine_warps_per_sm <= 0) t.combine_warps_per_sm = 64;
+  }
   double best = 0.0;
   cpm_status rc = time_products<T>(c, u, v, nrhs, ld, st, &best);
   if (rc) return rc;
   info->product_ms_default = best;
   if (rpl > 0) {
-    const int np1 = c->p + 1;
-    std::vector<int> xhs;
-    for (int xh : {1, 2, 3, 4}) {
-      if (np1 % xh) continue;
-      if (sizeof(T) == 8 && np1 / xh > 2) continue;  // FP64 node values held at most two x wide
-      xhs.push_back(xh);
+    if (sizeof(T) == 4) {
+      int best_g = t.cells_blocks_per_sm;
+      for (int g : {4, 8, 16, 32}) {
+        t.cells_blocks_per_sm = g;
+        double ms = 0.0;
+        rc = time_products<T>(c, u, v, nrhs, ld, st, &ms);
+        if (rc) return rc;
+        if (ms < best) { best = ms; best_g = g; }
+      }
+      t.cells_blocks_per_sm = best_g;
     }
-    // the defaults made explicit, so that the report names the kept choice
-    if (t.cells_xh[pi][rpl - 1] <= 0) t.cells_xh[pi][rpl - 1] = cpm_cells_default_xh(np1, sizeof(T) == 8, rpl);
-    if (t.cells_blocks_per_sm <= 0) t.cells_blocks_per_sm = 16;
-    if (t.combine_warps_per_sm <= 0) t.combine_warps_per_sm = 64;
-    int best_xh = t.cells_xh[pi][rpl - 1];
-    for (int xh : xhs) {
-      t.cells_xh[pi][rpl - 1] = xh;
-      double ms = 0.0;
-      rc = time_products<T>(c, u, v, nrhs, ld, st, &ms);
-      if (rc) return rc;
-      if (ms < best) { best = ms; best_xh = xh; }
-    }
-    t.cells_xh[pi][rpl - 1] = best_xh;
-    int best_g = t.cells_blocks_per_sm;
-    for (int g : {4, 8, 16, 32}) {
-      t.cells_blocks_per_sm = g;
-      double ms = 0.0;
-      rc = time_products<T>(c, u, v, nrhs, ld, st, &ms);
-      if (rc) return rc;
-      if (ms < best) { best = ms; best_g = g; }
-    }
-    t.cells_blocks_per_sm = best_g;
     int best_w = t.combine_warps_per_sm;
     for (int wps : {16, 32, 64, 128}) {
       t.combine_warps_per_sm = wps;
@@ -106,7 +95,8 @@ cpm_status tune_products(cpm_ctx *c, int nrhs, int64_t ld, T *u, T *v, cudaStrea
       if (ms < best) { best = ms; best_w = wps; }
     }
     t.combine_warps_per_sm = best_w;
-    info->cells_xh = t.cells_xh[pi][rpl - 1];
+    const int xh = t.cells_xh[pi][rpl - 1];
+    info->cells_xh = xh > 0 ? xh : cpm_cells_default_xh(c->p + 1, sizeof(T) == 8, rpl);
   }
   if (nrhs == 1 && c->ncells > 0) {
     // the single right-hand side product: a gather per cell or per row then the combine, or fused
@@ -121,7 +111,8 @@ cpm_status tune_products(cpm_ctx *c, int nrhs, int64_t ld, T *u, T *v, cudaStrea
     t.single_mode = best_m;
     info->single_mode = best_m;
   }
-  info->cells_blocks_per_sm = t.cells_blocks_per_sm;
+  info->cells_blocks_per_sm =
+      (t.cells_blocks_per_sm > 0 || rpl == 0) ? t.cells_blocks_per_sm : cpm_cells_default_blocks(rpl);
   info->combine_warps_per_sm = t.combine_warps_per_sm;
   info->product_ms = best;
   return CPM_OK;

@@ -294,3 +294,19 @@ def test_autotune_choices_keep_the_products(oracle_mod, torch_mod):
     x, st = band.solve(0.0, 1.0, band.rhs(g=torch.ones((band.NC, 64), dtype=torch.float64, device="cuda"), nrhs=64),
                        tol=1e-10, mode="fp32_ir")
     assert st.status == "CPM_OK"
+
+
+@pytest.mark.parametrize("dtype, nrhs, products", [("float32", 64, 9), ("float32", 65, 9), ("float64", 64, 5)])
+def test_autotune_times_what_has_an_effect(torch_mod, dtype, nrhs, products):
+    """Four products each (one untimed) of the shapes in force and of every candidate: four grids of the FP32 cell
+    gather and four of the combine.  The report names the defaults that the products take."""
+    torch = torch_mod
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.config2(1 / 16)
+    band = Band(w.shape, w.h).set_boundary(w.curves)
+    band.reserve(nrhs, fp32_ir=True)
+    band.profile(True)
+    info = band.autotune(nrhs, getattr(torch, dtype))
+    assert band.profile(False)["applies"] == 4 * products
+    assert info["product_ms"] <= info["product_ms_default"]
+    assert info["cells_blocks_per_sm"] in ((4,) if dtype == "float64" else (4, 8, 16, 32))
