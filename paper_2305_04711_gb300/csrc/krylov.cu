@@ -728,7 +728,10 @@ cpm_status ir_refine(cpm_ctx *c, ApplyFn<double> ap64, const Op<float> &op32, do
     for (int q = 0; q < nrhs; ++q) left += !done_col(rn2[q], fn2[q], tol, floors[q]);
     // a sixteenth of the batch or less: an FP64 solve of these columns alone is
     // cheaper than another FP32 step of all (sphere h = 1/128: an FP64 iteration of
-    // one column 0.49 ms, an FP32 iteration of 64 3.9 ms)
+    // one column 0.49 ms, an FP32 iteration of 64 3.9 ms; batches of 16 to 64 columns on
+    // spheres of h = 1/16 to 1/64 and the torus at h = 1/32 that ended so were 1 to 7 %
+    // faster by it; an FP64 iteration of one column takes less than an FP32 one of 16
+    // there, and the FP32 phase has about 1.3 times as many)
     if (nrep > 0 && left * 16 <= nrhs) break;
     for (int q = 0; q < nrhs; ++q) {
       flag[q] = 0.0;
