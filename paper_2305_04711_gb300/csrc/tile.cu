@@ -298,8 +298,12 @@ int cpm_launch_gather_tile(const cpm_ctx *c, T cs, const T *u, T *a, int nrhs, i
   const T *tc;
   if constexpr (sizeof(T) == 8) tc = reinterpret_cast<const T *>(c->d_tc64);
   else tc = reinterpret_cast<const T *>(c->d_tc32);
-  if (diff) launch_tile_any<T, true>(c, tc, cs, u, a, nrhs, ld, st);
-  else launch_tile_any<T, false>(c, tc, cs, u, a, nrhs, ld, st);
+  if constexpr (sizeof(T) == 8) {
+    if (diff) launch_tile_any<T, true>(c, tc, cs, u, a, nrhs, ld, st);
+    else launch_tile_any<T, false>(c, tc, cs, u, a, nrhs, ld, st);
+  } else {  // (no caller wants E u itself in FP32)
+    launch_tile_any<T, true>(c, tc, cs, u, a, nrhs, ld, st);
+  }
   return 1 + cpm_launch_correct_few<T>(c, cs, u, a, nrhs, ld, st);
 }
 #define CPM_TILE_INST(T)                                                                                       \
