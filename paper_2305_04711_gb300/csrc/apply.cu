@@ -7,7 +7,8 @@
 // fractional position t (FP64 and FP32 copies).  Two steps per product:
 //   gather : a_i = (E u - u)_i for PDE rows (tile.cu up to 15 columns, cells.cu
 //            from 16), rows near an interior boundary with the crossing-test
-//            flips (Eq. 10) added as a sparse correction;
+//            flips (Eq. 10) added as a sparse correction (small FP32 batches of
+//            2D bands: a thread per row and column here, flips included);
 //   combine: the FD stencil of the PDE rows and the BC rows
 //            v_alpha = sum_beta B_alpha,beta u_beta,
 // where a neighbour flipped to a BC DOF reads u of that DOF (E rows of BC DOFs
@@ -603,8 +604,8 @@ void cpm_prof_end(cpm_ctx *c, cudaStream_t st, int64_t row_rhs) {
 }
 
 cpm_status cpm_internal_extend(cpm_ctx *c, const double *u, double *a, int nrhs, int64_t ld, cudaStream_t st) {
-  if (nrhs < 16) cpm_launch_gather_tile<double>(c, 1.0, u, a, nrhs, ld, st, false);
-  else cpm_launch_gather_cells<double>(c, 1.0, u, a, nrhs, ld, st, false, 1);
+  cpm_count_launches(c, nrhs < 16 ? cpm_launch_gather_tile<double>(c, 1.0, u, a, nrhs, ld, st, false)
+                                  : cpm_launch_gather_cells<double>(c, 1.0, u, a, nrhs, ld, st, false, 1));
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }

@@ -67,7 +67,7 @@ cpm_status cpm_internal_surface_gradient(cpm_ctx *c, const double *u, double *X,
   if (rc) return rc;
   grad_kernel<<<cpm_grid(c->NS + c->NC, 256), 256, 0, st>>>(c->NS, c->NC, c->dim, 0.5 / c->h, c->d_nbr8, c->d_twin, a,
                                                             u, normalize, X);
-  cpm_count_launches(c, 2);
+  cpm_count_launches(c, 1);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }
@@ -78,7 +78,7 @@ cpm_status cpm_internal_surface_divergence(cpm_ctx *c, const double *X, double *
   cpm_status rc = cpm_internal_extend(c, X, xe, 3, 3, st);
   if (rc) return rc;
   div_kernel<<<cpm_grid(c->NS, 256), 256, 0, st>>>(c->NS, c->dim, 0.5 / c->h, c->d_nbr8, xe, X, b);
-  cpm_count_launches(c, 2);
+  cpm_count_launches(c, 1);
   CPM_CUDA_TRY(cudaGetLastError());
   return CPM_OK;
 }

@@ -73,3 +73,17 @@ def test_bumpy_sphere_band_matches_oracle(oracle_mod):
     pairs = [(i, rindex[k]) for i, k in enumerate(map(tuple, ijk.tolist())) if k in rindex]
     ga, gr = np.array(pairs).T
     assert np.max(np.abs(cp[ga] - ref.cp[gr])) < 1e-12
+
+
+def test_launches_of_the_field_steps_are_counted():
+    """The extension's gather and flipped entries, then the differences: three launches each near curves."""
+    need_gpu()
+    import torch
+    from paper_2305_04711_gb300.cpm import Band
+    w = ci.config2(1 / 16)
+    for curves, launches in ((w.curves, 6), ([], 4)):
+        band = Band(w.shape, w.h).set_boundary(curves)
+        u = torch.ones(band.N, dtype=torch.float64, device="cuda")
+        band.profile(True)
+        band.surface_divergence(band.surface_gradient(u))
+        assert band.profile(False)["launches"] == launches
