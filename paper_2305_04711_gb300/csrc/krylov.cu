@@ -374,6 +374,7 @@ struct GraphKey {
 struct SolveWork {
   int64_t N = 0, ld = 0;     // reserved rows and leading dimension
   bool has32 = false;
+  char *vecs = nullptr;      // the vectors below, one allocation
   double *v64[6] = {};       // FP64 Krylov vectors (FP64 solves, FP64 finish of FP32_IR)
   float *v32[6] = {};        // FP32 Krylov vectors (FP32_IR inner solves)
   float *d32 = nullptr;      // FP32_IR correction of one inner solve
@@ -397,10 +398,7 @@ struct SolveWork {
 
 static void free_work(SolveWork *w) {
   if (!w) return;
-  for (auto p : w->v64) cudaFree(p);
-  for (auto p : w->v32) cudaFree(p);
-  cudaFree(w->d32);
-  cudaFree(w->r64); cudaFree(w->xc);
+  cudaFree(w->vecs);
   cudaFree(w->part); cudaFree(w->sc); cudaFree(w->out); cudaFree(w->cols); cudaFree(w->ticket);
   if (w->h_pin) cudaFreeHost(w->h_pin);
   for (auto &g : w->graphs)
@@ -430,12 +428,20 @@ cpm_status cpm_reserve_solve(cpm_ctx *c, int64_t ld, bool fp32) {
   auto al = [&](void **p, size_t bytes) {
     if (rc == CPM_OK && cudaMalloc(p, bytes) != cudaSuccess) { (void)cudaGetLastError(); rc = CPM_ERR_OOM; }
   };
-  for (auto &p : w->v64) al((void **)&p, n * sizeof(double));
-  al((void **)&w->r64, n * sizeof(double));
-  al((void **)&w->xc, n * sizeof(double));
-  if (fp32) {
-    for (auto &p : w->v32) al((void **)&p, n * sizeof(float));
-    al((void **)&w->d32, n * sizeof(float));
+  // (one allocation for all vectors: set-up of a small band is its allocations)
+  const size_t b64 = (n * sizeof(double) + 255) / 256 * 256, b32 = (n * sizeof(float) + 255) / 256 * 256;
+  al((void **)&w->vecs, 8 * b64 + (fp32 ? 7 * b32 : 0));
+  if (rc == CPM_OK) {
+    char *at = w->vecs;
+    for (double **p : {&w->v64[0], &w->v64[1], &w->v64[2], &w->v64[3], &w->v64[4], &w->v64[5], &w->r64, &w->xc}) {
+      *p = reinterpret_cast<double *>(at);
+      at += b64;
+    }
+    if (fp32)
+      for (float **p : {&w->v32[0], &w->v32[1], &w->v32[2], &w->v32[3], &w->v32[4], &w->v32[5], &w->d32}) {
+        *p = reinterpret_cast<float *>(at);
+        at += b32;
+      }
   }
   w->G = 2 * c->nsm;
   // partials for up to 4 blocks per SM (the autotuner's widest choice)
